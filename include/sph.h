@@ -115,7 +115,8 @@ typedef struct sph_params {
     int32_t pair_warps;      /* warps per CTA of the pair kernel, 0 = default */
     int32_t pair_ctas_per_sm;/* resident pair CTAs per SM, 0 = default */
     int32_t compensated;     /* mixed form: compensated FP32 pair sums (1) */
-    int32_t pair_group;      /* mixed form: particles per warp sharing candidate loads (1, 2 or 4), 0 = default 4 */
+    int32_t pair_group;      /* mixed form: particles per warp sharing candidate loads (1, 2 or 4; 1 runs as 2
+                                where h < 7/3 dp), 0 = default 4 */
     int32_t integrator;      /* SPH_VERLET (default) or SPH_SYMPLECTIC */
     int32_t delta_mode;      /* SPH_DELTA_ALL_FLUID (default) or SPH_DELTA_FULL_SUPPORT */
     int32_t persistent;      /* 1: sph_step runs all its steps in one persistent cooperative launch

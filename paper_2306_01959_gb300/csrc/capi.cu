@@ -47,7 +47,15 @@ struct sph_s {
     int64_t N = 0;
     int32_t C = 0;
     int32_t ninst = 0;
-    int32_t max_active = 0;
+    // Grid: cells of 2h / base_div (the cell_div of the parameters), each divided
+    // again by `fine`: the automatic cell size of the mixed form is 2h for callers
+    // (sph_sizes, sph_cells) while its pair pass works on cells of h.  pub_fine is
+    // the division callers see (1; after autotuning, the tuned one).  p.cell_div
+    // is base_div * fine.
+    int32_t base_div = 1, fine = 1, pub_fine = 1;
+    bool auto_div = false;  // the mixed form's automatic cell size
+    bool tiled = false;     // the mixed pair pass is the tiled one (pair_mixed.cuh), else pair_wide.cuh
+    int32_t ntiles = 0, ntiles_alloc = 0;  // tiles of the mixed pair pass
     int32_t C_alloc = 0;      // cells the workspace holds: the largest grid, at cell_div 3
     int32_t reorder_ctas = 16; // resident CTAs per SM of the per-cell sort and gather (tuned)
     int32_t list_cap = 0;      // neighbour-list entries per particle (0: no lists)
@@ -91,7 +99,7 @@ static int cuda_fail(sph_t *s, cudaError_t e, const char *where)
     } while (0)
 
 static size_t layout(Bufs &b, char *base, int64_t N, int32_t C, int32_t ninst, int mode, int32_t list_cap,
-                     bool fp64_sym)
+                     bool fp64_sym, int32_t ntiles)
 {
     Layout L;
     L.base = base;
@@ -105,9 +113,12 @@ static size_t layout(Bufs &b, char *base, int64_t N, int32_t C, int32_t ninst, i
     b.count = L.take<uint32_t>((size_t)C + 1);
     b.cell_start = L.take<int32_t>((size_t)C + 2);
     b.active = L.take<int32_t>((size_t)C);
+    b.tiles = ntiles ? L.take<int32_t>((size_t)ntiles) : nullptr;
     b.scan_blocks = L.take<uint64_t>(((size_t)C + 1 + kScanTile - 1) / kScanTile);
     b.perm = L.take<int32_t>(N);
-    b.ptmp = L.take<int32_t>(N);
+    b.ptmp = mode == SPH_FP64 ? L.take<int32_t>(N) : nullptr;
+    b.pkey = mode == SPH_MIXED ? L.take<uint64_t>(N) : nullptr;
+    b.xof = mode == SPH_MIXED ? L.take<float>(N) : nullptr;
     b.scell = L.take<int32_t>(N);
     b.sA = L.take<char>(N * vsz);
     b.sB = L.take<char>(N * vsz);
@@ -156,7 +167,15 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
         return fail(s, SPH_EINVAL, "n_inst must be in [1, 65535] with a non-NULL instance array");
     s->p = *p;
     s->mode = p->precision;
-    s->p.cell_div = effective_cell_div(*p);
+    s->base_div = effective_cell_div(*p);
+    // cells of h for the mixed pair pass unless the caller chose a size; the lists work on cells of 2h + s
+    s->tiled = p->precision == SPH_MIXED;
+    for (int k = 0; k < n_inst; ++k)
+        s->tiled = s->tiled && tiles_fit(in[k], *p);
+    s->auto_div = s->tiled && p->cell_div == 0;
+    s->fine = s->auto_div ? 2 : 1;
+    s->pub_fine = 1;
+    s->p.cell_div = s->base_div * s->fine;
     s->inst.resize(n_inst);
     int64_t N = 0, C = 0;
     for (int k = 0; k < n_inst; ++k) {
@@ -166,7 +185,7 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
             return fail(s, rc, "instance " + std::to_string(k) + ": " + e);
         HostInst &hi = s->inst[k];
         hi.d = in[k];
-        fill_inst(hi, *p);
+        fill_inst(hi, *p, s->fine, s->tiled);
         hi.dev.pbase = (int32_t)N;
         hi.dev.cell_base = (int32_t)C;
         N += hi.nf + hi.nw + hi.no + hi.ng;
@@ -194,6 +213,20 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
     if (C3 >= ((int64_t)1 << 31) - 4)
         return fail(s, SPH_EINVAL, "too many cells (limit 2^31)");
     s->C_alloc = (int32_t)std::max<int64_t>(C3, C);
+    if (s->tiled) {
+        // room for the tiles of every cell size the autotuner may choose
+        for (int d = 1; d <= 2; ++d) {
+            sph_params pd = *p;
+            if (!s->auto_div)
+                pd.cell_div = d;
+            std::vector<HostInst> tmp = s->inst;
+            for (HostInst &hi : tmp)
+                fill_inst(hi, pd, s->auto_div ? d : 1, true);
+            s->ntiles_alloc = std::max(s->ntiles_alloc, (int32_t)fill_tiles(tmp, d, N));
+        }
+        s->ntiles = (int32_t)fill_tiles(s->inst, s->p.cell_div, N);
+        s->ntiles_alloc = std::max(s->ntiles_alloc, s->ntiles);
+    }
     s->list_cap = 0;
     if (p->list_skin > 0) {
         // entries (j << 5 | cell offset) hold sorted indices below 2^26
@@ -215,7 +248,6 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
     s->N = N;
     s->C = (int32_t)C;
     s->ninst = n_inst;
-    s->max_active = (int32_t)std::min<int64_t>(C, N);
     return SPH_OK;
 }
 
@@ -254,7 +286,8 @@ int sph_workspace_size(int32_t n_inst, const sph_instance *inst, const sph_param
     if (rc)
         return rc;
     Bufs b{};
-    *bytes = layout(b, nullptr, tmp.N, tmp.C_alloc, tmp.ninst, tmp.mode, tmp.list_cap, tmp.p.pair_symmetric != 0);
+    *bytes = layout(b, nullptr, tmp.N, tmp.C_alloc, tmp.ninst, tmp.mode, tmp.list_cap, tmp.p.pair_symmetric != 0,
+                    tmp.ntiles_alloc);
     return SPH_OK;
 }
 
@@ -289,8 +322,8 @@ static void enqueue_prepare(sph_t *s, cudaStream_t st)
     if (s->b.lflag)
         cudaMemsetAsync(s->b.lflag, 1, 1, st);  // rebuild request: the structure and then the lists
     launch_bin(s->b, s->mode, s->N, s->C, st);
-    launch_cells(s->b, s->N, s->C, st);
-    launch_reorder(s->b, s->mode, s->N, s->C, s->ninst, s->max_active, s->reorder_ctas, st);
+    launch_cells(s->b, s->mode, s->N, s->C, st);
+    launch_reorder(s->b, s->mode, s->N, s->ninst, s->reorder_ctas, st);
 }
 
 // count: also sum the per-class work counts of the mixed form (a separate
@@ -303,9 +336,12 @@ static void enqueue_pair(sph_t *s, cudaStream_t st, bool count = false, bool nei
                          count || neighbours, st);
     } else if (s->b.lflag && !count) {
         launch_list_pass(s->b, s->N, s->ninst, s->p.delta_mode, st);
+    } else if (!s->tiled) {
+        launch_pair_wide(s->b, s->ninst, s->p.cell_div, s->pair_warps, s->pair_ctas, s->pair_group,
+                         s->p.compensated, count || neighbours, s->p.delta_mode, st);
     } else
-        launch_pair_mixed(s->b, s->N, s->ninst, s->p.cell_div, s->pair_warps, s->pair_ctas, s->pair_group,
-                          s->p.compensated, s->max_active, count, s->p.delta_mode, st);
+        launch_pair_mixed(s->b, s->ninst, s->p.cell_div, s->pair_warps, s->pair_ctas, s->pair_group,
+                          s->p.compensated, count || neighbours, s->p.delta_mode, st);
 }
 
 // Neighbour structure of the rebinned state and the sorted gather.  With
@@ -317,10 +353,10 @@ static void enqueue_rebuild(sph_t *s, cudaStream_t st)
     rec(s, PH_CELLS, true);
     if (s->b.lflag)
         launch_bin(s->b, s->mode, s->N, s->C, st);
-    launch_cells(s->b, s->N, s->C, st);
+    launch_cells(s->b, s->mode, s->N, s->C, st);
     rec(s, PH_CELLS, false);
     rec(s, PH_REORDER, true);
-    launch_reorder(s->b, s->mode, s->N, s->C, s->ninst, s->max_active, s->reorder_ctas, st);
+    launch_reorder(s->b, s->mode, s->N, s->ninst, s->reorder_ctas, st);
     if (s->b.lflag)
         launch_list_regather(s->b, s->N, s->ninst, st);
     rec(s, PH_REORDER, false);
@@ -398,6 +434,56 @@ static int check_status(sph_t *s)
     return SPH_OK;
 }
 
+// Cells of the grid callers see (cell counts per axis are multiples of `fine`).
+static int64_t public_cells(const sph_t *s)
+{
+    int64_t C = 0;
+    for (const HostInst &hi : s->inst) {
+        int64_t n = 1;
+        for (int a = 0; a < 3; ++a)
+            n *= hi.dev.n[a] / s->fine * s->pub_fine;
+        C += n;
+    }
+    return C;
+}
+
+// Switch the grid to cells of 2h / (base * fine): new per-instance constants,
+// the neighbour structure of the current state rebuilt on the new grid.
+static int apply_grid(sph_t *s, int base, int fine)
+{
+    if (base == s->base_div && fine == s->fine)
+        return SPH_OK;
+    sph_params p = s->p;
+    p.cell_div = base;
+    int64_t C = 0;
+    std::vector<Inst> idev(s->ninst);
+    for (int k = 0; k < s->ninst; ++k) {
+        HostInst &hi = s->inst[k];
+        const int32_t pbase = hi.dev.pbase;
+        fill_inst(hi, p, fine, s->tiled);
+        hi.dev.pbase = pbase;
+        hi.dev.cell_base = (int32_t)C;
+        C += hi.dev.ncells;
+    }
+    if (C > s->C_alloc)
+        return fail(s, SPH_EINVAL, "grid larger than the workspace holds");
+    CK(cudaStreamSynchronize(s->st));
+    s->base_div = base;
+    s->fine = fine;
+    s->p.cell_div = base * fine;
+    s->C = (int32_t)C;
+    if (s->tiled)
+        s->b.ntiles = s->ntiles = (int32_t)fill_tiles(s->inst, s->p.cell_div, s->N);
+    for (int k = 0; k < s->ninst; ++k)
+        idev[k] = s->inst[k].dev;
+    CK(cudaMemcpyAsync(s->b.inst, idev.data(), sizeof(Inst) * s->ninst, cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemsetAsync(s->b.count, 0, sizeof(uint32_t) * ((size_t)s->C_alloc + 1), s->st));
+    enqueue_prepare(s, s->st);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(s->st));
+    return SPH_OK;
+}
+
 static int create_common(sph_t **out, int32_t n_inst, const sph_instance *in, const sph_params *p, void *ws,
                          size_t bytes, uintptr_t stream)
 {
@@ -412,7 +498,8 @@ static int create_common(sph_t **out, int32_t n_inst, const sph_instance *in, co
         return rc;
     }
     Bufs tmpb{};
-    size_t need = layout(tmpb, nullptr, s->N, s->C_alloc, s->ninst, s->mode, s->list_cap, s->p.pair_symmetric != 0);
+    size_t need = layout(tmpb, nullptr, s->N, s->C_alloc, s->ninst, s->mode, s->list_cap, s->p.pair_symmetric != 0,
+                         s->ntiles_alloc);
     if (!ws || bytes < need || ((uintptr_t)ws & 255)) {
         std::fprintf(stderr, "sph_create: workspace needs %zu bytes, 256-byte aligned\n", need);
         delete s;
@@ -420,7 +507,8 @@ static int create_common(sph_t **out, int32_t n_inst, const sph_instance *in, co
     }
     s->ws = (char *)ws;
     s->ws_bytes = bytes;
-    layout(s->b, s->ws, s->N, s->C_alloc, s->ninst, s->mode, s->list_cap, s->p.pair_symmetric != 0);
+    layout(s->b, s->ws, s->N, s->C_alloc, s->ninst, s->mode, s->list_cap, s->p.pair_symmetric != 0, s->ntiles_alloc);
+    s->b.ntiles = s->ntiles;
     s->st = (cudaStream_t)stream;
     s->pair_warps = p->pair_warps;
     s->pair_ctas = p->pair_ctas_per_sm;
@@ -567,7 +655,7 @@ int sph_step(sph_t *s, double dt, int32_t nsteps)
         rec(s, PH_PERSIST, true);
         for (int done = 0; done < nsteps; done += 100000) {
             const int n = std::min(nsteps - done, 100000);
-            cudaError_t e = launch_persistent_steps(s->b, s->ninst, n, s->p.ns, s->p.cell_div, s->p.delta_mode, s->N,
+            cudaError_t e = launch_persistent_steps(s->b, s->tiled, s->ninst, n, s->p.ns, s->p.cell_div, s->p.delta_mode, s->N,
                                                     s->C, limit, s->st);
             if (e != cudaSuccess)
                 return cuda_fail(s, e, "persistent launch");
@@ -645,7 +733,7 @@ int sph_sizes(const sph_t *s, int32_t *n_inst, int64_t *n_particles, int64_t *n_
     if (n_particles)
         *n_particles = s->N;
     if (n_cells)
-        *n_cells = s->C;
+        *n_cells = public_cells(s);
     return SPH_OK;
 }
 
@@ -880,6 +968,11 @@ int sph_cells(sph_t *s, int64_t *cell, int64_t *sorted, int64_t *cell_start, int
     const int64_t N = s->N;
     if (s->b.lflag)
         enqueue_prepare(s, s->st);  // the lists keep the order of their last rebuild: rebin now
+    // the structure on the grid callers see; the pass's own one is rebuilt afterwards
+    const int base = s->base_div, fine = s->fine;
+    int rc = apply_grid(s, base, s->pub_fine);
+    if (rc)
+        return rc;
     std::vector<uint32_t> key(N);
     std::vector<int32_t> perm(N), cs((size_t)s->C + 1);
     int32_t misc[4];
@@ -888,6 +981,9 @@ int sph_cells(sph_t *s, int64_t *cell, int64_t *sorted, int64_t *cell_start, int
     CK(cudaMemcpyAsync(perm.data(), s->b.perm, 4 * N, cudaMemcpyDeviceToHost, s->st));
     CK(cudaMemcpyAsync(cs.data(), s->b.cell_start, 4 * ((size_t)s->C + 1), cudaMemcpyDeviceToHost, s->st));
     CK(cudaStreamSynchronize(s->st));
+    const int32_t n_cells = s->C;
+    if ((rc = apply_grid(s, base, fine)) != SPH_OK)
+        return rc;
     if (cell)
         for (int64_t i = 0; i < N; ++i)
             cell[i] = key[i];
@@ -895,7 +991,7 @@ int sph_cells(sph_t *s, int64_t *cell, int64_t *sorted, int64_t *cell_start, int
         for (int32_t k = 0; k < misc[0]; ++k)
             sorted[k] = perm[k];
     if (cell_start)
-        for (int64_t c = 0; c <= s->C; ++c)
+        for (int64_t c = 0; c <= n_cells; ++c)
             cell_start[c] = cs[c];
     if (n_in_out)
         *n_in_out = misc[0];
@@ -953,43 +1049,6 @@ const char *sph_phase_name(int32_t k) { return k >= 0 && k < PH_COUNT ? kPhaseNa
 
 int32_t sph_num_phases(void) { return PH_COUNT; }
 
-// Switch the grid to cells of size 2h/d: new per-instance constants, the
-// neighbour structure of the current state rebuilt on the new grid.
-static int apply_cell_div(sph_t *s, int d)
-{
-    if (d == s->p.cell_div)
-        return SPH_OK;
-    sph_params p = s->p;
-    p.cell_div = d;
-    int64_t C = 0;
-    std::vector<Inst> idev(s->ninst);
-    for (int k = 0; k < s->ninst; ++k) {
-        HostInst &hi = s->inst[k];
-        const int32_t pbase = hi.dev.pbase;
-        fill_inst(hi, p);
-        hi.dev.pbase = pbase;
-        hi.dev.cell_base = (int32_t)C;
-        C += hi.dev.ncells;
-        idev[k] = hi.dev;
-    }
-    if (C > s->C_alloc)
-        return fail(s, SPH_EINVAL, "grid larger than the workspace holds");
-    CK(cudaStreamSynchronize(s->st));
-    s->p.cell_div = d;
-    s->C = (int32_t)C;
-    s->max_active = (int32_t)std::min<int64_t>(C, s->N);
-    CK(cudaMemcpyAsync(s->b.inst, idev.data(), sizeof(Inst) * s->ninst, cudaMemcpyHostToDevice, s->st));
-    CK(cudaMemsetAsync(s->b.count, 0, sizeof(uint32_t) * ((size_t)s->C_alloc + 1), s->st));
-    enqueue_prepare(s, s->st);
-    CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(s->st));
-    if (s->graph) {
-        cudaGraphExecDestroy(s->graph);
-        s->graph = nullptr;
-    }
-    return SPH_OK;
-}
-
 int sph_autotune(sph_t *s, int32_t steps, int32_t best[3])
 {
     if (!s || steps < 1)
@@ -1000,14 +1059,18 @@ int sph_autotune(sph_t *s, int32_t steps, int32_t best[3])
         const int divs_mixed[] = {1, 2}, divs_fp64[] = {1, 2, 3};
         const int *divs = s->mode == SPH_MIXED ? divs_mixed : divs_fp64;
         const int nd = s->b.lflag ? 0 : (s->mode == SPH_MIXED ? 2 : 3);  // lists: cells of 2h + s only
-        const int d0 = s->p.cell_div;
-        int best_d = d0;
+        // the automatic grid keeps its box and is divided; a chosen one is replaced
+        int best_d = s->p.cell_div;
+        if (s->graph) {
+            cudaGraphExecDestroy(s->graph);
+            s->graph = nullptr;
+        }
         float best_d_ms = 1e30f;
         cudaEvent_t a0, a1;
         CK(cudaEventCreate(&a0));
         CK(cudaEventCreate(&a1));
         for (int k = 0; k < nd; ++k) {
-            int rc = apply_cell_div(s, divs[k]);
+            int rc = s->auto_div ? apply_grid(s, 1, divs[k]) : apply_grid(s, divs[k], 1);
             if (rc)
                 return rc;
             enqueue_pair(s, s->st);  // warm-up
@@ -1027,22 +1090,27 @@ int sph_autotune(sph_t *s, int32_t steps, int32_t best[3])
         }
         cudaEventDestroy(a0);
         cudaEventDestroy(a1);
-        int rc = apply_cell_div(s, best_d);
-        if (rc)
-            return rc;
+        if (nd > 0) {
+            int rc = s->auto_div ? apply_grid(s, 1, best_d) : apply_grid(s, best_d, 1);
+            if (rc)
+                return rc;
+            s->pub_fine = s->fine;
+        }
     }
     // (warps per CTA, CTAs per SM, particles per warp)
-    const int cand_mixed[][3] = {{8, 2, 4}, {8, 2, 2}, {8, 2, 1}, {4, 3, 2}, {16, 1, 1}};
+    const int cand_mixed[][3] = {{8, 2, 4}, {8, 2, 2}, {16, 1, 4}};
+    const int cand_wide[][3] = {{8, 2, 4}, {8, 2, 2}, {8, 2, 1}, {4, 3, 2}, {16, 1, 1}};
     const int cand_fp64[][3] = {{8, 4, 1}, {8, 8, 1}, {4, 8, 1}, {4, 16, 1}};
     const bool mixed = s->mode == SPH_MIXED;
-    const int nc = mixed ? (int)(sizeof(cand_mixed) / sizeof(cand_mixed[0])) : (int)(sizeof(cand_fp64) / sizeof(cand_fp64[0]));
+    const int(*cand)[3] = !mixed ? cand_fp64 : (s->tiled ? cand_mixed : cand_wide);
+    const int nc = !mixed ? 4 : (s->tiled ? 3 : 5);
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     float best_ms = 1e30f;
     int bw = s->pair_warps, bc = s->pair_ctas, bg = s->pair_group;
     for (int k = 0; k < (s->b.lflag ? 0 : nc); ++k) {  // the list pass has one shape
-        const int *cd = mixed ? cand_mixed[k] : cand_fp64[k];
+        const int *cd = cand[k];
         s->pair_warps = cd[0];
         s->pair_ctas = cd[1];
         s->pair_group = cd[2];
@@ -1079,8 +1147,10 @@ int sph_autotune(sph_t *s, int32_t steps, int32_t best[3])
             if (s->b.lflag)
                 CK(cudaMemsetAsync(s->b.lflag, 1, 1, s->st));  // the sort runs on rebuild requests only
             CK(cudaEventRecord(e0, s->st));
-            for (int r = 0; r < steps; ++r)
-                launch_reorder(s->b, s->mode, s->N, s->C, s->ninst, s->max_active, s->reorder_ctas, s->st);
+            for (int r = 0; r < steps; ++r) {
+                CK(cudaMemsetAsync(s->b.misc + 4, 0, sizeof(int32_t), s->st));  // the tiles are listed anew
+                launch_reorder(s->b, s->mode, s->N, s->ninst, s->reorder_ctas, s->st);
+            }
             CK(cudaEventRecord(e1, s->st));
             CK(cudaEventSynchronize(e1));
             CK(cudaGetLastError());

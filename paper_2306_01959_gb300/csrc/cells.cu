@@ -19,9 +19,10 @@ __device__ __forceinline__ bool gated_off(const int32_t *gate) { return gate && 
 // Binning of the canonical state (used at creation, after a state load and,
 // with neighbour lists, at a rebuild).
 // ---------------------------------------------------------------------------
+template <int MODE>
 __global__ void k_bin(const dvec4 *__restrict__ pos, const uint16_t *__restrict__ inst_of,
                       const Inst *__restrict__ inst, uint32_t *__restrict__ key, uint32_t *__restrict__ count,
-                      int64_t N, uint32_t C, const int32_t *gate)
+                      float *__restrict__ xof, int64_t N, uint32_t C, const int32_t *gate)
 {
     if (gated_off(gate))
         return;
@@ -30,8 +31,12 @@ __global__ void k_bin(const dvec4 *__restrict__ pos, const uint16_t *__restrict_
         dvec4 p = pos[id];
         int cx, cy, cz;
         uint32_t c = C;
-        if (cell_coords_exact(I, p.x, p.y, p.z, cx, cy, cz))
+        const bool in = MODE == SPH_FP64 ? cell_coords_exact(I, p.x, p.y, p.z, cx, cy, cz)
+                                         : cell_coords_fast(I, p.x, p.y, p.z, cx, cy, cz);
+        if (in)
             c = (uint32_t)(I.cell_base + (cz * I.n[1] + cy) * I.n[0] + cx);
+        if (MODE == SPH_MIXED && in)
+            xof[id] = x_offset(I, p.x, cx);
         key[id] = c;
         atomicAdd(&count[c], 1u);
     }
@@ -39,11 +44,13 @@ __global__ void k_bin(const dvec4 *__restrict__ pos, const uint16_t *__restrict_
 
 void launch_bin(const Bufs &b, int mode, int64_t N, int32_t C, cudaStream_t st)
 {
-    (void)mode;
     int blocks = (int)std::min<int64_t>((N + 255) / 256, 4096);
     if (blocks < 1)
         blocks = 1;
-    k_bin<<<blocks, 256, 0, st>>>(b.pos, b.inst_of, b.inst, b.key, b.count, N, (uint32_t)C, b.lflag);
+    if (mode == SPH_FP64)
+        k_bin<SPH_FP64><<<blocks, 256, 0, st>>>(b.pos, b.inst_of, b.inst, b.key, b.count, b.xof, N, (uint32_t)C, b.lflag);
+    else
+        k_bin<SPH_MIXED><<<blocks, 256, 0, st>>>(b.pos, b.inst_of, b.inst, b.key, b.count, b.xof, N, (uint32_t)C, b.lflag);
 }
 
 // One launch per phase; the bodies live in cells.cuh.
@@ -71,17 +78,15 @@ __global__ void k_scan_final(const uint32_t *__restrict__ count, const uint64_t 
     scan_final_tile(count, blocks, cell_start, active, misc, C, blockIdx.x);
 }
 
-__global__ void k_scatter(const uint32_t *__restrict__ key, uint32_t *__restrict__ count,
-                          const int32_t *__restrict__ cell_start, int32_t *__restrict__ tmp, int32_t *misc,
-                          int64_t N, const int32_t *gate)
+template <int MODE>
+__global__ void k_scatter(Bufs b, int64_t N)
 {
-    if (gated_off(gate))
+    if (gated_off(b.lflag))
         return;
-    scatter_range(key, count, cell_start, tmp, misc, N, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
-                  (int64_t)gridDim.x * blockDim.x);
+    scatter_phase<MODE>(b, N, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
-void launch_cells(const Bufs &b, int64_t N, int32_t C, cudaStream_t st)
+void launch_cells(const Bufs &b, int mode, int64_t N, int32_t C, cudaStream_t st)
 {
     int nb = (int)((C + 1 + kScanTile - 1) / kScanTile);
     k_scan_reduce<<<nb, kScanThreads, 0, st>>>(b.count, b.scan_blocks, C, b.lflag);
@@ -90,29 +95,32 @@ void launch_cells(const Bufs &b, int64_t N, int32_t C, cudaStream_t st)
     int blocks = (int)std::min<int64_t>((N + 255) / 256, 8192);
     if (blocks < 1)
         blocks = 1;
-    k_scatter<<<blocks, 256, 0, st>>>(b.key, b.count, b.cell_start, b.ptmp, b.misc, N, b.lflag);
+    if (mode == SPH_FP64)
+        k_scatter<SPH_FP64><<<blocks, 256, 0, st>>>(b, N);
+    else
+        k_scatter<SPH_MIXED><<<blocks, 256, 0, st>>>(b, N);
 }
 
+// One thread per particle, gathers in flight from as many threads as fit: the
+// ranking loop is short (about 9 particles per cell of size h on a lattice of
+// h = 2.08 dp), so a warp per cell, as the cells of 2h had, would idle most lanes.
 template <int MODE>
-__global__ void __launch_bounds__(256) k_sort_reorder(Bufs b, int32_t C, int32_t ninst)
+__global__ void __launch_bounds__(256) k_sort_reorder(Bufs b, int32_t ninst)
 {
-    (void)C;
     if (gated_off(b.lflag))
         return;
-    __shared__ uint64_t skeys[8][kSortCap];
-    sort_reorder_warps<MODE>(b, ninst, skeys[threadIdx.x >> 5], (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                             (gridDim.x * blockDim.x) >> 5);
+    if (MODE == SPH_MIXED)
+        tile_list_range(b, ninst, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+    sort_reorder_range<MODE>(b, ninst, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-void launch_reorder(const Bufs &b, int mode, int64_t N, int32_t C, int32_t ninst, int32_t max_active,
-                    int32_t ctas_per_sm, cudaStream_t st)
+void launch_reorder(const Bufs &b, int mode, int64_t N, int32_t ninst, int32_t ctas_per_sm, cudaStream_t st)
 {
-    (void)N;
-    int blocks = std::max(1, std::min((max_active + 7) / 8, sm_count() * std::max(1, ctas_per_sm)));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((N + 255) / 256, (int64_t)sm_count() * std::max(1, ctas_per_sm)));
     if (mode == SPH_FP64)
-        k_sort_reorder<SPH_FP64><<<blocks, 256, 0, st>>>(b, C, ninst);
+        k_sort_reorder<SPH_FP64><<<blocks, 256, 0, st>>>(b, ninst);
     else
-        k_sort_reorder<SPH_MIXED><<<blocks, 256, 0, st>>>(b, C, ninst);
+        k_sort_reorder<SPH_MIXED><<<blocks, 256, 0, st>>>(b, ninst);
 }
 
 }  // namespace sph

@@ -45,6 +45,9 @@ __device__ __forceinline__ bool cell_coords_fast(const Inst &I, double x, double
     return true;
 }
 
+// x offset of a particle from the origin of its cell (mixed form).
+__device__ __forceinline__ float x_offset(const Inst &I, double x, int cx) { return (float)(x - (I.lo[0] + cx * I.oc)); }
+
 // Streaming multiprocessors of the current device (queried once per device;
 // grids of the memory-bound kernels are capped at a multiple of it).
 inline int sm_count()
@@ -176,6 +179,20 @@ __device__ __forceinline__ int inst_of_cell(const Inst *inst, int ninst, int32_t
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
         if (inst[mid].cell_base <= c)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    return lo;
+}
+
+// Instance owning a global tile id.
+__device__ __forceinline__ int inst_of_tile(const Inst *inst, int ninst, int32_t t)
+{
+    int lo = 0, hi = ninst - 1;
+    while (lo < hi) {
+        int mid = (lo + hi + 1) >> 1;
+        if (inst[mid].tile_base <= t)
             lo = mid;
         else
             hi = mid - 1;

@@ -62,6 +62,8 @@ __device__ __forceinline__ void rebin_particle(const Bufs &b, const Inst &I, int
                           : cell_coords_fast(I, p.x, p.y, p.z, cx, cy, cz);
     if (in)
         c = (uint32_t)(I.cell_base + (cz * I.n[1] + cy) * I.n[0] + cx);
+    if (!exact && in)
+        b.xof[id] = x_offset(I, p.x, cx);
     b.key[id] = c;
     atomicAdd(&b.count[c], 1u);
 }

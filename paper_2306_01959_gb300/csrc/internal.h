@@ -44,14 +44,20 @@ struct Inst {
     double h, c0, rho0, alpha, delta, gamma, g, cfl, mass, B, eta2, sup2, dt_min, ztop, dp;
     double kF;  // 105 / (16 pi h^5): grad_i W_ij = -kF (1 - q/2)^3 (r_i - r_j)
     double kW;  // 21 / (16 pi h^3)
+    // spacing of the cell origins of the mixed form's FP32 offsets: cs rounded to
+    // 20 mantissa bits, so that a shift by a few cells is exact in FP32 (with
+    // neighbour lists: cs)
+    double oc;
     int32_t n[3];
     int32_t cell_base, ncells;
+    // tiles of the mixed pair pass: boxes of tdim cells, ntile per axis
+    int32_t tdim[3], ntile[3], tile_base;
     int32_t pbase, np, nf, nw, no, ng;
     int32_t csound;
     int32_t delta_mode;  // SPH_DELTA_ALL_FLUID or SPH_DELTA_FULL_SUPPORT
     double gate_v[3];  // prescribed velocity of the gate particles
     // FP32 copies for the mixed form
-    float csf, hf, inv_hf, c0f, rho0f, inv_rho0f, alphaf, massf, Bf, eta2f, sup2f, kFf, dfac;  // dfac = 2 delta h c0
+    float csf, ocf, hf, inv_hf, c0f, rho0f, inv_rho0f, alphaf, massf, Bf, eta2f, sup2f, kFf, dfac;  // dfac = 2 delta h c0
     float gammaf, gf;
     float gate_vf[3];
     // FP64 form: squared radius of a conservative FP32 pre-test on the FP32
@@ -79,9 +85,13 @@ struct Bufs {
     uint32_t *count;         // C + 1 per-cell counters (zero between steps)
     int32_t *cell_start;     // C + 2 lower bounds into the sorted order
     int32_t *active;         // non-empty cells in ascending order
+    int32_t *tiles;          // mixed form: non-empty tiles (misc[4] of them, no fixed order)
+    int32_t ntiles;          // mixed form: tiles of all grids; 0 with wide neighbourhoods (pair_wide.cuh)
     uint64_t *scan_blocks;   // block partials of the cell scan
     int32_t *perm;           // sorted index -> particle id
-    int32_t *ptmp;           // scatter target before the per-cell id sort
+    int32_t *ptmp;           // FP64 form: scatter target before the per-cell id sort
+    uint64_t *pkey;          // mixed form: the same with the sort key, x offset (orderable bits) << 32 | id
+    float *xof;              // mixed form, id order: x offset from the origin of the particle's cell
     int32_t *scell;          // sorted index -> cell
     // sorted particle data for the pair kernel
     void *sA;                // FP64: dvec4 (x, y, z, rho); mixed: float4 (offset to cell origin, rho - rho0)
@@ -117,7 +127,8 @@ struct Bufs {
     double *dt_fixed;        // [1]
     long long *step;         // [1] step counter
     int32_t *euler;          // [1] 1 when the current step is first-order
-    int32_t *misc;           // [0] n_in, [1] n_active, [2] status, [3] pair work queue
+    int32_t *misc;           // [0] n_in, [1] n_active, [2] status, [3] pair work queue,
+                             // [4] n_tiles
     unsigned *bar;           // grid-barrier counter of the persistent time loop
     Inst *inst;              // [ninst]
     // probes and diagnostics scratch
@@ -130,19 +141,24 @@ struct Bufs {
 constexpr int kMaxProbe = 65536;
 constexpr int kDiagBlocks = 256;
 constexpr int kScanTile = 4096;
+// Particles a CTA of the mixed pair pass stages: two CTAs of 8 warps fill the
+// shared memory of an SM.
+constexpr int kStage = 2880;
 
 // Kernel launchers (implemented in the .cu files).  All launch on `st`.
 void launch_bin(const Bufs &b, int mode, int64_t N, int32_t C, cudaStream_t st);
-void launch_cells(const Bufs &b, int64_t N, int32_t C, cudaStream_t st);
-void launch_reorder(const Bufs &b, int mode, int64_t N, int32_t C, int32_t ninst, int32_t max_active,
-                    int32_t ctas_per_sm, cudaStream_t st);
+void launch_cells(const Bufs &b, int mode, int64_t N, int32_t C, cudaStream_t st);
+void launch_reorder(const Bufs &b, int mode, int64_t N, int32_t ninst, int32_t ctas_per_sm, cudaStream_t st);
 // neighbours: the pass must write every particle's nneigh (with
 // pair_symmetric the partners' counts are left out of time steps).
 void launch_pair_fp64(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas,
                       int32_t delta_mode, bool neighbours, cudaStream_t st);
-void launch_pair_mixed(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int32_t warps,
-                       int32_t ctas, int32_t group, int32_t compensated, int32_t max_active, bool count,
-                       int32_t delta_mode, cudaStream_t st);
+// stats: also write every particle's neighbour and pair counts and sum the work
+// counts (a separate instantiation, so that time steps pay nothing for them).
+void launch_pair_mixed(const Bufs &b, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas, int32_t group,
+                       int32_t compensated, bool stats, int32_t delta_mode, cudaStream_t st);
+void launch_pair_wide(const Bufs &b, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas, int32_t group,
+                      int32_t compensated, bool stats, int32_t delta_mode, cudaStream_t st);
 // Neighbour lists (pair_list.cu): the build (when lflag[0] requests it) and
 // the list pass; the gather of a step that keeps the lists.
 void launch_list_pass(const Bufs &b, int64_t N, int32_t ninst, int32_t delta_mode, cudaStream_t st);
@@ -159,7 +175,7 @@ void launch_probe_force(const Bufs &b, int mode, int32_t inst, int32_t ninst, in
                         cudaStream_t st);
 // One cooperative launch of nsteps Verlet steps of the mixed form over all
 // instances (persist.cu); spin_limit bounds every grid-barrier wait.
-cudaError_t launch_persistent_steps(const Bufs &b, int32_t ninst, int32_t nsteps, int32_t ns, int32_t cell_div,
+cudaError_t launch_persistent_steps(const Bufs &b, bool tiled, int32_t ninst, int32_t nsteps, int32_t ns, int32_t cell_div,
                                     int32_t delta_mode, int64_t N, int32_t C, long long spin_limit, cudaStream_t st);
 void launch_diagnostics(const Bufs &b, int mode, int32_t inst, int32_t C, cudaStream_t st);
 
@@ -172,7 +188,14 @@ struct HostInst {
 
 int validate_instance(const sph_instance &in, const sph_params &p, std::string &err);
 int effective_cell_div(const sph_params &p);
-void fill_inst(HostInst &hi, const sph_params &p);
+// cell_div cells per 2h; the grid spans the same box whatever `fine` is, which
+// divides each of those cells again (the mixed form's own grid, see sph_s).
+// tiled: the mixed form's tiled pair pass will run on it.
+void fill_inst(HostInst &hi, const sph_params &p, int fine = 1, bool tiled = false);
+// Whether the tiled pair pass (pair_mixed.cuh) suits an instance.
+bool tiles_fit(const sph_instance &in, const sph_params &p);
+// Tile dimensions of every instance (mixed form) and their count; n_total particles in all.
+int64_t fill_tiles(std::vector<HostInst> &inst, int cell_div, int64_t n_total);
 void build_scene(const HostInst &hi, const sph_params &p, double *r, double *rho, uint8_t *type);
 
 }  // namespace sph

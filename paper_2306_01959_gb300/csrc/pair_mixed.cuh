@@ -2,68 +2,78 @@
 // Mixed-precision form of the pair pass (Eqs. 3-8), device body: FP32 pair
 // arithmetic on cell-relative offsets, with compensated FP32 accumulation.
 //
-// Work decomposition (persistent CTAs, one work item = one non-empty home
-// cell):
-//  1. The CTA stages the particles of every cell within cell_div cells of the
-//     home cell into shared memory.  Rows of cells along x are contiguous in
-//     the sorted order, so each (dy, dz) row is one copy (one warp per row).
-//     Every staged position is shifted from its own cell origin to the home
-//     cell origin; the FP32 offsets stay small (|x| < (cell_div + 1) cs), so
-//     relative distances keep full FP32 precision however large the tank is.
-//  2. A warp takes G particles i of the home cell at a time (G = 1, 2 or 4).
-//     Lanes test 32 staged candidates per step against the G particles
-//     (|r_ij|^2 < (2h)^2), one shared-memory load serving all G tests; the
-//     interacting candidates are compacted by ballot into one list per
-//     particle.  The pair arithmetic then runs over each list on 32 full
-//     lanes (only the last batch of a list is partial).
-//  3. Each lane accumulates its pair terms; the 32 lane sums of a particle are
-//     combined by a shuffle tree.  If a neighbourhood holds more particles
-//     than the staging buffer, it is processed in chunks and the partial sums
-//     are carried in shared memory between chunks.
+// Work decomposition (persistent CTAs; one work item = one non-empty tile, a
+// box of tdim cells):
+//  1. The CTA stages the particles of the tile and of every cell within
+//     cell_div cells of it into shared memory.  Rows of cells along x are
+//     contiguous in the sorted order and sorted by x, so each (y, z) row is one
+//     copy.  Every staged position is shifted from its own cell origin to the
+//     tile's centre cell; the FP32 offsets stay small, so relative distances
+//     keep full FP32 precision however large the tank is.  The origins lie on a
+//     lattice whose spacing (Inst::oc) has few mantissa bits, so the shifts are
+//     exact in FP32.
+//  2. A warp takes a cluster of G particles (G = 2 or 4) that follow one
+//     another along x in one row of the tile: compact in space, so that the
+//     candidates near any of them are mostly near all of them.  For each row of
+//     cells around, a binary search gives the exact x-window of the cluster.
+//  3. Lanes test the windowed candidates, 32 at a time, against the G particles
+//     in packed FP32x2 arithmetic; those within 2h of any of them are compacted
+//     by ballot into ONE list for the cluster.
+//  4. The pair arithmetic runs over that list, one candidate per lane, for all
+//     G particles at once: a candidate's data is loaded and prepared once for G
+//     pair terms, and two particles share each packed FP32x2 instruction.  A
+//     candidate beyond 2h of a particle has its (1 - q/2) set to zero, which
+//     makes its terms exactly zero.
+//  5. The 32 lane sums of the cluster are combined by a value-splitting shuffle
+//     butterfly and written out; nothing is carried between warps.
+// A tile whose neighbourhood exceeds the staging buffer (a dense clump), or that
+// holds values a zero weight could not cancel (non-finite or huge), takes the
+// same path with the candidates read from global memory and every term masked.
+//
+// Why this split: one list per particle, a group's particles spread over a cell of
+// 2h (pair_wide.cuh), costs four ballots and prefix counts per 32 candidates, 900
+// candidate tests per particle and a load of the candidate per pair term: 1.45e9
+// warp instructions on the 0.9 M-particle obstacle case.  Rows of cross-section h
+// leave 640 tests, one list per cluster a quarter of the ballots, and the pair terms
+// evaluated for nothing (1.4 per useful one) cost less than the tests and stores
+// they replace: 0.90e9 instructions, 1.98 -> 1.17 ms per pass (8.1 M particles:
+// 19.4 -> 11.5 ms; h = 1.5 dp, 2.0 M particles: 3.38 -> 1.61 ms).
+// What bounds it: issue slots and fixed latencies at 16 warps per SM (128
+// registers); a list step of 32 candidates takes about 170 warp instructions for 4
+// pair terms, 135 of them arithmetic, a step of the sweep about 50.
 //
 // Compensated sums: the lane sums (at most a few tens of terms each) are
-// combined across lanes and across chunks with Knuth's TwoSum, carrying the
-// rounding error of every addition, so the result is the compensated sum of
-// the lane partials.
+// combined across lanes with Knuth's TwoSum, carrying the rounding error of
+// every addition, so the result is the compensated sum of the lane partials.
+#include <type_traits>
+
 #include "device.cuh"
 
 namespace sph {
 
-constexpr int kMaxRowsM = 49;  // (2 * 3 + 1)^2 rows at cell_div = 3
-constexpr int kMaxI = 128;     // particles of a home cell handled per pass
-// capacity of a per-particle candidate list (entries); a list without room for
-// the next row window is drained first, so the capacity only bounds shared memory
-constexpr int kList = 512;
+constexpr int kMaxRowsM = 96;  // staged rows of a tile: (tdim_y + 2 cell_div)(tdim_z + 2 cell_div)
+constexpr int kMaxHome = 16;   // rows of the tile itself
+constexpr int kMaxWin = 51;    // rows within cell_div of a particle's, (2 * 3 + 1)^2, and the end of the list
+constexpr int kList = 448;     // capacity of a warp's candidate list; drained when short of room
 
-// Staging capacity of a CTA (a multiple of 32): the whole neighbourhood of a
-// typical home cell at each cell size.
-__host__ __device__ __forceinline__ int mixed_max_stage(int cell_div)
-{
-    return cell_div == 1 ? 2048 : (cell_div == 2 ? 1536 : 1280);
-}
-
-// Dynamic shared memory of a CTA of NW warps with G particles per warp.
-__host__ __device__ __forceinline__ size_t mixed_dyn_smem(int max_stage, int NW, int G)
-{
-    size_t dyn = (size_t)max_stage * (2 * sizeof(float4) + 1);
-    dyn = (dyn + 15) & ~(size_t)15;
-    return dyn + (size_t)NW * G * kList * sizeof(uint16_t);
-}
-
-struct RowM {
-    int32_t bnd[8];  // cell_start of cells x0 .. x1 + 1 (x-cell boundaries); -1 outside the grid
-};
+// Dynamic shared memory of a CTA of NW warps: staged A and B (with a dummy slot
+// out of everything's reach) and type flags, then the warps' lists and windows.
+constexpr int kOffB = (kStage + 1) * (int)sizeof(float4);  // byte offsets in it
+constexpr int kOffF = 2 * kOffB;
+constexpr int kOffWarp = (kOffF + kStage + 1 + 15) / 16 * 16;
+constexpr int kWarpBytes = kList * (int)sizeof(int32_t) + (kMaxWin + 1) * (int)sizeof(int2);
+__host__ __device__ __forceinline__ size_t mixed_dyn_smem(int NW) { return kOffWarp + (size_t)NW * kWarpBytes; }
 
 struct PairSmem {
-    int32_t item;
+    int32_t item;   // tile, -1 when the queue is exhausted
+    int32_t next;   // next cluster of the tile
+    int32_t wild;   // a staged value is not finite or huge: take the masked path
     unsigned long long st_ff, st_visc, st_cand;  // work counts of this CTA
-    int32_t pre[kMaxRowsM + 1];
-    RowM row[kMaxRowsM];
-    float acc[kMaxI][9];  // drho, ax, ay, az, mumax, and the error terms of the 4 sums
-    float dd[kMaxI][2];   // SPH_DELTA_FULL_SUPPORT: the delta term of Eq. 7 and its error term
-    int32_t nb[kMaxI];    // SPH_DELTA_FULL_SUPPORT: the particle has a boundary neighbour
-    int32_t nn[kMaxI];
-    int32_t np[kMaxI];
+    int32_t pre[kMaxRowsM + 1];  // staged index of each row's first particle
+    int32_t gs[kMaxRowsM];       // its sorted index
+    int32_t hst[kMaxHome], hlen[kMaxHome];  // the tile's own particles of each home row
+    int32_t hyz[kMaxHome];                  // y | z << 16 of the home row in the tile
+    int32_t hpre[kMaxHome + 1];             // clusters before each home row
 };
 
 __device__ __forceinline__ void two_sum(float &s, float &e, float x)
@@ -206,36 +216,190 @@ __device__ __forceinline__ void hit_tests(const SweepPos<G> &sp, const float4 a,
     }
 }
 
-// ---------------------------------------------------------------------------
-// Combination of the 32 lane sums of one particle and of the chunks.
-// ---------------------------------------------------------------------------
-// The 4G sums (d rho/dt and the three acceleration components of each of the G
-// particles of a warp) are combined across the 32 lanes by a value-splitting
-// butterfly: at each of the first log2(4G) levels a lane keeps half of its
-// values and adds its partner's copies of them, so a level moves half as many
-// values as the one before; the remaining levels are a plain butterfly on the
-// one value left.  Lane 32/(4G) * v then holds the total of value v and adds it
-// to the particle's running sums in shared memory (TwoSum-compensated when
-// COMP).  mumax is a plain max butterfly; the counts are warp-uniform.
-template <int G, bool COMP, bool DFS>
-__device__ __forceinline__ void combine_group(PairSmem &S, const LaneAcc (&acc)[G], const int32_t (&slot)[G],
-                                              const bool (&valid)[G], const int (&nsum)[G], const int (&npair)[G],
-                                              unsigned nbits)
+__device__ __forceinline__ float rcp_ftz(float x)
 {
-    constexpr int K = 4 * G;
-    const int lane = threadIdx.x & 31;
-    float v[K], e[K];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        v[4 * g + 0] = acc[g].drho;
-        v[4 * g + 1] = acc[g].ax;
-        v[4 * g + 2] = acc[g].ay;
-        v[4 * g + 3] = acc[g].az;
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float sqrt_ftz(float x)
+{
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// A value the compiler keeps in its register instead of computing it again
+// wherever it is used (lane and per-warp offsets in the inner loops).
+__device__ __forceinline__ int keep(int v)
+{
+    asm volatile("" : "+r"(v));
+    return v;
+}
+// Shared-memory accesses of the inner loops by 32-bit address (the window base
+// stays in a register; immediate offset OFF).
+template <int OFF>
+__device__ __forceinline__ float4 lds_f4(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4 + %5];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(a), "n"(OFF)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ int32_t lds_i32(uint32_t a)
+{
+    int32_t v;
+    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float lds_f32(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ int2 lds_i2(uint32_t a)
+{
+    int2 v;
+    asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ uint32_t lds_u8(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u8 %0, [%1 + %2];" : "=r"(v) : "r"(a), "n"(OFF) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts_i32(uint32_t a, int32_t v)
+{
+    asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts_i2(uint32_t a, int2 v)
+{
+    asm volatile("st.shared.v2.s32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+
+// Two particles of a cluster.  Their velocities are negated, as their positions
+// are in pair_cluster, so that differences are additions.
+struct PackI {
+    float2 d, rho, inv, Pr, nac;  // rho - rho0, rho, 1/rho, P/rho, -alpha h c
+    float2 nux, nuy, nuz;
+};
+struct PackAcc {
+    float2 drho, ax, ay, az, mu;  // in units of t^3 (the caller scales by m F(0)); mu / h
+    float2 dd;                    // delta term of Eq. 7 summed apart (SPH_DELTA_FULL_SUPPORT only)
+};
+// One candidate.
+struct CandJ {
+    float x, y, z, ux, uy, uz, d, rho, inv, vd, P, nac;  // vd = 2 delta h c0 / rho, 0 for a boundary particle
+};
+
+__device__ __forceinline__ CandJ load_cand(const PairConst &k, const float4 a, const float4 b, bool fluid)
+{
+    CandJ j;
+    const float xj = fmaf(a.w, k.inv_rho0, 1.f);
+    j.x = a.x;
+    j.y = a.y;
+    j.z = a.z;
+    j.ux = b.x;
+    j.uy = b.y;
+    j.uz = b.z;
+    j.d = a.w;
+    j.rho = k.rho0 + a.w;
+    j.inv = rcp_ftz(j.rho);
+    j.vd = fluid ? k.dfac * j.inv : 0.f;
+    j.P = b.w;
+    j.nac = k.csound_const ? k.nahc0 : k.nahc0 * xj * xj * xj;
+    return j;
+}
+
+// r_ij = r_j - r_i and |r_ij|^2 for two particles i (negated positions); the
+// same arithmetic in the candidate sweep and in the pair terms, so that both
+// agree on which pairs lie within 2h.  The first operations take the candidate's
+// scalar with each half: a packed operand (v, v) would cost two moves.
+__device__ __forceinline__ float2 dist2_pack(float x, float y, float z, float2 nx, float2 ny, float2 nz, float2 &dx,
+                                             float2 &dy, float2 &dz)
+{
+    dx = make_float2(x + nx.x, x + nx.y);
+    dy = make_float2(y + ny.x, y + ny.y);
+    dz = make_float2(z + nz.x, z + nz.y);
+    return __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+}
+
+// The pair terms of candidate j on two particles.  fs: see below (ALLF: all of
+// the cluster are fluid), fj: the candidate is fluid.  SAFE: the terms are
+// masked one by one instead of through a zero t.  Returns the masks of
+// interacting pairs (bits 0, 1) and of approaching ones among them (bits 2, 3).
+template <bool ALLF, bool DFS, bool SAFE>
+__device__ __forceinline__ unsigned pair_terms_pack(const PairConst &k, const PackI &p, float2 nx, float2 ny, float2 nz,
+                                                    const CandJ &j, float2 fs, bool fj, PackAcc &a)
+{
+    float2 dx, dy, dz;
+    const float2 r2 = dist2_pack(j.x, j.y, j.z, nx, ny, nz, dx, dy, dz);
+    // pairs of two boundary particles do not interact: fs is (2h)^2 for a fluid particle, 0 for a boundary one
+    const bool p0 = r2.x < (ALLF || fj ? k.sup2 : fs.x), p1 = r2.y < (ALLF || fj ? k.sup2 : fs.y);
+    float2 t = make_float2(fmaf(-k.half_inv_h, sqrt_ftz(r2.x), 1.f), fmaf(-k.half_inv_h, sqrt_ftz(r2.y), 1.f));
+    t.x = p0 ? t.x : 0.f;
+    t.y = p1 ? t.y : 0.f;
+    const float2 t3 = __fmul2_rn(__fmul2_rn(t, t), t);  // m_j F / (m F(0))
+    const float2 dux = make_float2(j.ux + p.nux.x, j.ux + p.nux.y), duy = make_float2(j.uy + p.nuy.x, j.uy + p.nuy.y),
+                 duz = make_float2(j.uz + p.nuz.x, j.uz + p.nuz.y);
+    const float2 udr = __ffma2_rn(duz, dz, __ffma2_rn(duy, dy, __fmul2_rn(dux, dx)));  // u_ij . r_ij
+    // Eq. 7: u_ij . r_ij, plus between fluid particles the delta term 2 delta h c0 (rho_i - rho_j) / rho_j
+    float2 g = make_float2(p.d.x - j.d, p.d.y - j.d);
+    if (!ALLF) {
+        g.x = fs.x > 0.f ? g.x : 0.f;
+        g.y = fs.y > 0.f ? g.y : 0.f;
     }
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-        e[k] = 0.f;
-    int idx = 0;  // which of the K values this lane ends up holding
+    // Eqs. 4-5: mu = h muh; min(muh, 0) switches the viscosity on for approaching pairs
+    float2 ire = make_float2(rcp_ftz(r2.x + k.eta2), rcp_ftz(r2.y + k.eta2));
+    ire.x = p0 ? ire.x : 0.f;  // a masked pair leaves the running maximum of mu alone
+    ire.y = p1 ? ire.y : 0.f;
+    const float2 muh = __fmul2_rn(udr, ire);
+    const float2 mn = make_float2(fminf(muh.x, 0.f), fminf(muh.y, 0.f));
+    const float2 ir = make_float2(rcp_ftz(p.rho.x + j.rho), rcp_ftz(p.rho.y + j.rho));
+    const float2 nac = make_float2(p.nac.x + j.nac, p.nac.y + j.nac);
+    const float2 visc = __fmul2_rn(__fmul2_rn(nac, mn), ir);
+    // Eq. 3: a_i += m_j F ((P_i + P_j)/(rho_i rho_j) + Pi_ij) r_ij
+    float2 coef = make_float2(fmaf(fmaf(j.P, p.inv.x, p.Pr.x), j.inv, visc.x), fmaf(fmaf(j.P, p.inv.y, p.Pr.y), j.inv, visc.y));
+    coef = __fmul2_rn(coef, t3);
+    if (SAFE) {
+        coef.x = p0 ? coef.x : 0.f;
+        coef.y = p1 ? coef.y : 0.f;
+        const float2 del = make_float2(g.x * j.vd, g.y * j.vd);
+        float2 c = __fmul2_rn(t3, DFS ? udr : __fadd2_rn(udr, del));
+        a.drho = __fadd2_rn(a.drho, make_float2(p0 ? c.x : 0.f, p1 ? c.y : 0.f));
+        if (DFS) {
+            c = __fmul2_rn(t3, del);
+            a.dd = __fadd2_rn(a.dd, make_float2(p0 ? c.x : 0.f, p1 ? c.y : 0.f));
+        }
+    } else if (DFS) {
+        a.drho = __ffma2_rn(t3, udr, a.drho);
+        a.dd = __ffma2_rn(t3, make_float2(g.x * j.vd, g.y * j.vd), a.dd);
+    } else {
+        a.drho = __ffma2_rn(t3, make_float2(fmaf(g.x, j.vd, udr.x), fmaf(g.y, j.vd, udr.y)), a.drho);
+    }
+    a.ax = __ffma2_rn(coef, dx, a.ax);
+    a.ay = __ffma2_rn(coef, dy, a.ay);
+    a.az = __ffma2_rn(coef, dz, a.az);
+    a.mu.x = fmaxf(a.mu.x, muh.x);
+    a.mu.y = fmaxf(a.mu.y, muh.y);
+    return (p0 ? 1u : 0u) | (p1 ? 2u : 0u) | (p0 && udr.x < 0.f ? 4u : 0u) | (p1 && udr.y < 0.f ? 8u : 0u);
+}
+
+// Combination of the 32 lane sums of the K = 4 G values of a cluster by a
+// value-splitting butterfly: at each of the first log2 K levels a lane keeps
+// half of its values and adds its partner's copies of them, so a level moves
+// half as many values as the one before; the remaining levels add the one value
+// left.  Lane (32 / K) m then holds, for one value `idx`, the total and (COMP)
+// its error term.
+template <int K, bool COMP>
+__device__ __forceinline__ int warp_split_totals(float (&v)[K], float (&e)[K], int lane)
+{
+    int idx = 0;
 #pragma unroll
     for (int k = K, o = 16; k > 1; k >>= 1, o >>= 1) {
         const bool upper = (lane & o) != 0;
@@ -247,9 +411,12 @@ __device__ __forceinline__ void combine_group(PairSmem &S, const LaneAcc (&acc)[
             const float send = upper ? v[i] : v[i + half];
             const float recv = __shfl_xor_sync(0xffffffffu, send, o);
             if (COMP) {
-                const float ke = upper ? e[i + half] : e[i];
-                const float se = upper ? e[i] : e[i + half];
-                float ee = ke + __shfl_xor_sync(0xffffffffu, se, o);
+                float ee = 0.f;
+                if (k < K) {  // the lanes start without error terms
+                    const float ke = upper ? e[i + half] : e[i];
+                    const float se = upper ? e[i] : e[i + half];
+                    ee = ke + __shfl_xor_sync(0xffffffffu, se, o);
+                }
                 float sum = keep;
                 two_sum(sum, ee, recv);
                 v[i] = sum;
@@ -270,39 +437,296 @@ __device__ __forceinline__ void combine_group(PairSmem &S, const LaneAcc (&acc)[
             v[0] += recv;
         }
     }
-    float mu[G];
+    return idx;
+}
+
+// Geometry of the tile a CTA works on.
+struct TileGeo {
+    int32_t t0[3];   // first cell
+    int32_t cen[3];  // cell whose origin is the frame's
+    int nry;         // staged rows along y
+    int32_t total;   // staged particles
+    int row0, row1;  // (dy & 0xff) | dz << 8 of this lane's row around a particle's (the first 32, the next)
+    float dy0, dz0;  // distance of the true cell lattice from the frame's lattice at the frame's origin
+};
+
+// One cluster (G particles of one home row) by one warp.  STG: candidates from
+// the staged copy; otherwise from global memory, with every term masked.
+template <int NW, int G, bool COMP, bool STAT, bool DFS, bool STG>
+__device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const PairConst &kc, const TileGeo &T, int kdiv,
+                                             int q, uint32_t st, uint32_t list, int lane, PairSmem &S,
+                                             unsigned (&lc)[2], unsigned long long &wc_cand)
+{
+    constexpr int P = G / 2;
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t win = list + kList * (uint32_t)sizeof(int32_t);  // this warp's windows follow its list
+    const float4 *gA = reinterpret_cast<const float4 *>(b.sA);
+    const float4 *gB = reinterpret_cast<const float4 *>(b.sB);
+    const int32_t dummy = STG ? kStage : -1;
+    // position and density offset of candidate t in the tile's frame
+    auto cand_a = [&](int32_t t) -> float4 {
+        if (STG)
+            return lds_f4<0>(st + 16u * (uint32_t)t);
+        if (t < 0)
+            return make_float4(1e15f, 1e15f, 1e15f, 0.f);
+        float4 a = gA[t];
+        int cx, cy, cz;
+        decompose(I, b.scell[t], cx, cy, cz);
+        a.x += (float)(cx - T.cen[0]) * I.ocf;
+        a.y += (float)(cy - T.cen[1]) * I.ocf;
+        a.z += (float)(cz - T.cen[2]) * I.ocf;
+        return a;
+    };
+    auto cand_x = [&](int32_t t) -> float { return STG ? lds_f32(st + 16u * (uint32_t)t) : cand_a(t).x; };
+    auto cand_b = [&](int32_t t) -> float4 {
+        if (STG)
+            return lds_f4<kOffB>(st + 16u * (uint32_t)t);
+        return t < 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : gB[t];
+    };
+    auto cand_f = [&](int32_t t) -> bool {
+        return STG ? lds_u8<kOffF>(st + (uint32_t)t) == T_FLUID : (t >= 0 && b.sflag[t] == T_FLUID);
+    };
+
+    // home row of cluster q, its particles
+    const int nh = I.tdim[1] * I.tdim[2];
+    const int rr = __popc(__ballot_sync(0xffffffffu, lane < nh && S.hpre[min(lane, nh - 1) + 1] <= q));
+    const int k0 = (q - S.hpre[rr]) * G;
+    const int nreal = min(G, S.hlen[rr] - k0);  // a short cluster repeats its last particle; nothing is stored for it
+    const int hy = S.hyz[rr] & 0xffff, hz = S.hyz[rr] >> 16;
+    const int32_t s0 = S.hst[rr] + k0;
+    const int hrow = (hz + kdiv) * T.nry + hy + kdiv;
+    const int32_t i0 = STG ? S.pre[hrow] + (s0 - S.gs[hrow]) : s0;
+    float2 nx[P], ny[P], nz[P];
+    unsigned fl = 0;  // bit g: particle g is fluid
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-        mu[g] = acc[g].mumax;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            mu[g] = fmaxf(mu[g], __shfl_xor_sync(0xffffffffu, mu[g], o));
+        const int32_t t = i0 + min(g, nreal - 1);
+        const float4 a = cand_a(t);
+        (g & 1 ? nx[g / 2].y : nx[g / 2].x) = -a.x;
+        (g & 1 ? ny[g / 2].y : ny[g / 2].x) = -a.y;
+        (g & 1 ? nz[g / 2].y : nz[g / 2].x) = -a.z;
+        fl |= (cand_f(t) ? 1u : 0u) << g;
     }
-    if ((lane & (32 / K - 1)) == 0) {
-        const int gsel = idx >> 2, c = idx & 3;
-        int32_t sl = slot[0];
-        bool ok = valid[0];
-#pragma unroll
-        for (int g = 1; g < G; ++g)
-            if (gsel == g) {
-                sl = slot[g];
-                ok = valid[g];
+    constexpr unsigned kAll = (1u << G) - 1u;
+
+    // Exact x-windows: a candidate of a row can lie within 2h of particle g only
+    // if |x_j - x_g| <= sqrt((2h)^2 - d^2), d the distance from g to the row's
+    // y-z cross-section; the windows of the G particles are merged.  One lane per
+    // row; the non-empty windows are listed in `win`.
+    const int nrow = (2 * kdiv + 1) * (2 * kdiv + 1);
+    int nwin = 0;
+    for (int r0 = 0; r0 < nrow; r0 += 32) {
+        int32_t lo = 0, hi = 0;
+        if (r0 + lane < nrow) {
+            const int dyz = r0 ? T.row1 : T.row0;
+            const int dy = (int)(int8_t)(dyz & 0xff), dz = dyz >> 8;
+            const int row = hrow + dz * T.nry + dy;
+            int32_t ra = S.pre[row], rb = S.pre[row + 1];
+            if (!STG) {
+                rb = S.gs[row] + (rb - ra);
+                ra = S.gs[row];
             }
-        if (ok) {
-            float *A = S.acc[sl];
-            if (COMP)
-                two_sum(A[c], A[5 + c], v[0] + e[0]);
-            else
-                A[c] += v[0];
+            if (ra < rb) {
+                const float y0 = (float)(T.t0[1] + hy + dy - T.cen[1]) * kc.cs + T.dy0;
+                const float z0 = (float)(T.t0[2] + hz + dz - T.cen[2]) * kc.cs + T.dz0;
+                float xl = 3.0e38f, xh = -3.0e38f;
+                const float eps = 2e-6f * kc.cs;
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const float px = -(g & 1 ? nx[g / 2].y : nx[g / 2].x), py = -(g & 1 ? ny[g / 2].y : ny[g / 2].x),
+                                pz = -(g & 1 ? nz[g / 2].y : nz[g / 2].x);
+                    const float ey = fmaxf(fmaxf(y0 - py, py - (y0 + kc.cs)) - eps, 0.f);
+                    const float ez = fmaxf(fmaxf(z0 - pz, pz - (z0 + kc.cs)) - eps, 0.f);
+                    const float rem = kc.sup2 - ey * ey - ez * ez;
+                    if (rem > 0.f) {
+                        const float w = sqrt_ftz(rem) * 1.0001f + eps;
+                        xl = fminf(xl, px - w);
+                        xh = fmaxf(xh, px + w);
+                    }
+                }
+                if (xl <= xh) {
+                    int32_t a0 = ra, a1 = rb;
+                    while (a0 < a1) {
+                        const int32_t m = (a0 + a1) >> 1;
+                        if (cand_x(m) < xl)
+                            a0 = m + 1;
+                        else
+                            a1 = m;
+                    }
+                    lo = a0;
+                    a1 = rb;
+                    while (a0 < a1) {
+                        const int32_t m = (a0 + a1) >> 1;
+                        if (cand_x(m) <= xh)
+                            a0 = m + 1;
+                        else
+                            a1 = m;
+                    }
+                    hi = a0;
+                }
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, lo < hi);
+        if (lo < hi)
+            sts_i2(win + 8u * (nwin + __popc(m & lt)), make_int2(lo, hi));
+        nwin += __popc(m);
+        if (lane == 0)
+            sts_i2(win + 8u * nwin, make_int2(1, 1));  // an empty window ends the list (an odd one out is paired with it)
+        __syncwarp();
+        if (STAT) {
+            const int c = warp_sum(hi - lo);
+            if (lane == 0)
+                wc_cand += (unsigned long long)c;
         }
     }
+    __syncwarp();
+
+    PackAcc acc[P];
+#pragma unroll
+    for (int h = 0; h < P; ++h)
+        acc[h] = PackAcc{dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
+    int nn[G], np[G];
+    unsigned nbits = 0;  // bit g: particle g has a boundary particle within 2h
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+        nn[g] = np[g] = 0;
+
+    // Pair terms of list entries [0, n), n a multiple of 32.
+    auto evaluate = [&](int n) {
+        PackI pi[P];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int32_t t = i0 + min(g, nreal - 1);
+            const float d = cand_a(t).w;
+            const float4 bb = cand_b(t);
+            const float rho = kc.rho0 + d, inv = rcp_ftz(rho), xi = fmaf(d, kc.inv_rho0, 1.f);
+            const float nac = kc.csound_const ? kc.nahc0 : kc.nahc0 * xi * xi * xi;
+            PackI &p = pi[g / 2];
+#define SPH_SET(f, val) (g & 1 ? p.f.y : p.f.x) = (val)
+            SPH_SET(d, d);
+            SPH_SET(rho, rho);
+            SPH_SET(inv, inv);
+            SPH_SET(Pr, bb.w * inv);
+            SPH_SET(nac, nac);
+            SPH_SET(nux, -bb.x);
+            SPH_SET(nuy, -bb.y);
+            SPH_SET(nuz, -bb.z);
+#undef SPH_SET
+        }
+        float2 fs[P];
+#pragma unroll
+        for (int h = 0; h < P; ++h)
+            fs[h] = make_float2((fl >> (2 * h)) & 1u ? kc.sup2 : 0.f, (fl >> (2 * h + 1)) & 1u ? kc.sup2 : 0.f);
+        auto steps = [&](auto allf) {
+            constexpr bool ALLF = decltype(allf)::value;
+            uint32_t at = list + 4u * lane;
+            const uint32_t end = at + 4u * n;
+#pragma unroll 1
+            for (; at != end; at += 128u) {
+                const int32_t t = lds_i32(at);
+                const bool fj = cand_f(t);
+                const CandJ j = load_cand(kc, cand_a(t), cand_b(t), fj);
+#pragma unroll
+                for (int h = 0; h < P; ++h) {
+                    const unsigned m = pair_terms_pack<ALLF, DFS, !STG>(kc, pi[h], nx[h], ny[h], nz[h], j, fs[h], fj,
+                                                                        acc[h]);
+                    if (DFS && !fj)
+                        nbits |= (m & 3u) << (2 * h);
+                    if (STAT) {
+                        float2 dx, dy, dz;
+                        const float2 r2 = dist2_pack(j.x, j.y, j.z, nx[h], ny[h], nz[h], dx, dy, dz);
+                        nn[2 * h] += r2.x < kc.sup2;
+                        nn[2 * h + 1] += r2.y < kc.sup2;
+                        np[2 * h] += m & 1u;
+                        np[2 * h + 1] += (m >> 1) & 1u;
+                        const bool f0 = (fl >> (2 * h)) & 1u, f1 = (fl >> (2 * h + 1)) & 1u;
+                        const bool v0 = 2 * h < nreal, v1 = 2 * h + 1 < nreal;  // a repeated particle is not counted
+                        lc[0] += (v0 && f0 && fj && (m & 1u)) + (v1 && f1 && fj && (m & 2u));
+                        lc[1] += (v0 && (m & 4u)) + (v1 && (m & 8u));
+                    }
+                }
+            }
+        };
+        if (fl == kAll)
+            steps(std::true_type{});
+        else
+            steps(std::false_type{});
+    };
+
+    // Candidate sweep: two windows at a time, 16 lanes each.
+    int cnt = 0;
+    auto drain = [&]() {  // the full batches of the list; the rest moves to its front
+        __syncwarp();
+        const int full = cnt & ~31;
+        evaluate(full);
+        __syncwarp();
+        const int32_t rest = lds_i32(list + 4u * (full + lane));
+        __syncwarp();
+        sts_i32(list + 4u * lane, rest);
+        cnt -= full;
+        __syncwarp();
+    };
+    constexpr int kChunk = (kList - 96) / 32;  // steps between the checks for room
+    for (int w0 = 0; w0 < nwin; w0 += 2) {
+        const int2 w = lds_i2(win + 8u * (w0 + (lane >> 4)));
+        const int32_t last = w.y - 1;
+        int32_t t = w.x + (lane & 15);
+        int steps = __reduce_max_sync(0xffffffffu, (unsigned)(w.y - w.x + 15) >> 4);
+        while (steps > 0) {
+            const int n = min(steps, kChunk);
+            steps -= n;
+            // room for these steps and for the padding of the last batch
+            if (cnt + 32 * n > kList - 32)
+                drain();
+#pragma unroll 1
+            for (int k = 0; k < n; ++k, t += 16) {
+                const int32_t tc = min(t, last);
+                const float4 a = cand_a(tc);
+                float near = 3.0e38f;
+#pragma unroll
+                for (int h = 0; h < P; ++h) {
+                    float2 dx, dy, dz;
+                    const float2 r2 = dist2_pack(a.x, a.y, a.z, nx[h], ny[h], nz[h], dx, dy, dz);
+                    near = fminf(near, fminf(r2.x, r2.y));
+                }
+                bool take = near < kc.sup2 && t <= last;
+                // clusters of boundary particles interact with fluid only
+                if (!STAT && fl == 0u)
+                    take = take && cand_f(tc);
+                const unsigned m = __ballot_sync(0xffffffffu, take);
+                const int at = cnt + __popc(m & lt);
+                if (take && SPH_BOUNDS_OK(at < kList && (!STG || (t >= 0 && t < kStage)), &b.misc[2]))
+                    sts_i32(list + 4u * at, t);
+                cnt += __popc(m);
+            }
+        }
+    }
+    __syncwarp();
+    if (SPH_BOUNDS_OK(cnt + lane < kList, &b.misc[2]))
+        sts_i32(list + 4u * (cnt + lane), dummy);  // pads the last batch
+    __syncwarp();
+    evaluate((cnt + 31) & ~31);
+
+    // totals and write-out
+    constexpr int K = 4 * G;
+    float v[K], e[K];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        const PackAcc &A = acc[g / 2];
+        v[4 * g + 0] = g & 1 ? A.drho.y : A.drho.x;
+        v[4 * g + 1] = g & 1 ? A.ax.y : A.ax.x;
+        v[4 * g + 2] = g & 1 ? A.ay.y : A.ay.x;
+        v[4 * g + 3] = g & 1 ? A.az.y : A.az.x;
+    }
+    const int idx = warp_split_totals<K, COMP>(v, e, lane);
+    const int gsel = idx >> 2, c = idx & 3;
+    float sum = v[0], err = COMP ? e[0] : 0.f;
     if (DFS) {
-        // the delta sums: a TwoSum butterfly per particle; the boundary-neighbour
-        // flags: an OR over the lanes
+        // the delta term only with a fluid-only support
         const unsigned nball = __reduce_or_sync(0xffffffffu, nbits);
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            float dv = acc[g].dd, de = 0.f;
+            float dv = g & 1 ? acc[g / 2].dd.y : acc[g / 2].dd.x, de = 0.f;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 const float recv = __shfl_xor_sync(0xffffffffu, dv, o);
@@ -310,89 +734,139 @@ __device__ __forceinline__ void combine_group(PairSmem &S, const LaneAcc (&acc)[
                 two_sum(dv, ee, recv);
                 de = ee;
             }
-            if (lane == 0 && valid[g]) {
-                float *D = S.dd[slot[g]];
-                two_sum(D[0], D[1], dv + de);
-                S.nb[slot[g]] |= (nball >> g) & 1u;
+            if (gsel == g && c == 0 && !((nball >> g) & 1u)) {
+                two_sum(sum, err, dv);
+                err += de;
             }
         }
     }
-    if (lane == 0) {
-#pragma unroll
-        for (int g = 0; g < G; ++g)
-            if (valid[g]) {
-                float *A = S.acc[slot[g]];
-                A[4] = fmaxf(A[4], mu[g]);
-                S.nn[slot[g]] += nsum[g];
-                S.np[slot[g]] += npair[g];
-            }
+    if ((lane & (32 / K - 1)) == 0 && gsel < nreal) {
+        float val = kc.mkF * (sum + err);
+        if (c == 3 && ((fl >> gsel) & 1u))
+            val -= I.gf;
+        reinterpret_cast<float *>(b.deriv)[4 * (size_t)(s0 + gsel) + ((c + 3) & 3)] = val;  // (a, D rho)
     }
+    float mu = 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        // non-negative floats order like their bits
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(g & 1 ? acc[g / 2].mu.y : acc[g / 2].mu.x));
+        mu = lane == g ? __uint_as_float(m) : mu;
+    }
+    if (lane < nreal)
+        reinterpret_cast<float *>(b.mumax)[s0 + lane] = I.hf * mu;
+    if (STAT) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int a = warp_sum(nn[g]), p = warp_sum(np[g]);
+            if (lane == 0 && g < nreal) {
+                // the particle itself is a hit; it is evaluated unless it is a boundary particle
+                b.nneigh[s0 + g] = a - 1;
+                b.npair[s0 + g] = p - (int)((fl >> g) & 1u);
+                b.ncand[s0 + g] = T.total;
+            }
+        }
+    }
+    __syncwarp();
 }
 
-// The pair pass of one CTA: pulls home cells from the work queue b.misc[3]
-// until it is exhausted.  dyn: the dynamic shared memory (staging buffers and
-// candidate lists), S: the CTA's bookkeeping.
-template <int NW, int G, bool COMP, bool CNT, bool DFS>
-__device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kdiv, int max_stage, unsigned char *dyn,
-                                                PairSmem &S)
+// The path of the rare tiles, kept out of line so that it costs the others no
+// registers.
+template <int NW, int G, bool COMP, bool STAT, bool DFS>
+__device__ __noinline__ void pair_cluster_global(const Bufs &b, const Inst &I, const TileGeo &T, int kdiv, int q,
+                                                 uint32_t list, int lane, PairSmem &S, unsigned (&lc)[2],
+                                                 unsigned long long &wc_cand)
 {
-    float4 *stA = reinterpret_cast<float4 *>(dyn);
-    float4 *stB = stA + max_stage;
-    uint8_t *stF = reinterpret_cast<uint8_t *>(stB + max_stage);
-    constexpr int LC = kList;
-    // interacting-candidate lists, one per (warp, particle slot), after the staged data
-    uint16_t *lists = reinterpret_cast<uint16_t *>(dyn + ((size_t)max_stage * (2 * sizeof(float4) + 1) + 15) / 16 * 16);
+    pair_cluster<NW, G, COMP, STAT, DFS, false>(b, I, pair_const(I), T, kdiv, q, 0u, list, lane, S, lc, wc_cand);
+}
 
-    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
-    const unsigned lt = (1u << lane) - 1u;
+// The pair pass of one CTA: pulls tiles from the work queue b.misc[3] until it
+// is exhausted.  dyn: the dynamic shared memory, S: the CTA's bookkeeping.
+template <int NW, int G, bool COMP, bool STAT, bool DFS>
+__device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kdiv, unsigned char *dyn, PairSmem &S)
+{
+    float4 *stA = reinterpret_cast<float4 *>(dyn), *stB = reinterpret_cast<float4 *>(dyn + kOffB);
+    uint8_t *stF = dyn + kOffF;
+    const int tid = threadIdx.x, lane = keep(tid & 31), wib = keep(tid >> 5);
+    const uint32_t st = keep(static_cast<uint32_t>(__cvta_generic_to_shared(dyn)));
+    const uint32_t list = keep(st + kOffWarp + wib * kWarpBytes);  // this warp's list and windows
     const float4 *gA = reinterpret_cast<const float4 *>(b.sA);
     const float4 *gB = reinterpret_cast<const float4 *>(b.sB);
-    float4 *gD = reinterpret_cast<float4 *>(b.deriv);
-    float *gM = reinterpret_cast<float *>(b.mumax);
-    const int32_t n_active = b.misc[1];
-    uint32_t lc_ff = 0, lc_visc = 0;  // evaluated fluid-fluid and approaching pairs of this lane
-    unsigned long long wc_cand = 0;   // windowed candidates tested by this warp
+    const int32_t n_tiles = b.misc[4];
+    unsigned lc[2] = {0u, 0u};
+    unsigned long long wc_cand = 0;
+    const int side = 2 * kdiv + 1;
+    const int row0 = ((lane % side - kdiv) & 0xff) | ((lane / side - kdiv) << 8);
+    const int row1 = (((lane + 32) % side - kdiv) & 0xff) | (((lane + 32) / side - kdiv) << 8);
     if (tid == 0) {
         S.st_ff = 0ull;
         S.st_visc = 0ull;
         S.st_cand = 0ull;
+        stA[kStage] = make_float4(1e15f, 1e15f, 1e15f, 0.f);  // the dummy: beyond 2h of everything
+        stB[kStage] = make_float4(0.f, 0.f, 0.f, 0.f);
+        stF[kStage] = T_FLUID;
     }
 
     for (;;) {
-        if (tid == 0)
-            S.item = atomicAdd(&b.misc[3], 1);
-        __syncthreads();
-        const int32_t item = S.item;
-        if (item >= n_active)
+        if (tid == 0) {
+            const int32_t item = atomicAdd(&b.misc[3], 1);
+            S.item = item < n_tiles ? b.tiles[item] : -1;
+        }
+        __syncthreads();  // and every warp is done with the previous tile
+        const int32_t tile = S.item;
+        if (tile < 0)
             break;
-        const int32_t c = b.active[item];
-        const Inst &I = b.inst[inst_of_cell(b.inst, ninst, c)];
+        const Inst &I = b.inst[inst_of_tile(b.inst, ninst, tile)];
         const PairConst kc = pair_const(I);
-        int cx, cy, cz;
-        decompose(I, c, cx, cy, cz);
-        const int x0 = max(cx - kdiv, 0), x1 = min(cx + kdiv, I.n[0] - 1);
-        const int32_t h0 = b.cell_start[c], h1 = b.cell_start[c + 1];
-        // Rows of the neighbourhood: slot r = (dz + k) side + (dy + k).  One
-        // thread per (row, x-boundary) loads the cell starts; warp 0 turns the
-        // row lengths into offsets of the flattened candidate list.
-        const int side = 2 * kdiv + 1, nrow = side * side, nb = x1 - x0 + 2;
-        for (int t = tid; t < nrow * nb; t += blockDim.x) {
-            const int r = t / nb, m = t - r * nb;
-            const int z = cz + r / side - kdiv, y = cy + r % side - kdiv;
-            int32_t v = -1;
-            if (z >= 0 && z < I.n[2] && y >= 0 && y < I.n[1])
-                v = b.cell_start[I.cell_base + (z * I.n[1] + y) * I.n[0] + x0 + m];
-            S.row[r].bnd[m] = v;
+        TileGeo T;
+        T.row0 = row0;
+        T.row1 = row1;
+        {
+            const int32_t lt = tile - I.tile_base;
+            const int32_t q = lt / I.ntile[0];
+            T.t0[0] = (lt - q * I.ntile[0]) * I.tdim[0];
+            T.t0[2] = q / I.ntile[1];
+            T.t0[1] = (q - T.t0[2] * I.ntile[1]) * I.tdim[1];
+            T.t0[2] *= I.tdim[2];
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            T.cen[a] = T.t0[a] + I.tdim[a] / 2;
+        T.nry = I.tdim[1] + 2 * kdiv;
+        T.dy0 = (float)(T.cen[1] * (I.cs - I.oc));
+        T.dz0 = (float)(T.cen[2] * (I.cs - I.oc));
+        const int nrow = T.nry * (I.tdim[2] + 2 * kdiv), nh = I.tdim[1] * I.tdim[2];
+        const int x0 = max(T.t0[0] - kdiv, 0), x1 = min(T.t0[0] + I.tdim[0] + kdiv, I.n[0]);
+        // the staged rows (one thread per row) and the tile's own runs of them
+        for (int u = tid; u < nrow + nh; u += blockDim.x) {
+            const bool home = u >= nrow;
+            const int r = home ? u - nrow : u, ny = home ? I.tdim[1] : T.nry, k = home ? 0 : kdiv;
+            const int z = T.t0[2] + r / ny - k, y = T.t0[1] + r % ny - k;
+            int32_t a = 0, n = 0;
+            if (z >= 0 && z < I.n[2] && y >= 0 && y < I.n[1]) {
+                const int32_t row = I.cell_base + (z * I.n[1] + y) * I.n[0];
+                a = b.cell_start[row + (home ? T.t0[0] : x0)];
+                n = b.cell_start[row + (home ? min(T.t0[0] + I.tdim[0], I.n[0]) : x1)] - a;
+            }
+            if (home) {
+                S.hst[r] = a;
+                S.hlen[r] = n;
+                S.hyz[r] = (r % ny) | ((r / ny) << 16);
+            } else {
+                S.gs[r] = a;
+                S.pre[r + 1] = n;
+            }
+        }
+        if (tid == 0) {
+            S.next = 0;
+            S.wild = 0;
         }
         __syncthreads();
         if (wib == 0) {
             int carry = 0;
             for (int r0 = 0; r0 < nrow; r0 += 32) {
                 const int r = r0 + lane;
-                int len = 0;
-                if (r < nrow && S.row[r].bnd[0] >= 0)
-                    len = S.row[r].bnd[nb - 1] - S.row[r].bnd[0];
-                int x = len;
+                int x = r < nrow ? S.pre[r + 1] : 0;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const int y = __shfl_up_sync(0xffffffffu, x, o);
@@ -400,328 +874,80 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
                         x += y;
                 }
                 if (r < nrow)
-                    S.pre[r] = carry + x - len;
+                    S.pre[r + 1] = carry + x;
                 carry += __shfl_sync(0xffffffffu, x, 31);
             }
             if (lane == 0)
-                S.pre[nrow] = carry;
+                S.pre[0] = 0;
+        } else if (wib == 1) {
+            int x = lane < nh ? (S.hlen[lane] + G - 1) / G : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o)
+                    x += y;
+            }
+            if (lane < nh)
+                S.hpre[lane + 1] = x;
+            if (lane == 0)
+                S.hpre[0] = 0;
         }
         __syncthreads();
-        const int32_t total = S.pre[nrow];
-        // flattened index of the home cell's first particle (home row dy = dz = 0)
-        const int home_row = kdiv * side + kdiv;
-        const int32_t home_flat0 = S.pre[home_row] + (h0 - S.row[home_row].bnd[0]);
-
-        for (int32_t g0 = h0; g0 < h1; g0 += kMaxI) {
-            const int32_t g1 = min(h1, g0 + kMaxI);
-            __syncthreads();
-            for (int m = tid; m < (g1 - g0) * 9; m += blockDim.x)
-                (&S.acc[0][0])[m] = 0.f;
-            for (int m = tid; m < g1 - g0; m += blockDim.x) {
-                S.nn[m] = 0;
-                S.np[m] = 0;
-                S.dd[m][0] = 0.f;
-                S.dd[m][1] = 0.f;
-                S.nb[m] = 0;
-            }
-            for (int32_t f0 = 0; f0 < total; f0 += max_stage) {
-                const int32_t f1 = min(total, f0 + max_stage);
-                                __syncthreads();
-                // stage [f0, f1): one warp per row, lanes along the row
-                for (int r = wib; r < nrow; r += NW) {
-                    const int32_t p0 = S.pre[r], len = S.pre[r + 1] - p0;
-                    const int32_t l0 = max(f0 - p0, 0), l1 = min(f1 - p0, len);
-                    if (l0 >= l1)
+        T.total = S.pre[nrow];
+        const int nclus = S.hpre[nh];
+        const bool fits = T.total <= kStage;
+        if (fits) {
+            bool wild = false;
+            const float lim = 1e15f, dmin = -0.5f * kc.rho0;
+            for (int r = wib; r < nrow; r += NW) {
+                const int32_t p0 = S.pre[r], len = S.pre[r + 1] - p0, g0 = S.gs[r];
+                if (len == 0)
+                    continue;
+                const int zr = r / T.nry;
+                const int y = T.t0[1] + (r - zr * T.nry) - kdiv, z = T.t0[2] + zr - kdiv;
+                const float sy = (float)(y - T.cen[1]) * I.ocf, sz = (float)(z - T.cen[2]) * I.ocf;
+                const int32_t row = I.cell_base + (z * I.n[1] + y) * I.n[0] + T.cen[0];
+#pragma unroll 3
+                for (int32_t l = lane; l < len; l += 32) {
+                    const int32_t j = g0 + l;
+                    float4 a = gA[j];
+                    const float4 v = gB[j];
+                    const uint8_t f = b.sflag[j];
+                    a.x += (float)(b.scell[j] - row) * I.ocf;
+                    a.y += sy;
+                    a.z += sz;
+                    // a NaN or an infinity fails the comparison too
+                    wild = wild || !(fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + fabsf(v.w) + fabsf(a.w) < lim && a.w > dmin);
+                    const int32_t t = p0 + l;
+                    if (!SPH_BOUNDS_OK(t >= 0 && t < kStage, &b.misc[2]))
                         continue;
-                    const RowM &R = S.row[r];
-                    const float sy = (float)(r % side - kdiv) * kc.cs, sz = (float)(r / side - kdiv) * kc.cs;
-                    for (int32_t l = l0 + lane; l < l1; l += 32) {
-                        const int32_t j = R.bnd[0] + l;
-                        int xc = x0;
-                        for (int m = 1; m < nb - 1; ++m)
-                            xc += j >= R.bnd[m];
-                        float4 a = gA[j];
-                        a.x += (float)(xc - cx) * kc.cs;
-                        a.y += sy;
-                        a.z += sz;
-                        const int32_t t = p0 + l - f0;
-                        if (!SPH_BOUNDS_OK(t >= 0 && t < max_stage, &b.misc[2]))
-                            continue;
-                        stA[t] = a;
-                        stB[t] = gB[j];
-                        stF[t] = b.sflag[j];
-                    }
-                }
-                __syncthreads();
-                // Each warp takes G particles of the home cell.  Phase 1 sweeps the
-                // staged candidates once for all G particles and appends the
-                // interacting ones to one list per particle; phase 2 evaluates the
-                // pair terms 32 at a time.  A list short of room is drained early.
-                // Warps take G consecutive home particles at a time; in a short
-                // last group the empty slots repeat the last particle and are
-                // swept but neither evaluated nor stored.
-                for (int32_t ib = g0 + G * wib; ib < g1; ib += G * NW) {
-                    const int32_t ie = min(ib + G, g1);
-                    // Only the positions and type flags of the G particles stay in
-                    // registers through the sweep; the rest of a particle's state is
-                    // reloaded when its list is evaluated.
-                    float px[G], py[G], pz[G];
-                    LaneAcc acc[G];
-                    int cnt[G], nn[G], np[G];
-                    unsigned fl = 0;  // bit g: particle g is fluid
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        const int32_t ii = min(ib + g, ie - 1);
-                        const float4 Ai = gA[ii];
-                        px[g] = Ai.x;
-                        py[g] = Ai.y;
-                        pz[g] = Ai.z;
-                        fl |= (b.sflag[ii] == T_FLUID ? 1u : 0u) << g;
-                        acc[g] = LaneAcc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                        cnt[g] = 0;
-                        nn[g] = 0;
-                        np[g] = 0;
-                    }
-                    const bool all_fluid = fl == (1u << G) - 1u;
-                    unsigned nbits = 0;  // DFS: bit g set when a listed neighbour of particle g is a boundary particle
-                    SweepPos<G> sp;
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        float2 &vx = sp.nx[g / 2], &vy = sp.ny[g / 2], &vz = sp.nz[g / 2];
-                        if (g % 2 == 0) {
-                            vx.x = -px[g];
-                            vy.x = -py[g];
-                            vz.x = -pz[g];
-                        } else {
-                            vx.y = -px[g];
-                            vy.y = -py[g];
-                            vz.y = -pz[g];
-                        }
-                    }
-                    uint16_t *const wl0 = lists + wib * G * LC;
-                    auto drain = [&](int g, int upto) {
-                        // evaluate list entries [0, upto) of particle g, upto a multiple of 32 or cnt
-                        const int32_t ii = min(ib + g, ie - 1);
-                        const PartI P = load_part(kc, gA[ii], gB[ii], (fl >> g) & 1u);
-                        const uint16_t *lg = wl0 + g * LC;
-                        int k = 0;
-                        if (!CNT) {
-                            // two full batches at a time: two independent chains per lane
-                            for (; k + 64 <= upto; k += 64) {
-                                const int t0 = lg[k + lane], t1 = lg[k + 32 + lane];
-                                LaneAcc a1{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                                const bool f0 = stF[t0] == T_FLUID, f1 = stF[t1] == T_FLUID;
-                                pair_term_f<DFS>(kc, P, stA[t0], stB[t0], P.fluid && f0, acc[g]);
-                                pair_term_f<DFS>(kc, P, stA[t1], stB[t1], P.fluid && f1, a1);
-                                if (DFS) {
-                                    nbits |= (f0 && f1 ? 0u : 1u) << g;
-                                    acc[g].dd += a1.dd;
-                                }
-                                acc[g].drho += a1.drho;
-                                acc[g].ax += a1.ax;
-                                acc[g].ay += a1.ay;
-                                acc[g].az += a1.az;
-                                acc[g].mumax = fmaxf(acc[g].mumax, a1.mumax);
-                            }
-                        }
-                        for (; k < upto; k += 32) {
-                            if (lane < upto - k) {
-                                const int t = lg[k + lane];
-                                const bool fj = stF[t] == T_FLUID;
-                                const int f = pair_term_f<DFS>(kc, P, stA[t], stB[t], P.fluid && fj, acc[g]);
-                                if (DFS)
-                                    nbits |= (fj ? 0u : 1u) << g;
-                                if (CNT && ib + g < ie) {  // a repeated particle is not counted
-                                    lc_ff += f & 1;
-                                    lc_visc += f >> 1;
-                                }
-                            }
-                        }
-                    };
-                    // Exact x-windows per row: a candidate j of row r can lie within 2h
-                    // of i only if |x_j - x_i| <= w_r = sqrt((2h)^2 - d_r^2), d_r the
-                    // distance from i to the row's y-z cross-section.  Cells are sorted
-                    // by x, so each row is sorted by x and each window is a contiguous
-                    // range, found by binary search (one lane per row); the windows of
-                    // the G particles are merged.
-                    int wlo[2] = {0, 0}, whi[2] = {0, 0};
-#pragma unroll
-                    for (int pass = 0; pass < 2; ++pass) {
-                        const int r = pass * 32 + lane;
-                        if (pass * 32 < nrow && r < nrow) {
-                            const int32_t ra = max(S.pre[r], f0) - f0, rb = min(S.pre[r + 1], f1) - f0;
-                            if (ra < rb) {
-                                const float ry = (float)(r % side - kdiv), rz = (float)(r / side - kdiv);
-                                float xl = 3.0e38f, xh = -3.0e38f;
-#pragma unroll
-                                for (int g = 0; g < G; ++g) {
-                                    float dy = ry > 0.f ? ry * kc.cs - py[g] : (ry < 0.f ? py[g] - (ry + 1.f) * kc.cs : 0.f);
-                                    float dz = rz > 0.f ? rz * kc.cs - pz[g] : (rz < 0.f ? pz[g] - (rz + 1.f) * kc.cs : 0.f);
-                                    dy = fmaxf(dy, 0.f);
-                                    dz = fmaxf(dz, 0.f);
-                                    const float rem = kc.sup2 - dy * dy - dz * dz;
-                                    if (rem > 0.f) {
-                                        const float w = sqrtf(rem) * 1.0001f + 1e-6f * kc.cs;
-                                        xl = fminf(xl, px[g] - w);
-                                        xh = fmaxf(xh, px[g] + w);
-                                    }
-                                }
-                                if (xl <= xh) {
-                                    int a0 = ra, a1 = rb;
-                                    while (a0 < a1) {
-                                        const int m = (a0 + a1) >> 1;
-                                        if (stA[m].x < xl)
-                                            a0 = m + 1;
-                                        else
-                                            a1 = m;
-                                    }
-                                    wlo[pass] = a0;
-                                    a1 = rb;
-                                    while (a0 < a1) {
-                                        const int m = (a0 + a1) >> 1;
-                                        if (stA[m].x <= xh)
-                                            a0 = m + 1;
-                                        else
-                                            a1 = m;
-                                    }
-                                    whi[pass] = a0;
-                                }
-                            }
-                        }
-                    }
-                    if (CNT) {
-                        const int wsum = warp_sum((whi[0] - wlo[0]) + (whi[1] - wlo[1]));
-                        if (lane == 0)
-                            wc_cand += (unsigned long long)wsum;
-                    }
-                    // Drain the full 32-entry batches of every list and keep the rest.
-                    auto flush = [&]() {
-                        __syncwarp();
-#pragma unroll
-                        for (int g = 0; g < G; ++g) {
-                            const int done = cnt[g] & ~31;
-                            if (ib + g < ie)
-                                drain(g, done);
-                            __syncwarp();
-                            if (lane < cnt[g] - done)
-                                if (SPH_BOUNDS_OK(done + lane < LC, &b.misc[2]))
-                                    wl0[g * LC + lane] = wl0[g * LC + done + lane];
-                            np[g] += done;
-                            cnt[g] -= done;
-                            __syncwarp();
-                        }
-                    };
-                    // One 32-candidate step: G tests per candidate, ballot compaction.
-                    auto sweep = [&](int32_t base, int32_t lo, int32_t hi) {
-                        const int32_t t = base + lane;
-                        const bool valid = t < hi;
-                        float4 a = stA[valid ? t : lo];
-                        a.x = valid ? a.x : 1.0e30f;  // a lane past the window misses every test
-                        bool hits[G];
-                        hit_tests<G>(sp, a, kc.sup2, hits);
-                        if (all_fluid) {
-#pragma unroll
-                            for (int g = 0; g < G; ++g) {
-                                const bool take = hits[g];
-                                const unsigned m = __ballot_sync(0xffffffffu, take);
-                                if (take && SPH_BOUNDS_OK(cnt[g] + __popc(m & lt) < LC && t < max_stage, &b.misc[2]))
-                                    wl0[g * LC + cnt[g] + __popc(m & lt)] = (uint16_t)t;
-                                cnt[g] += __popc(m);
-                            }
-                        } else {
-                            const bool fj = stF[valid ? t : lo] == T_FLUID;
-#pragma unroll
-                            for (int g = 0; g < G; ++g) {
-                                const bool hit = hits[g];
-                                const bool take = hit && (((fl >> g) & 1u) || fj);
-                                nn[g] += __popc(__ballot_sync(0xffffffffu, hit));
-                                const unsigned m = __ballot_sync(0xffffffffu, take);
-                                if (take && SPH_BOUNDS_OK(cnt[g] + __popc(m & lt) < LC && t < max_stage, &b.misc[2]))
-                                    wl0[g * LC + cnt[g] + __popc(m & lt)] = (uint16_t)t;
-                                cnt[g] += __popc(m);
-                            }
-                        }
-                    };
-                    for (int r = 0; r < nrow; ++r) {
-                        const int lo = __shfl_sync(0xffffffffu, r < 32 ? wlo[0] : wlo[1], r & 31);
-                        const int hi = __shfl_sync(0xffffffffu, r < 32 ? whi[0] : whi[1], r & 31);
-                        // Room for the whole row window in every list is made before the
-                        // row; only a window longer than LC - 32 is checked step by step.
-                        bool need = false;
-#pragma unroll
-                        for (int g = 0; g < G; ++g)
-                            need = need || cnt[g] + (hi - lo) > LC;
-                        if (need)
-                            flush();
-                        if (hi - lo <= LC - 32) {
-                            for (int32_t base = lo; base < hi; base += 32)
-                                sweep(base, lo, hi);
-                        } else {
-                            for (int32_t base = lo; base < hi; base += 32) {
-                                sweep(base, lo, hi);
-                                bool full = false;
-#pragma unroll
-                                for (int g = 0; g < G; ++g)
-                                    full = full || cnt[g] > LC - 32;
-                                if (full)
-                                    flush();
-                            }
-                        }
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        if (ib + g < ie)
-                            drain(g, cnt[g]);
-                        np[g] += cnt[g];
-                    }
-                    {
-                        int32_t slot[G];
-                        bool valid[G];
-                        int nsum[G], npair[G];
-#pragma unroll
-                        for (int g = 0; g < G; ++g) {
-                            const int32_t ii = ib + g;
-                            // the staged copy of i itself is a hit (and a zero term) in its chunk
-                            const int32_t self = home_flat0 + (ii - h0);
-                            const int selfc = (ii < ie && self >= f0 && self < f1) ? 1 : 0;
-                            slot[g] = ii - g0;
-                            valid[g] = ii < ie;
-                            // every hit of a fluid particle is evaluated, so nn = np there
-                            nsum[g] = (((fl >> g) & 1u) ? np[g] : nn[g]) - selfc;
-                            npair[g] = np[g] - selfc;
-                        }
-                        combine_group<G, COMP, DFS>(S, acc, slot, valid, nsum, npair, nbits);
-                    }
-                    __syncwarp();
+                    stA[t] = a;
+                    stB[t] = v;
+                    stF[t] = f;
                 }
             }
-            __syncthreads();
-            for (int32_t ii = g0 + tid; ii < g1; ii += blockDim.x) {
-                const float *A = S.acc[ii - g0];
-                float az = A[3] + A[8];
-                if (b.sflag[ii] == T_FLUID)
-                    az -= I.gf;
-                float drho = A[0] + A[5];
-                if (DFS && !S.nb[ii - g0]) {  // the delta term only with a fluid-only support
-                    float e = A[5];
-                    float sum = A[0];
-                    two_sum(sum, e, S.dd[ii - g0][0]);
-                    drho = sum + (e + S.dd[ii - g0][1]);
-                }
-                gD[ii] = make_float4(A[1] + A[6], A[2] + A[7], az, drho);
-                gM[ii] = I.hf * A[4];
-                b.nneigh[ii] = S.nn[ii - g0];
-                b.npair[ii] = S.np[ii - g0];
-                b.ncand[ii] = total;
-            }
+            if (wild)
+                S.wild = 1;
         }
         __syncthreads();
+        const bool staged = fits && !S.wild;
+        for (;;) {
+            int q = 0;
+            if (lane == 0)
+                q = atomicAdd(&S.next, 1);
+            q = __shfl_sync(0xffffffffu, q, 0);
+            if (q >= nclus)
+                break;
+            if (staged)
+                pair_cluster<NW, G, COMP, STAT, DFS, true>(b, I, kc, T, kdiv, q, st, list, lane, S, lc, wc_cand);
+            else
+                pair_cluster_global<NW, G, COMP, STAT, DFS>(b, I, T, kdiv, q, list, lane, S, lc, wc_cand);
+        }
     }
-    if (!CNT)
+    if (!STAT)
         return;
     // work counts: lanes -> warp -> CTA -> device
-    const uint32_t wff = (uint32_t)warp_sum((int)lc_ff), wvi = (uint32_t)warp_sum((int)lc_visc);
+    const unsigned wff = (unsigned)warp_sum((int)lc[0]), wvi = (unsigned)warp_sum((int)lc[1]);
     if (lane == 0) {
         atomicAdd(&S.st_ff, (unsigned long long)wff);
         atomicAdd(&S.st_visc, (unsigned long long)wvi);

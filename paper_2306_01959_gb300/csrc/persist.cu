@@ -15,7 +15,7 @@
 // out at its next barrier, so the launch always ends.  A cooperative launch
 // guarantees that all CTAs are resident at once.
 #include "cells.cuh"
-#include "pair_mixed.cuh"
+#include "pair_wide.cuh"
 #include "step.cuh"
 
 namespace sph {
@@ -52,24 +52,26 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &target, lo
     return *s_ok != 0;
 }
 
-template <bool DFS>
+template <bool TILED, bool DFS>
 __global__ void __launch_bounds__(kPersistWarps * 32, 2)
-    k_persistent_steps(Bufs b, int ninst, int nsteps, int ns, int kdiv, int max_stage, int64_t N, uint32_t C,
-                       int ntiles, long long spin_limit)
+    k_persistent_steps(Bufs b, int ninst, int nsteps, int ns, int kdiv, int max_stage, int64_t N, uint32_t C, int ntiles,
+                       long long spin_limit)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ PairSmem S;
+    __shared__ typename std::conditional<TILED, PairSmem, WideSmem>::type S;
     __shared__ int s_ok;
     unsigned target = 0;
     const int tid = threadIdx.x;
     const int gthread = blockIdx.x * blockDim.x + tid, gstride = gridDim.x * blockDim.x;
-    const int gwarp = gthread >> 5, nwarps = gstride >> 5;
     int32_t *status = &b.misc[2];
 #define SPH_BARRIER()                                                       \
     if (!grid_barrier(b.bar, target, spin_limit, status, &s_ok))            \
         return;
     for (int step = 0; step < nsteps; ++step) {
-        pair_mixed_body<kPersistWarps, kPersistGroup, true, false, DFS>(b, ninst, kdiv, max_stage, dyn, S);
+        if constexpr (TILED)
+            pair_mixed_body<kPersistWarps, kPersistGroup, true, false, DFS>(b, ninst, kdiv, dyn, S);
+        else
+            pair_wide_body<kPersistWarps, kPersistGroup, true, false, DFS>(b, ninst, kdiv, max_stage, dyn, S);
         SPH_BARRIER();
         dt_reduce_part<SPH_MIXED>(b, ninst, blockIdx.x, gridDim.x);
         SPH_BARRIER();
@@ -82,40 +84,39 @@ __global__ void __launch_bounds__(kPersistWarps * 32, 2)
         integrate_range<SPH_MIXED>(b, N, C, gthread, gstride);
         SPH_BARRIER();
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x)
-            scan_reduce_tile(b.count, b.scan_blocks, C, t);
+            scan_reduce_tile<kPersistWarps * 32>(b.count, b.scan_blocks, C, t);
         SPH_BARRIER();
         if (blockIdx.x == 0)
             scan_blocks_block(b.scan_blocks, ntiles);
         SPH_BARRIER();
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x)
-            scan_final_tile(b.count, b.scan_blocks, b.cell_start, b.active, b.misc, C, t);
+            scan_final_tile<kPersistWarps * 32>(b.count, b.scan_blocks, b.cell_start, b.active, b.misc, C, t);
         SPH_BARRIER();
-        scatter_range(b.key, b.count, b.cell_start, b.ptmp, b.misc, N, gthread, gstride);
+        scatter_phase<SPH_MIXED>(b, N, gthread, gstride);
         SPH_BARRIER();
-        // the sort keys use the pair pass's staging memory, idle in this phase
-        sort_reorder_warps<SPH_MIXED>(b, ninst, reinterpret_cast<uint64_t *>(dyn) + (tid >> 5) * kSortCap, gwarp,
-                                      nwarps);
+        tile_list_range(b, ninst, gthread, gstride);
+        sort_reorder_range<SPH_MIXED>(b, ninst, gthread, gstride);
         SPH_BARRIER();
     }
 #undef SPH_BARRIER
 }
 
-template <bool DFS>
+template <bool TILED, bool DFS>
 cudaError_t launch_typed(const Bufs &b, int ninst, int nsteps, int ns, int cell_div, int64_t N, int32_t C,
                          long long spin_limit, cudaStream_t st)
 {
-    const int max_stage = mixed_max_stage(cell_div);
-    const size_t dyn = mixed_dyn_smem(max_stage, kPersistWarps, kPersistGroup);
+    int max_stage = wide_max_stage(cell_div);
+    const size_t dyn = TILED ? mixed_dyn_smem(kPersistWarps) : wide_dyn_smem(max_stage, kPersistWarps, kPersistGroup);
     static size_t dyn_set = 0;
     cudaError_t e;
     if (dyn > dyn_set) {
-        e = cudaFuncSetAttribute(k_persistent_steps<DFS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        e = cudaFuncSetAttribute(k_persistent_steps<TILED, DFS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
         if (e != cudaSuccess)
             return e;
         dyn_set = dyn;
     }
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persistent_steps<DFS>, kPersistWarps * 32, dyn);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persistent_steps<TILED, DFS>, kPersistWarps * 32, dyn);
     if (e != cudaSuccess)
         return e;
     if (per_sm < 1)
@@ -123,24 +124,26 @@ cudaError_t launch_typed(const Bufs &b, int ninst, int nsteps, int ns, int cell_
     const int grid = per_sm * sm_count();
     int ntiles = (int)((C + 1 + kScanTile - 1) / kScanTile);
     uint32_t Cu = (uint32_t)C;
-    void *args[] = {(void *)&b, &ninst, &nsteps, &ns, &cell_div, (void *)&max_stage, &N, &Cu, &ntiles, &spin_limit};
+    void *args[] = {(void *)&b, &ninst, &nsteps, &ns, &cell_div, &max_stage, &N, &Cu, &ntiles, &spin_limit};
     e = cudaMemsetAsync(b.bar, 0, sizeof(unsigned), st);
     if (e != cudaSuccess)
         return e;
     e = cudaMemsetAsync(b.misc + 3, 0, sizeof(int32_t), st);
     if (e != cudaSuccess)
         return e;
-    return cudaLaunchCooperativeKernel((const void *)k_persistent_steps<DFS>, grid, kPersistWarps * 32, args, dyn, st);
+    return cudaLaunchCooperativeKernel((const void *)k_persistent_steps<TILED, DFS>, grid, kPersistWarps * 32, args, dyn, st);
 }
 
 }  // namespace
 
-cudaError_t launch_persistent_steps(const Bufs &b, int32_t ninst, int32_t nsteps, int32_t ns, int32_t cell_div,
-                                    int32_t delta_mode, int64_t N, int32_t C, long long spin_limit, cudaStream_t st)
+cudaError_t launch_persistent_steps(const Bufs &b, bool tiled, int32_t ninst, int32_t nsteps, int32_t ns,
+                                    int32_t cell_div, int32_t delta_mode, int64_t N, int32_t C, long long spin_limit,
+                                    cudaStream_t st)
 {
-    if (delta_mode == SPH_DELTA_FULL_SUPPORT)
-        return launch_typed<true>(b, ninst, nsteps, ns, cell_div, N, C, spin_limit, st);
-    return launch_typed<false>(b, ninst, nsteps, ns, cell_div, N, C, spin_limit, st);
+    const bool dfs = delta_mode == SPH_DELTA_FULL_SUPPORT;
+    auto launch = tiled ? (dfs ? launch_typed<true, true> : launch_typed<true, false>)
+                        : (dfs ? launch_typed<false, true> : launch_typed<false, false>);
+    return launch(b, ninst, nsteps, ns, cell_div, N, C, spin_limit, st);
 }
 
 }  // namespace sph

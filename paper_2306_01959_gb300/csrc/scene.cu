@@ -23,8 +23,8 @@ static int64_t nint(double x) { return (int64_t)std::floor(x + 0.5); }
 
 int effective_cell_div(const sph_params &p)
 {
-    // automatic: cells of size 2h for the mixed form (its pair kernel stages
-    // whole 27-cell neighbourhoods), cells of size h for the FP64 form
+    // automatic: cells of size 2h for the mixed form (what callers see; its tiled
+    // pair pass divides them again), cells of size h for the FP64 form
     if (p.cell_div > 0)
         return p.cell_div;
     return p.precision == SPH_MIXED ? 1 : 2;
@@ -107,7 +107,7 @@ int validate_instance(const sph_instance &in, const sph_params &p, std::string &
     return SPH_OK;
 }
 
-void fill_inst(HostInst &hi, const sph_params &p)
+void fill_inst(HostInst &hi, const sph_params &p, int fine, bool tiled)
 {
     const sph_instance &in = hi.d;
     double dp = in.dp;
@@ -133,6 +133,19 @@ void fill_inst(HostInst &hi, const sph_params &p)
         d.lo[a] = -Ld;
         d.n[a] = (int32_t)std::ceil((hi3[a] - d.lo[a]) / d.cs);
     }
+    // a finer grid of the same box: halving the spacing (fine = 2) is exact, so a
+    // particle's coarse cell is its fine cell divided by two
+    d.cs /= fine;
+    d.inv_cs *= fine;
+    for (int a = 0; a < 3; ++a)
+        d.n[a] *= fine;
+    d.oc = d.cs;
+    if (tiled) {
+        int e;
+        const double f = std::frexp(d.cs, &e);
+        d.oc = std::ldexp(std::nearbyint(std::ldexp(f, 20)), e - 20);
+    }
+    d.ocf = (float)d.oc;
     d.ncells = d.n[0] * d.n[1] * d.n[2];
     d.h = in.h;
     d.c0 = in.c0;
@@ -192,6 +205,56 @@ void fill_inst(HostInst &hi, const sph_params &p)
     d.dfac = (float)(2.0 * d.delta * d.h * d.c0);
     d.gammaf = (float)d.gamma;
     d.gf = (float)d.g;
+}
+
+// The tiled pair pass stages a tile of at least (2h)^3 with the cells within 2h of
+// it: 6h each way.  On the particle lattice (the densest state of a weakly
+// compressible flow, at its worst alignment) that has to fit the staging buffer,
+// which it does for h < 7/3 dp; beyond, the neighbourhoods are staged in chunks by
+// the other kernel (pair_wide.cuh).  Neighbour lists keep to that one too: their
+// cells are wider than 2h.
+bool tiles_fit(const sph_instance &in, const sph_params &p)
+{
+    const double n = std::floor(6.0 * in.h / in.dp * (1.0 + 1e-9)) + 1.0;
+    return !(p.list_skin > 0) && n * n * n <= kStage;
+}
+
+// A larger tile stages fewer candidates per particle of its own (27 at (2h)^3, 18 at
+// twice that length); it has to fit the staging buffer like the smallest, and there
+// must be enough tiles to fill the GPU (2 CTAs on each of 152 SMs) four times over.
+int64_t fill_tiles(std::vector<HostInst> &inst, int k, int64_t n_total)
+{
+    int64_t base = 0;
+    for (HostInst &hi : inst) {
+        Inst &d = hi.dev;
+        const double c = d.cs / d.dp;  // cell size in particle spacings
+        int best[3] = {k, k, k};
+        double most = k * k * k * c * c * c;
+        for (int tz = k; tz <= 2 * k; tz += k)
+            for (int ty = tz; ty <= 2 * k; ty += k)
+                for (int tx = k; tx <= 4 * k; ++tx) {
+                    if (ty * tz > 16 || (ty + 2 * k) * (tz + 2 * k) > 96)
+                        continue;
+                    const double staged = (std::floor((tx + 2 * k) * c) + 1) * (std::floor((ty + 2 * k) * c) + 1) *
+                                          (std::floor((tz + 2 * k) * c) + 1);
+                    const double own = tx * ty * tz * c * c * c;
+                    if (staged <= kStage && own * 1216 <= (double)n_total && own > most * 1.01) {
+                        most = own;
+                        best[0] = tx;
+                        best[1] = ty;
+                        best[2] = tz;
+                    }
+                }
+        int64_t nt = 1;
+        for (int a = 0; a < 3; ++a) {
+            d.tdim[a] = best[a];
+            d.ntile[a] = (d.n[a] + best[a] - 1) / best[a];
+            nt *= d.ntile[a];
+        }
+        d.tile_base = (int32_t)base;
+        base += nt;
+    }
+    return base;
 }
 
 void build_scene(const HostInst &hi, const sph_params &p, double *r, double *rho, uint8_t *type)

@@ -208,6 +208,8 @@ __device__ __forceinline__ void integrate_range(const Bufs &b, int64_t N, uint32
         }
         if (in)
             c = (uint32_t)(I.cell_base + (cz * I.n[1] + cy) * I.n[0] + cx);
+        if (MODE == SPH_MIXED && in)
+            b.xof[id] = x_offset(I, p.x, cx);
         b.key[id] = c;
         atomicAdd(&b.count[c], 1u);
     }
