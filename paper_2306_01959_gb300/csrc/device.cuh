@@ -125,11 +125,13 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-__device__ __forceinline__ double warp_max(double v)
+// Maximum of non-negative doubles by their bit patterns, which order alike (the
+// integer units instead of the FP64 pipe).
+__device__ __forceinline__ long long warp_max_bits(long long v)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
-        v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+        v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 
@@ -138,9 +140,9 @@ __device__ __forceinline__ double warp_max(double v)
 // values and adds its partner's copies of them, the remaining levels add the
 // one value left, so K values cost K FP64 additions per lane (5 K for K
 // separate butterflies).  On return v[k] of lane 0 holds the total of value k
-// (other lanes: undefined).  The order of the additions is fixed.
+// (other lanes: undefined), times `scale`.  The order of the additions is fixed.
 template <int K>
-__device__ __forceinline__ void warp_totals(double (&v)[K])
+__device__ __forceinline__ void warp_totals(double (&v)[K], double scale = 1.0)
 {
     const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -158,7 +160,7 @@ __device__ __forceinline__ void warp_totals(double (&v)[K])
     for (int o = 16 / K; o > 0; o >>= 1)
         v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
     // lane (32 / K) k holds the total of value k
-    const double mine = v[0];
+    const double mine = scale * v[0];
 #pragma unroll
     for (int k = 0; k < K; ++k)
         v[k] = __shfl_sync(0xffffffffu, mine, k * (32 / K));

@@ -44,6 +44,8 @@ struct Inst {
     double h, c0, rho0, alpha, delta, gamma, g, cfl, mass, B, eta2, sup2, dt_min, ztop, dp;
     double kF;  // 105 / (16 pi h^5): grad_i W_ij = -kF (1 - q/2)^3 (r_i - r_j)
     double kW;  // 21 / (16 pi h^3)
+    // factors of the FP64 pair terms
+    double half_inv_h, kFm, dfac_d, nah;  // 0.5 / h, kF m, 2 delta h c0, -alpha h
     // spacing of the cell origins of the mixed form's FP32 offsets: cs rounded to
     // 20 mantissa bits, so that a shift by a few cells is exact in FP32 (with
     // neighbour lists: cs)

@@ -28,22 +28,50 @@ struct AccD {
     long long mumax_bits;
 };
 
-// Constants of an instance used by every pair, computed once per particle.
+// Constants of an instance used by every pair.
 struct PairConstD {
     double half_inv_h, kFm, dfac, nah, eta2;  // kFm = kF m, dfac = 2 delta h c0, nah = -alpha h
 };
 
 __device__ __forceinline__ PairConstD pair_const_d(const Inst &I)
 {
-    return PairConstD{0.5 / I.h, I.kF * I.mass, 2.0 * I.delta * I.h * I.c0, -I.alpha * I.h, I.eta2};
+    return PairConstD{I.half_inv_h, I.kFm, I.dfac_d, I.nah, I.eta2};
+}
+
+// The FP64 pipe of this GPU issues one warp operation every 64 cycles per
+// scheduler, so the pair term is priced in FP64 operations alone; the library's
+// reciprocal square root and correctly rounded reciprocals took about 10 and 8
+// of them each.  Both start here from the hardware's 20-bit approximation and
+// take one step of third order (Householder's method, from the series of
+// (1 - e)^-1 and (1 - e)^-1/2 in the residual e of the approximation): the
+// remaining error, e^3 < 2^-57, is below the rounding of the last operation.
+
+// 1 / a for a normal a (3 operations).
+__device__ __forceinline__ double rcp3(double a)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// sqrt(a) for a >= 0 (5 operations); 0 for 0: the approximation is taken at
+// no less than 2^-1000 (an integer maximum of the bit patterns).
+__device__ __forceinline__ double sqrt3(double a)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(__longlong_as_double(max(__double_as_longlong(a), 23LL << 52))));
+    const double s = a * y;
+    const double e = fma(-s, y, 1.0);
+    return fma(s * e, fma(0.375, e, 0.5), s);
 }
 
 // Contribution of neighbour j to particle i (Eqs. 3-7), in double.
 // Continuity uses the standard sign (u_i - u_j) . grad_i W_ij; the delta
 // term acts between fluid particles; the viscosity of Eq. 4 applies when
 // u_ij . r_ij < 0.  1/rho and c of both particles come precomputed, so a pair
-// costs one reciprocal square root and two correctly rounded reciprocals (mu,
-// and the viscosity's mean density when it applies).  m_j F = -kF m t^3 with
+// costs one square root and one reciprocal, that of (|r_ij|^2 + eta^2)(rho_i +
+// rho_j): 39 FP64 operations.  m_j F = -kF m t^3 with
 // t = 1 - q/2: the sums of D rho/Dt and of the acceleration are accumulated
 // with t^3 in place of m_j F and the caller scales them by -kF m, and the
 // running maximum is of mu / h, which the caller scales by h.  With DFS the
@@ -59,10 +87,7 @@ __device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, doub
     double rx = xj - xi, ry = yj - yi, rz = zj - zi;  // r_ij = r_j - r_i
     double ux = uxj - uxi, uy = uyj - uyi, uz = uzj - uzi;  // u_ij = u_j - u_i
     double r2 = rx * rx + ry * ry + rz * rz;
-    // |r_ij| = r2 / sqrt(r2); the integer max (on the bit pattern) lifts r2 = 0
-    // (coincident particles) to the smallest subnormal, so that r = 0 there
-    double r = r2 * rsqrt(__longlong_as_double(max(__double_as_longlong(r2), 1LL)));
-    double t = 1.0 - r * k.half_inv_h;
+    double t = 1.0 - sqrt3(r2) * k.half_inv_h;
     double t3 = t * t * t;  // m_j F / (-kF m), grad_i W_ij = F (r_i - r_j) = -F r_ij
     double udotr = ux * rx + uy * ry + uz * rz;  // u_ij . r_ij
     // Eq. 7: sum_j m_j (u_i - u_j) . grad_i W_ij = m_j F (u_ij . r_ij), plus the delta term
@@ -76,11 +101,13 @@ __device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, doub
         a.drho = fma(t3, udotr - g, a.drho);
     }
     // Eqs. 4-5: Pi_ij = -alpha c_bar mu / rho_bar, c_bar / rho_bar = (c_i + c_j) / (rho_i + rho_j),
-    // mu = h (u_ij . r_ij) / (|r_ij|^2 + eta^2) = h muh
-    double muh = udotr * __drcp_rn(r2 + k.eta2);
+    // mu = h (u_ij . r_ij) / (|r_ij|^2 + eta^2) = h muh, muh = mur (rho_i + rho_j)
+    double rsum = rhoi + rhoj;
+    double mur = udotr * rcp3((r2 + k.eta2) * rsum);
+    double muh = mur * rsum;
     double visc = 0.0;
     if (__double2hiint(udotr) < 0)  // u_ij . r_ij < 0 (a -0.0 gives a zero term)
-        visc = fma(k.nah, cj, k.nah * ci) * muh * __drcp_rn(rhoi + rhoj);
+        visc = fma(k.nah, cj, k.nah * ci) * mur;
     // Eq. 3: a_i -= m_j (...) grad_i W_ij = m_j (...) F r_ij, with
     // (P_i + P_j) / (rho_i rho_j) = (P_i / rho_i + P_j / rho_i) / rho_j
     double coef = fma(fma(Pj, inv_rhoi, Pi * inv_rhoi), inv_rhoj, visc) * t3;
@@ -107,18 +134,19 @@ __device__ __forceinline__ void pair_share_j(const PairConstD &k, double xi, dou
     double rx = xj - xi, ry = yj - yi, rz = zj - zi;
     double ux = uxj - uxi, uy = uyj - uyi, uz = uzj - uzi;
     double r2 = rx * rx + ry * ry + rz * rz;
-    double r = r2 * rsqrt(__longlong_as_double(max(__double_as_longlong(r2), 1LL)));
-    double t = 1.0 - r * k.half_inv_h;
+    double t = 1.0 - sqrt3(r2) * k.half_inv_h;
     double t3 = t * t * t;
     double udotr = ux * rx + uy * ry + uz * rz;
     const bool ff = fluid_i && fluid_j;
     double g = ff ? fma(-k.dfac * rhoi, inv_rhoj, k.dfac) : 0.0;
     double gj = ff ? fma(-k.dfac * rhoj, inv_rhoi, k.dfac) : 0.0;
     a.drho = fma(t3, udotr - g, a.drho);
-    double muh = udotr * __drcp_rn(r2 + k.eta2);
+    double rsum = rhoi + rhoj;
+    double mur = udotr * rcp3((r2 + k.eta2) * rsum);
+    double muh = mur * rsum;
     double visc = 0.0;
     if (__double2hiint(udotr) < 0)
-        visc = fma(k.nah, cj, k.nah * ci) * muh * __drcp_rn(rhoi + rhoj);
+        visc = fma(k.nah, cj, k.nah * ci) * mur;
     double coef = fma(fma(Pj, inv_rhoi, Pi * inv_rhoi), inv_rhoj, visc) * t3;
     a.ax += coef * rx;
     a.ay += coef * ry;
@@ -251,13 +279,14 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
         double tot[K] = {acc.drho, acc.ax, acc.ay, acc.az};
         if (DFS)
             tot[4] = acc.dd;
-        warp_totals<K>(tot);  // lane 0 holds the totals
-        double drho_sum = tot[0];
+        // lane 0 holds the totals; every operation here is paid for by the whole warp,
+        // so each lane scales its one total before the exchange
+        warp_totals<K>(tot, sF);
+        double drho = tot[0];
         if (DFS && !__any_sync(0xffffffffu, touches_boundary))
-            drho_sum -= tot[K > 4 ? 4 : 0];
-        double drho = sF * drho_sum;
-        double ax = sF * tot[1], ay = sF * tot[2], az = sF * tot[3];
-        double mumax = I.h * warp_max(__longlong_as_double(acc.mumax_bits));
+            drho -= tot[K > 4 ? 4 : 0];
+        double ax = tot[1], ay = tot[2], az = tot[3];
+        double mumax = I.h * __longlong_as_double(warp_max_bits(acc.mumax_bits));
         int nsum = warp_sum(nn);
         if (lane == 0) {
             if (fluid_i)

@@ -165,6 +165,10 @@ void fill_inst(HostInst &hi, const sph_params &p, int fine, bool tiled)
     const double pi = 3.14159265358979323846;
     d.kW = 21.0 / (16.0 * pi * in.h * in.h * in.h);
     d.kF = 5.0 * d.kW / (in.h * in.h);
+    d.half_inv_h = 0.5 / d.h;
+    d.kFm = d.kF * d.mass;
+    d.dfac_d = 2.0 * d.delta * d.h * d.c0;
+    d.nah = -d.alpha * d.h;
     d.csound = p.csound;
     d.delta_mode = p.delta_mode;
     d.nf = (int32_t)hi.nf;
