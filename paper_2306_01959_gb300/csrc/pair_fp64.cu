@@ -30,12 +30,15 @@ struct AccD {
 
 // Constants of an instance used by every pair.
 struct PairConstD {
-    double half_inv_h, kFm, dfac, nah, eta2;  // kFm = kF m, dfac = 2 delta h c0, nah = -alpha h
+    double half_inv_h, dfac, nah, eta2;  // dfac = 2 delta h c0, nah = -alpha h
+    unsigned long long kh, eta;          // fixed-point positions only
 };
 
+template <bool FIX>
 __device__ __forceinline__ PairConstD pair_const_d(const Inst &I)
 {
-    return PairConstD{I.half_inv_h, I.kFm, I.dfac_d, I.nah, I.eta2};
+    return FIX ? PairConstD{I.fx_hinv, I.fx_dfac, I.fx_nah, (double)I.fx_eta, I.fx_kh, I.fx_eta}
+               : PairConstD{I.half_inv_h, I.dfac_d, I.nah, I.eta2, 0ull, 0ull};
 }
 
 // The FP64 pipe of this GPU issues one warp operation every 64 cycles per
@@ -66,6 +69,101 @@ __device__ __forceinline__ double sqrt3(double a)
     return fma(s * e, fma(0.375, e, 0.5), s);
 }
 
+// ---------------------------------------------------------------------------
+// Fixed-point distances.  The FP64 pipe is the bound and the integer pipes idle
+// beside it, so the steps from the positions to t^3 = (1 - q/2)^3, 15 of the 39
+// FP64 operations of a pair, run in 64-bit integers instead.  Positions are
+// multiples of 2^-s with 2h in [2^52, 2^53) units: differences are exact, and the
+// rounding of a position, 2^-54 of 2h, is below that of the doubles over most of
+// a tank.  With D = 2^10 times a difference, R = sum (D^2 / 2^64) is r^2 to 2^-60 of
+// (2h)^2, r comes from it by one third-order step from the FP32 reciprocal square
+// root (as sqrt3), t and its cube are 62-bit fractions: |error of t^3| <= 2.4e-16,
+// against 2.8e-16 for the FP64 operations (both against extended precision, any
+// distance above 2h / 64 and 2h from 0.01 to 2; closer pairs, whose R has fewer
+// bits, take the FP64 operations).
+// 0.9 M-particle case: 16.8 -> 13.2 ms per pass (20.1 ms before the pair terms were
+// shortened); grids of more than 512 supports keep the doubles, whose resolution
+// there is no better but which the integers could not hold.
+// Scaling by powers of two is exact, so the sums carry the units along: with r_ij
+// in units of 2^-s, t^3 in 2^-62 and |r_ij|^2 + eta^2 in 2^(44 - 2s), the constants
+// of PairConstD absorb the factors and pair_sF, pair_hmu undo them.
+// ---------------------------------------------------------------------------
+// An integer of at most 2^53 in magnitude (exact), or any below 2^63 (truncated).
+__device__ __forceinline__ double int_to_double(long long v)
+{
+    const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int n = __clzll((long long)u);
+    const unsigned long long m = (u << (n & 63)) >> 11;
+    const int hi = (int)(m >> 32) + ((1085 - n) << 20);
+    const int sign = (int)((unsigned long long)v >> 32) & (int)0x80000000;
+    return u ? __hiloint2double(hi | sign, (int)m) : 0.0;
+}
+
+// t^3 in units of 2^-62 from R = |r_ij|^2 (see above), 2^48 <= R < 2^62.
+__device__ __forceinline__ long long fixed_t3(unsigned long long R, unsigned long long kh)
+{
+    const int n = __clzll((long long)R) & ~1;
+    const unsigned long long m = R << n;  // [2^62, 2^64): v = m / 2^62 in [1, 4)
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((float)(unsigned)(m >> 32)));
+    const unsigned Y = __float2uint_rz(y * 140737488355328.f);  // 2^32 / sqrt(v), saturating
+    auto mul = [&](unsigned long long a) {  // a Y / 2^32
+        return (a >> 32) * Y + __umulhi((unsigned)a, Y);
+    };
+    const unsigned long long S = mul(m);                                // sqrt(v), 62 fraction bits
+    const long long E = (1ll << 62) - (long long)mul(S);                // 1 - v y^2
+    const int e = (int)(E >> 12);
+    const long long g = (E >> 1) + ((3 * (((long long)e * e) >> 38)) >> 3);  // E / 2 + 3/8 E^2
+    const unsigned long long q = S + (__mul64hi((long long)S, g << 22) >> 20);
+    const unsigned long long r = q >> (n / 2 - 1);  // in units of 2^-(s + 10)
+    const long long t = max((1ll << 62) - (long long)__umul64hi(r, kh), 0ll);
+    const unsigned long long t1 = (unsigned long long)t << 1;
+    return (long long)__umul64hi(__umul64hi(t1, t1) << 1, t1);
+}
+
+// Geometry of a pair: r_ij, |r_ij|^2 + eta^2 and t^3, in the units of k.  The
+// positions are doubles, or (FIX) 64-bit integers in the same registers.
+struct PairGeoD {
+    double rx, ry, rz, re, t3;
+};
+template <bool FIX>
+__device__ __forceinline__ PairGeoD pair_geo_d(const PairConstD &k, double xi, double yi, double zi, double xj,
+                                               double yj, double zj)
+{
+    PairGeoD p;
+    if (FIX) {
+        const long long dx = __double_as_longlong(xj) - __double_as_longlong(xi);
+        const long long dy = __double_as_longlong(yj) - __double_as_longlong(yi);
+        const long long dz = __double_as_longlong(zj) - __double_as_longlong(zi);
+        const unsigned long long ax = (unsigned long long)(dx < 0 ? -dx : dx) << 10;
+        const unsigned long long ay = (unsigned long long)(dy < 0 ? -dy : dy) << 10;
+        const unsigned long long az = (unsigned long long)(dz < 0 ? -dz : dz) << 10;
+        const unsigned long long R = __umul64hi(ax, ax) + __umul64hi(ay, ay) + __umul64hi(az, az);
+        p.rx = int_to_double(dx);
+        p.ry = int_to_double(dy);
+        p.rz = int_to_double(dz);
+        if (R >= (1ull << 48)) {
+            p.re = int_to_double((long long)(R + k.eta));
+            // (a pair just within 2h can round to 2h, at most 2^62)
+            p.t3 = int_to_double(fixed_t3(min(R, (1ull << 62) - 1), k.kh));
+        } else {
+            const double r2 = p.rx * p.rx + p.ry * p.ry + p.rz * p.rz;
+            const double t = 1.0 - sqrt3(r2) * k.half_inv_h;
+            p.re = fma(r2, 0x1p-44, k.eta2);
+            p.t3 = t * t * t * 0x1p62;
+        }
+    } else {
+        p.rx = xj - xi;
+        p.ry = yj - yi;
+        p.rz = zj - zi;
+        const double r2 = p.rx * p.rx + p.ry * p.ry + p.rz * p.rz;
+        const double t = 1.0 - sqrt3(r2) * k.half_inv_h;
+        p.re = r2 + k.eta2;
+        p.t3 = t * t * t;  // m_j F / (-kF m)
+    }
+    return p;
+}
+
 // Contribution of neighbour j to particle i (Eqs. 3-7), in double.
 // Continuity uses the standard sign (u_i - u_j) . grad_i W_ij; the delta
 // term acts between fluid particles; the viscosity of Eq. 4 applies when
@@ -77,18 +175,16 @@ __device__ __forceinline__ double sqrt3(double a)
 // running maximum is of mu / h, which the caller scales by h.  With DFS the
 // delta term is summed apart (the caller drops it for a fluid particle that
 // has a boundary neighbour).
-template <bool DFS>
+template <bool DFS, bool FIX>
 __device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, double yi, double zi, double uxi,
                                             double uyi, double uzi, double rhoi, double inv_rhoi, double Pi,
                                             double ci, bool fluid_i, double xj, double yj, double zj, double uxj,
                                             double uyj, double uzj, double rhoj, double inv_rhoj, double Pj,
                                             double cj, bool fluid_j, AccD &a)
 {
-    double rx = xj - xi, ry = yj - yi, rz = zj - zi;  // r_ij = r_j - r_i
+    const PairGeoD p = pair_geo_d<FIX>(k, xi, yi, zi, xj, yj, zj);
+    const double rx = p.rx, ry = p.ry, rz = p.rz, t3 = p.t3;  // r_ij = r_j - r_i; grad_i W_ij = F (r_i - r_j) = -F r_ij
     double ux = uxj - uxi, uy = uyj - uyi, uz = uzj - uzi;  // u_ij = u_j - u_i
-    double r2 = rx * rx + ry * ry + rz * rz;
-    double t = 1.0 - sqrt3(r2) * k.half_inv_h;
-    double t3 = t * t * t;  // m_j F / (-kF m), grad_i W_ij = F (r_i - r_j) = -F r_ij
     double udotr = ux * rx + uy * ry + uz * rz;  // u_ij . r_ij
     // Eq. 7: sum_j m_j (u_i - u_j) . grad_i W_ij = m_j F (u_ij . r_ij), plus the delta term
     // 2 delta h c0 (rho_j - rho_i) (r_ij . grad_i W_ij) / |r_ij|^2 m_j / rho_j, where
@@ -103,7 +199,7 @@ __device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, doub
     // Eqs. 4-5: Pi_ij = -alpha c_bar mu / rho_bar, c_bar / rho_bar = (c_i + c_j) / (rho_i + rho_j),
     // mu = h (u_ij . r_ij) / (|r_ij|^2 + eta^2) = h muh, muh = mur (rho_i + rho_j)
     double rsum = rhoi + rhoj;
-    double mur = udotr * rcp3((r2 + k.eta2) * rsum);
+    double mur = udotr * rcp3(p.re * rsum);
     double muh = mur * rsum;
     double visc = 0.0;
     if (__double2hiint(udotr) < 0)  // u_ij . r_ij < 0 (a -0.0 gives a zero term)
@@ -124,6 +220,7 @@ __device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, doub
 // has the same continuity term and j's own delta term
 // 2 delta h c0 (1 - rho_j / rho_i), mu is the same; units as pair_term_d
 // (t^3 in place of m F, mu / h).  i's own share is accumulated in a.
+template <bool FIX>
 __device__ __forceinline__ void pair_share_j(const PairConstD &k, double xi, double yi, double zi, double uxi,
                                              double uyi, double uzi, double rhoi, double inv_rhoi, double Pi,
                                              double ci, bool fluid_i, double xj, double yj, double zj, double uxj,
@@ -131,18 +228,16 @@ __device__ __forceinline__ void pair_share_j(const PairConstD &k, double xi, dou
                                              double cj, bool fluid_j, dvec4 *jacc, long long *jmu, int32_t j,
                                              AccD &a)
 {
-    double rx = xj - xi, ry = yj - yi, rz = zj - zi;
+    const PairGeoD p = pair_geo_d<FIX>(k, xi, yi, zi, xj, yj, zj);
+    const double rx = p.rx, ry = p.ry, rz = p.rz, t3 = p.t3;
     double ux = uxj - uxi, uy = uyj - uyi, uz = uzj - uzi;
-    double r2 = rx * rx + ry * ry + rz * rz;
-    double t = 1.0 - sqrt3(r2) * k.half_inv_h;
-    double t3 = t * t * t;
     double udotr = ux * rx + uy * ry + uz * rz;
     const bool ff = fluid_i && fluid_j;
     double g = ff ? fma(-k.dfac * rhoi, inv_rhoj, k.dfac) : 0.0;
     double gj = ff ? fma(-k.dfac * rhoj, inv_rhoi, k.dfac) : 0.0;
     a.drho = fma(t3, udotr - g, a.drho);
     double rsum = rhoi + rhoj;
-    double mur = udotr * rcp3((r2 + k.eta2) * rsum);
+    double mur = udotr * rcp3(p.re * rsum);
     double muh = mur * rsum;
     double visc = 0.0;
     if (__double2hiint(udotr) < 0)
@@ -172,7 +267,8 @@ __device__ __forceinline__ double dist2_rn(double xi, double yi, double zi, doub
 // the partner's share by pair_share_j; k_pair_fp64_finish adds the shares.
 // CNT (with SYM): also count the partners' neighbours (nneigh is read by
 // sph_derivatives and the work counts, not by a time step).
-template <bool DFS, bool SYM, bool CNT = true>
+// FIX: fixed-point sorted positions.
+template <bool FIX, bool DFS, bool SYM, bool CNT = true>
 __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
 {
     extern __shared__ int32_t smem_q[];
@@ -194,7 +290,7 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
         const double2 Ci = b.sC[i];
         const float4 Di = b.sD[i];
         const bool fluid_i = b.sflag[i] == T_FLUID;
-        const PairConstD kc = pair_const_d(I);
+        const PairConstD kc = pair_const_d<FIX>(I);
         AccD acc = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
         bool touches_boundary = false;  // DFS: some neighbour j is a boundary particle
         int nn = 0;
@@ -207,11 +303,11 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
                 dvec4 Aj = sA[j], Bj = sB[j];
                 double2 Cj = b.sC[j];
                 if (SYM)
-                    pair_share_j(kc, Ai.x, Ai.y, Ai.z, Bi.x, Bi.y, Bi.z, Ai.w, Ci.x, Bi.w, Ci.y, fluid_i, Aj.x, Aj.y,
+                    pair_share_j<FIX>(kc, Ai.x, Ai.y, Ai.z, Bi.x, Bi.y, Bi.z, Ai.w, Ci.x, Bi.w, Ci.y, fluid_i, Aj.x, Aj.y,
                                  Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, b.sflag[j] == T_FLUID, b.fjacc, b.fjmu,
                                  j, acc);
                 else
-                    pair_term_d<DFS>(kc, Ai.x, Ai.y, Ai.z, Bi.x, Bi.y, Bi.z, Ai.w, Ci.x, Bi.w, Ci.y, fluid_i, Aj.x,
+                    pair_term_d<DFS, FIX>(kc, Ai.x, Ai.y, Ai.z, Bi.x, Bi.y, Bi.z, Ai.w, Ci.x, Bi.w, Ci.y, fluid_i, Aj.x,
                                      Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, b.sflag[j] == T_FLUID, acc);
             }
         };
@@ -241,8 +337,8 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
                         const float d2f = fx * fx + fy * fy + fz * fz;
                         bool hit = d2f < I.sup2_inner;
                         if (!hit && d2f < I.sup2_filter) {
-                            dvec4 Aj = sA[j];
-                            hit = dist2_rn(Ai.x, Ai.y, Ai.z, Aj.x, Aj.y, Aj.z) < I.sup2;
+                            const dvec4 ri = b.pos[b.perm[i]], rj = b.pos[b.perm[j]];
+                            hit = dist2_rn(ri.x, ri.y, ri.z, rj.x, rj.y, rj.z) < I.sup2;
                         }
                         if (hit) {
                             ++nn;
@@ -274,7 +370,7 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
         }
         flush(qn);
         __syncwarp();
-        const double sF = -kc.kFm;  // t^3 -> m_j F
+        const double sF = I.pair_sF;  // t^3 -> m_j F
         constexpr int K = DFS ? 8 : 4;
         double tot[K] = {acc.drho, acc.ax, acc.ay, acc.az};
         if (DFS)
@@ -286,7 +382,7 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
         if (DFS && !__any_sync(0xffffffffu, touches_boundary))
             drho -= tot[K > 4 ? 4 : 0];
         double ax = tot[1], ay = tot[2], az = tot[3];
-        double mumax = I.h * __longlong_as_double(warp_max_bits(acc.mumax_bits));
+        double mumax = I.pair_hmu * __longlong_as_double(warp_max_bits(acc.mumax_bits));
         int nsum = warp_sum(nn);
         if (lane == 0) {
             if (fluid_i)
@@ -307,47 +403,56 @@ __global__ void k_pair_fp64_finish(Bufs b, int ninst)
     const int32_t n_in = b.misc[0];
     for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n_in; s += gridDim.x * blockDim.x) {
         const Inst &I = b.inst[inst_of_cell(b.inst, ninst, b.scell[s])];
-        const double sF = -I.kF * I.mass;
+        const double sF = I.pair_sF;
         const dvec4 j = b.fjacc[s];
         dvec4 *D = reinterpret_cast<dvec4 *>(b.deriv) + s;
         const dvec4 d = *D;
         *D = make_dvec4(d.x + sF * j.x, d.y + sF * j.y, d.z + sF * j.z, d.w + sF * j.w);
         double *M = reinterpret_cast<double *>(b.mumax) + s;
-        *M = fmax(*M, I.h * __longlong_as_double(b.fjmu[s]));
+        *M = fmax(*M, I.pair_hmu * __longlong_as_double(b.fjmu[s]));
         if (CNT)
             b.nneigh[s] += b.fjnn[s];
     }
 }
 
-void launch_pair_fp64(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas,
-                      int32_t delta_mode, bool neighbours, cudaStream_t st)
+template <bool FIX>
+static void launch_form(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int grid, int warps,
+                        int32_t delta_mode, bool neighbours, cudaStream_t st)
 {
-    if (warps <= 0 || warps > 8)
-        warps = 8;  // the kernel is compiled for at most 256 threads per CTA
-    if (ctas <= 0)
-        ctas = 8;
-    const int sms = sm_count();
+    const size_t dyn = warps * kQ * sizeof(int32_t);
     if (b.fjacc) {
         // the partners' accumulators start at zero (mu / h >= 0 as bits)
         cudaMemsetAsync(b.fjacc, 0, sizeof(dvec4) * (size_t)N, st);
         cudaMemsetAsync(b.fjmu, 0, sizeof(long long) * (size_t)N, st);
-        const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((N + 255) / 256, (int64_t)sms * 8));
+        const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((N + 255) / 256, (int64_t)sm_count() * 8));
         if (neighbours) {
             cudaMemsetAsync(b.fjnn, 0, sizeof(int32_t) * (size_t)N, st);
-            k_pair_fp64<false, true, true><<<sms * ctas, warps * 32, warps * kQ * sizeof(int32_t), st>>>(b, ninst,
-                                                                                                      cell_div);
+            k_pair_fp64<FIX, false, true, true><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
             k_pair_fp64_finish<true><<<blocks, 256, 0, st>>>(b, ninst);
         } else {
-            k_pair_fp64<false, true, false><<<sms * ctas, warps * 32, warps * kQ * sizeof(int32_t), st>>>(b, ninst,
-                                                                                                       cell_div);
+            k_pair_fp64<FIX, false, true, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
             k_pair_fp64_finish<false><<<blocks, 256, 0, st>>>(b, ninst);
         }
         return;
     }
     if (delta_mode == SPH_DELTA_FULL_SUPPORT)
-        k_pair_fp64<true, false><<<sms * ctas, warps * 32, warps * kQ * sizeof(int32_t), st>>>(b, ninst, cell_div);
+        k_pair_fp64<FIX, true, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
     else
-        k_pair_fp64<false, false><<<sms * ctas, warps * 32, warps * kQ * sizeof(int32_t), st>>>(b, ninst, cell_div);
+        k_pair_fp64<FIX, false, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
+}
+
+void launch_pair_fp64(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas,
+                      int32_t delta_mode, bool neighbours, bool fixed, cudaStream_t st)
+{
+    if (warps <= 0 || warps > 8)
+        warps = 8;  // the kernel is compiled for at most 256 threads per CTA
+    if (ctas <= 0)
+        ctas = 8;
+    const int grid = sm_count() * ctas;
+    if (fixed)
+        launch_form<true>(b, N, ninst, cell_div, grid, warps, delta_mode, neighbours, st);
+    else
+        launch_form<false>(b, N, ninst, cell_div, grid, warps, delta_mode, neighbours, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -394,7 +499,7 @@ __global__ void k_probe_force(Bufs b, int inst, int kdiv)
         double xb, yb, zb, uxb, uyb, uzb, rhob;
         load_state<MODE>(b, I, idb, xb, yb, zb, uxb, uyb, uzb, rhob);
         double Pb = tait_d(I, rhob), cb = sound_d(I, rhob);
-        const PairConstD kc = pair_const_d(I);
+        const PairConstD kc = pair_const_d<false>(I);
         int cx, cy, cz;
         decompose(I, b.scell[s], cx, cy, cz);
         AccD acc = {0, 0, 0, 0, 0};
@@ -416,12 +521,12 @@ __global__ void k_probe_force(Bufs b, int inst, int kdiv)
                     double xj, yj, zj, uxj, uyj, uzj, rhoj;
                     load_state<MODE>(b, I, idj, xj, yj, zj, uxj, uyj, uzj, rhoj);
                     if (dist2_rn(xb, yb, zb, xj, yj, zj) < I.sup2)
-                        pair_term_d<false>(kc, xb, yb, zb, uxb, uyb, uzb, rhob, 1.0 / rhob, Pb, cb, false, xj, yj, zj, uxj,
+                        pair_term_d<false, false>(kc, xb, yb, zb, uxb, uyb, uzb, rhob, 1.0 / rhob, Pb, cb, false, xj, yj, zj, uxj,
                                     uyj, uzj, rhoj, 1.0 / rhoj, tait_d(I, rhoj), sound_d(I, rhoj), true, acc);
                 }
             }
         }
-        const double sF = -kc.kFm * I.mass;  // t^3 -> m_j F, times the obstacle particle's mass
+        const double sF = -I.kFm * I.mass;  // t^3 -> m_j F, times the obstacle particle's mass
         fx += sF * acc.ax;
         fy += sF * acc.ay;
         fz += sF * acc.az;
