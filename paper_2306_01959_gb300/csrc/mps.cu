@@ -9,7 +9,7 @@
 // at r* (counting sort by cell, per-cell sort by id, so the candidate order is
 // (cell, id) as in the method's definition of the neighbourhood).  The system
 // of Eq. 23 lives in sorted-index space: row i holds the diagonal and up to
-// `row_width` off-diagonal entries stored column-major (entry k of every row
+// `row_width` off-diagonal entries, stored for 32 rows at a time (entry k of the 32
 // contiguous), so that the one-thread-per-row product reads coalesced; rows of
 // particles that are not unknowns are identity rows with a zero right-hand
 // side, which keeps every vector the length of the sorted order.
@@ -25,9 +25,7 @@ namespace {
 
 using namespace sph;
 
-constexpr int kCgBlocks = 1024;  // fixed block count of the reductions (deterministic sums)
-constexpr int kCgThreads = 256;
-constexpr int kCgChunk = 16;     // CG iterations launched between convergence checks
+constexpr int kCgChunk = 16;  // the iteration cap is rounded up to a multiple of this
 
 struct MpsConst {
     double lo[3];
@@ -45,18 +43,26 @@ struct MpsBufs {
     uint8_t *moved;            // id order: predicted in this step (reset by k_mps_finish)
     double *P;                 // id order: pressure of the last step (clamped)
     uint32_t *key, *count;
-    int32_t *cell_start, *active, *perm, *ptmp, *misc;  // misc: [0] n_in, [1] n_active, [2] status
+    int32_t *cell_start, *active, *perm, *ptmp, *misc;  // misc: [0] n_in, [1] n_active, [2] status, [5] a list overflowed
     uint64_t *scan_blocks;
     dvec4 *spos;               // sorted: x, y, z, type
     float4 *sposf;             // sorted: FP32 copies of x, y, z (the candidate pre-test)
-    double *snd, *ssig;        // sorted: n*, centroid deviation
+    double *snd;               // sorted: n*
+    int32_t *ncan;             // sorted: candidates listed for the particle, then its pressure neighbours
     uint8_t *surf;             // sorted: free-surface flag
-    int32_t *ecnt, *ecol;      // sorted rows: entry count; entry k of row i at [k * N + i]
+    int32_t *ecnt, *ecol;      // sorted rows: entry count; entry k of row i at row_entry(i, k)
     double *eval, *diag, *rhs;
-    double *x, *r, *p, *q, *part, *scal;  // scal: [0] rho, [1] |b|^2, [2] alpha, [3] beta
-    int32_t *cgi;              // [0] iterations, [1] done
+    double *x, *r, *p, *q, *part, *scal;  // scal: [0] r.r, [1] |b|^2
+    int32_t *cgi;              // [0] iterations, [1] done, [2] barrier counter of the solve
     MpsConst *c;
 };
+
+// Entry k of row i: 32 rows share a block of memory, entry by entry, so that a warp
+// of one row per lane reads whole lines and stays within a few kilobytes.
+__device__ __forceinline__ int64_t row_entry(int width, int32_t i, int k)
+{
+    return ((int64_t)(i >> 5) * width + k) * 32 + (i & 31);
+}
 
 // The weight of Eq. 16 (r_e / |r_ij| - 1 within r_e, 0 beyond and for
 // coincident particles) from the squared distance, through one reciprocal
@@ -217,9 +223,185 @@ __device__ __forceinline__ double wsum(double v)
     return v;
 }
 
+// ---------------------------------------------------------------- candidate lists
+// One thread per particle lists the candidates that pass the FP32 pre-test in the
+// columns of the system, in (cell, id) order;
+// the FP64 passes over them then run one particle per thread.  The FP64 pipe bounds
+// the neighbour passes, and per warp it does one operation for 32 pairs or 32
+// particles: with a warp per particle a quarter of the lanes held no pair, and the
+// work of the particle itself (totals, the deviation's root and quotient, the 3 x 3
+// system of Eq. 24) cost as much as 32 particles' worth here.
+// A particle with more candidates than row_width sets misc[5]: the warp-per-particle
+// kernels below, which search by themselves, then take the place of the list ones.
+__global__ void __launch_bounds__(256) k_mps_list(MpsBufs b, int fluid_only)
+{
+    const MpsConst &C = *b.c;
+    const int32_t n_in = b.misc[0];
+    const int width = C.width;
+    for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n_in; s += gridDim.x * blockDim.x) {
+        const int32_t id = b.perm[s];
+        if (fluid_only && b.type[id] != MPS_FLUID)
+            continue;
+        const float4 pi = b.sposf[s];
+        const int32_t c = (int32_t)b.key[id];
+        const int cx = c % C.n[0], t = c / C.n[0], cy = t % C.n[1], cz = t / C.n[1];
+        const int x0 = max(cx - 1, 0), x1 = min(cx + 1, C.n[0] - 1);
+        int32_t *col = b.ecol + row_entry(width, s, 0);
+        int cnt = 0;
+        for (int z = max(cz - 1, 0); z <= min(cz + 1, C.n[2] - 1); ++z)
+            for (int y = max(cy - 1, 0); y <= min(cy + 1, C.n[1] - 1); ++y) {
+                const int32_t row = (z * C.n[1] + y) * C.n[0];
+                const int32_t j0 = b.cell_start[row + x0], j1 = b.cell_start[row + x1 + 1];
+#pragma unroll 4
+                for (int32_t j = j0; j < j1; ++j) {
+                    const float4 a = b.sposf[j];
+                    const float dx = a.x - pi.x, dy = a.y - pi.y, dz = a.z - pi.z;
+                    if (dx * dx + dy * dy + dz * dz <= C.re2f && j != s) {
+                        if (cnt < width)
+                            col[32 * cnt] = j;
+                        ++cnt;
+                    }
+                }
+            }
+        b.ncan[s] = cnt;
+        if (cnt > width)
+            b.misc[5] = 1;
+    }
+}
+
+// 1 / sqrt(a) for a normal a > 0: the hardware's 20-bit approximation and one
+// third-order step (Householder's method; remaining error below the rounding).
+__device__ __forceinline__ double rsqrt3(double a)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// A listed pair: r_j - r_i, 1/|r_ij| and the weight of Eq. 16; false (and 0) beyond
+// r_e and for coincident particles, compared by the bit patterns (non-negative
+// doubles order like them).
+struct MpsPair {
+    double dx, dy, dz, inv, w;
+};
+__device__ __forceinline__ bool mps_pair(const dvec4 pi, const dvec4 pj, double re, long long re2_bits, MpsPair &p)
+{
+    p.dx = pj.x - pi.x;
+    p.dy = pj.y - pi.y;
+    p.dz = pj.z - pi.z;
+    const double d2 = p.dx * p.dx + p.dy * p.dy + p.dz * p.dz;
+    const long long bits = __double_as_longlong(d2);
+    const bool in = bits > (1ll << 52) && bits <= re2_bits;
+    p.inv = rsqrt3(in ? d2 : 1.0);
+    p.w = in ? re * p.inv - 1.0 : 0.0;
+    return in;
+}
+
+// Calls f(j, r_j) for the entries of a list or row, four loads in flight; past the end
+// j = s, which is no pair.
+template <class F>
+__device__ __forceinline__ void for_row(const MpsBufs &b, int width, int32_t s, int cnt, F &&f)
+{
+    const int32_t *col = b.ecol + row_entry(width, s, 0);
+    for (int e = 0; e < cnt; e += 4) {
+        int32_t j[4];
+        dvec4 pj[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            j[u] = e + u < cnt ? col[32 * (e + u)] : s;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            pj[u] = b.spos[j[u]];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            f(j[u], pj[u]);
+    }
+}
+
+// Eqs. 21-22 over the lists.
+__global__ void __launch_bounds__(256) k_mps_predict_rows(MpsBufs b)
+{
+    if (b.misc[5])
+        return;
+    const MpsConst &C = *b.c;
+    const int32_t n_in = b.misc[0];
+    const double re = C.re, k = C.nu * C.lapc, dt = C.dt, g = C.g;
+    const long long re2 = __double_as_longlong(re * re);
+    for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n_in; s += gridDim.x * blockDim.x) {
+        const dvec4 pi = b.spos[s];
+        if ((int)pi.w != MPS_FLUID)
+            continue;
+        const int32_t id = b.perm[s];
+        const dvec4 ui = b.vel[id];
+        const int cnt = b.ncan[s];
+        double lx = 0.0, ly = 0.0, lz = 0.0;
+        for_row(b, C.width, s, cnt, [&](int32_t j, const dvec4 &pj) {
+            MpsPair p;
+            mps_pair(pi, pj, re, re2, p);
+            const dvec4 uj = b.vel[b.perm[j]];
+            lx += (uj.x - ui.x) * p.w;
+            ly += (uj.y - ui.y) * p.w;
+            lz += (uj.z - ui.z) * p.w;
+        });
+        b.moved[id] = 1;
+        const dvec4 us = make_dvec4(ui.x + dt * (k * lx), ui.y + dt * (k * ly), ui.z + dt * (k * lz - g), 0.0);
+        b.ustar[id] = us;
+        const dvec4 q = b.pos[id];
+        b.pos[id] = make_dvec4(q.x + dt * us.x, q.y + dt * us.y, q.z + dt * us.z, 0.0);
+    }
+}
+
+// Eqs. 17, 28-30 and the rows of Eq. 23 over the lists, which become the rows: the
+// neighbours with a pressure (not dummy) and their coefficients; ncan keeps their
+// number for the gradient.  Columns of free-surface particles stay in: their p is
+// exactly zero throughout the solve.
+__global__ void __launch_bounds__(256) k_mps_density_rows(MpsBufs b)
+{
+    if (b.misc[5])
+        return;
+    const MpsConst &C = *b.c;
+    const int32_t n_in = b.misc[0];
+    const double re = C.re, lapc = C.lapc;
+    const long long re2 = __double_as_longlong(re * re);
+    for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n_in; s += gridDim.x * blockDim.x) {
+        const dvec4 pi = b.spos[s];
+        const bool solid = (int)pi.w != MPS_DUMMY;
+        const int cnt = b.ncan[s];
+        double sw = 0.0, sx = 0.0, sy = 0.0, sz = 0.0, sp = 0.0;
+        const int64_t e0 = row_entry(C.width, s, 0);
+        int m = 0;
+        for_row(b, C.width, s, cnt, [&](int32_t j, const dvec4 &pj) {
+            MpsPair p;
+            const bool in = mps_pair(pi, pj, re, re2, p);
+            sw += p.w;
+            sx += p.dx * p.w;
+            sy += p.dy * p.w;
+            sz += p.dz * p.w;
+            if (in && solid && (int)__double2hiint(pj.w) != 0x40000000) {  // w = 2.0 marks a dummy particle
+                sp += p.w;
+                b.ecol[e0 + 32 * m] = j;
+                b.eval[e0 + 32 * m] = -lapc * p.w;
+                ++m;
+            }
+        });
+        const double sig = sw > 0.0 ? sqrt(sx * sx + sy * sy + sz * sz) / sw : 0.0;
+        const bool surf = solid && sw < C.beta1 * C.n0 && sig > C.varrho1 * C.l0;
+        const bool unknown = solid && !surf;
+        b.snd[s] = sw;
+        b.surf[s] = surf ? 1 : 0;
+        b.ncan[s] = m;
+        b.ecnt[s] = unknown ? m : 0;
+        b.diag[s] = unknown ? lapc * sp + C.rho * C.kc / (C.dt * C.dt) : 1.0;
+        b.rhs[s] = unknown ? C.kr * C.rho / (C.dt * C.dt) * (sw - C.n0) / C.n0 : 0.0;
+    }
+}
+
 // ---------------------------------------------------------------- Eqs. 21-22
 __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_predict(MpsBufs b)
 {
+    if (!b.misc[5])
+        return;  // the lists hold every candidate
     __shared__ int32_t nbuf[kMpsWarps][64];
     int32_t *buf = nbuf[threadIdx.x >> 5];
     const MpsConst &C = *b.c;
@@ -267,6 +449,8 @@ __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_predict(MpsBufs b)
 // ---------------------------------------------------------------- Eq. 17, Eqs. 28-30
 __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_density(MpsBufs b)
 {
+    if (!b.misc[5])
+        return;
     __shared__ int32_t nbuf[kMpsWarps][64];
     int32_t *buf = nbuf[threadIdx.x >> 5];
     const MpsConst &C = *b.c;
@@ -298,7 +482,6 @@ __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_density(MpsBufs b)
         if ((threadIdx.x & 31) == 0) {
             const double sig = sw > 0.0 ? sqrt(sx * sx + sy * sy + sz * sz) / sw : 0.0;
             b.snd[s] = sw;
-            b.ssig[s] = sig;
             b.surf[s] = ((int)pi.w != MPS_DUMMY && sw < C.beta1 * C.n0 && sig > C.varrho1 * C.l0) ? 1 : 0;
         }
     }
@@ -308,8 +491,10 @@ __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_density(MpsBufs b)
 // Row of sorted particle s (times -1, so that the system is SPD):
 //   (lapc sum_{j non-dummy} w_ij + rho kappa_c / dt^2) P_s - lapc sum_{j unknown} w_ij P_j
 //     = kappa_r rho / dt^2 (n*_s - n0) / n0.
-__global__ void __launch_bounds__(kMpsWarps * 32) k_mps_assemble(MpsBufs b, int32_t Ns)
+__global__ void __launch_bounds__(kMpsWarps * 32) k_mps_assemble(MpsBufs b)
 {
+    if (!b.misc[5])
+        return;
     __shared__ int32_t nbuf[kMpsWarps][64];
     int32_t *buf = nbuf[threadIdx.x >> 5];
     const MpsConst &C = *b.c;
@@ -351,8 +536,8 @@ __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_assemble(MpsBufs b, int3
             if (take) {
                 const int k = cnt + __popc(m & lt);
                 if (k < C.width) {
-                    b.ecol[(int64_t)k * Ns + s] = j;
-                    b.eval[(int64_t)k * Ns + s] = -C.lapc * w;
+                    b.ecol[row_entry(C.width, s, k)] = j;
+                    b.eval[row_entry(C.width, s, k)] = -C.lapc * w;
                 } else {
                     over = true;
                 }
@@ -372,8 +557,16 @@ __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_assemble(MpsBufs b, int3
 }
 
 // ---------------------------------------------------------------- CG
-// Block sums over a fixed grid of kCgBlocks blocks; the partials are summed by
-// one block in a fixed order, so every dot product is deterministic.
+// The whole solve in one cooperative launch: the product with p.q, the update with
+// r.r and the direction stand between grid barriers instead of kernel boundaries
+// (a coarse tank spent 36 us per iteration on five launches and their gaps), and
+// the convergence test needs no word from the host.  Every dot product adds a
+// fixed partition in a fixed order: thread, CTA, then the CTAs' partial sums, which
+// every CTA adds for itself.
+constexpr int kCgThreads = 256;
+constexpr int kCgMaxBlocks = 2048;  // partial sums held per dot product
+constexpr int kCgSpin = 20000000;   // polls of a barrier wait before it gives up
+
 __device__ __forceinline__ double block_sum(double v, double *sh)
 {
     v = wsum(v);
@@ -383,110 +576,135 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
         sh[w] = v;
     __syncthreads();
     double t = 0.0;
-    if (threadIdx.x < 32) {
-        t = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-        t = wsum(t);
-    }
-    return t;  // valid in thread 0
+    for (int k = 0; k < kCgThreads / 32; ++k)
+        t += sh[k];
+    return t;
 }
 
-__global__ void k_cg_init(MpsBufs b, int32_t Ns)
+// Grid barrier (every CTA is resident); false when the wait ran out.
+__device__ __forceinline__ bool cg_barrier(MpsBufs &b, unsigned &target, int *s_ok)
 {
-    __shared__ double sh[32];
+    __syncthreads();
+    target += gridDim.x;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&b.cgi[2], 1);
+        int polls = 0;
+        bool ok = true;
+        // (the counter may wrap)
+        while ((int)(*(volatile unsigned *)&b.cgi[2] - target) < 0) {
+            if (++polls > kCgSpin) {
+                atomicOr(&b.misc[2], ST_TIMEOUT);
+                ok = false;
+                break;
+            }
+            __nanosleep(20);
+        }
+        __threadfence();
+        *s_ok = ok;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+}
+
+__global__ void __launch_bounds__(kCgThreads) k_cg_solve(MpsBufs b, int max_iterations)
+{
+    const int width = b.c->width;
+    __shared__ double sh[kCgThreads / 32];
+    __shared__ int s_ok;
+    unsigned target = 0;
+    int phase = 0;
     const int32_t n_in = b.misc[0];
+    const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    // the sum of v over the grid (a barrier); the two halves of part alternate
+    auto total = [&](double v, double &sum) {
+        double *part = b.part + (phase & 1) * kCgMaxBlocks;
+        ++phase;
+        v = block_sum(v, sh);
+        if (threadIdx.x == 0)
+            part[blockIdx.x] = v;
+        if (!cg_barrier(b, target, &s_ok))
+            return false;
+        double t = 0.0;
+        for (int k = threadIdx.x; k < (int)gridDim.x; k += kCgThreads)
+            t += __ldcg(part + k);
+        sum = block_sum(t, sh);
+        return true;
+    };
     double bb = 0.0;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < Ns; i += gridDim.x * blockDim.x) {
-        const double v = i < n_in ? b.rhs[i] : 0.0;
+    for (int32_t i = i0; i < n_in; i += stride) {
+        const double v = b.rhs[i];
         b.x[i] = 0.0;
         b.r[i] = v;
         b.p[i] = v;
         bb += v * v;
     }
-    bb = block_sum(bb, sh);
-    if (threadIdx.x == 0)
-        b.part[blockIdx.x] = bb;
-}
-
-// One block: total of the partials into scal[slot]; init also sets rho and
-// the counters.
-__global__ void k_cg_total(MpsBufs b, int slot, int init)
-{
-    __shared__ double sh[32];
-    if (!init && b.cgi[1])
+    if (!total(bb, bb))  // |b|^2; p is complete
         return;
-    double v = 0.0;
-    for (int k = threadIdx.x; k < kCgBlocks; k += blockDim.x)
-        v += b.part[k];
-    v = block_sum(v, sh);
-    if (threadIdx.x == 0) {
-        if (init) {
-            b.scal[1] = v;  // |b|^2
-            b.scal[0] = v;  // rho = r.r with r = b
-            b.cgi[0] = 0;
-            b.cgi[1] = v == 0.0;  // a zero right-hand side is solved by P = 0
-        } else if (slot == 2) {
-            b.scal[2] = b.scal[0] / v;  // alpha = rho / p.q
-        } else {
-            const double rho_new = v;
-            b.scal[3] = rho_new / b.scal[0];  // beta
-            b.scal[0] = rho_new;
-            b.cgi[0] += 1;
-            if (sqrt(rho_new) <= b.c->tol * sqrt(b.scal[1]) || !(rho_new == rho_new))
-                b.cgi[1] = 1;
-        }
-    }
-}
-
-__global__ void k_cg_spmv(MpsBufs b, int32_t Ns)
-{
-    __shared__ double sh[32];
-    if (b.cgi[1])
-        return;
-    const int32_t n_in = b.misc[0];
-    double pq = 0.0;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < Ns; i += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        if (i < n_in) {
-            s = b.diag[i] * b.p[i];
+    double rho = bb;  // r.r with r = b
+    int it = 0;
+    bool done = bb == 0.0;  // a zero right-hand side is solved by P = 0
+    while (!done && it < max_iterations) {
+        double pq = 0.0;
+        for (int32_t i = i0; i < n_in; i += stride) {
+            const double pi = b.p[i];
+            double s = b.diag[i] * pi;
             const int cnt = b.ecnt[i];
-            for (int k = 0; k < cnt; ++k)
-                s += b.eval[(int64_t)k * Ns + i] * b.p[b.ecol[(int64_t)k * Ns + i]];
+            // the matrix streams past the caches, which keep the vectors
+            const int64_t e0 = row_entry(width, i, 0);
+            const double *ev = b.eval + e0;
+            const int32_t *ec = b.ecol + e0;
+            int k = 0;
+            for (; k + 8 <= cnt; k += 8) {
+                double v[8], g[8];
+                int32_t c[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    c[u] = __ldcs(ec + 32 * (k + u));
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    v[u] = __ldcs(ev + 32 * (k + u));
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    g[u] = b.p[c[u]];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    s += v[u] * g[u];
+            }
+            for (; k < cnt; ++k)
+                s += __ldcs(ev + 32 * k) * b.p[__ldcs(ec + 32 * k)];
+            b.q[i] = s;
+            pq += pi * s;
         }
-        b.q[i] = s;
-        pq += b.p[i] * s;
+        if (!total(pq, pq))
+            return;
+        const double alpha = rho / pq;
+        double rr = 0.0;
+        for (int32_t i = i0; i < n_in; i += stride) {
+            b.x[i] += alpha * b.p[i];
+            const double ri = b.r[i] - alpha * b.q[i];
+            b.r[i] = ri;
+            rr += ri * ri;
+        }
+        if (!total(rr, rr))
+            return;
+        const double beta = rr / rho;
+        rho = rr;
+        ++it;
+        done = sqrt(rr) <= b.c->tol * sqrt(bb) || !(rr == rr);
+        if (done)
+            break;
+        for (int32_t i = i0; i < n_in; i += stride)
+            b.p[i] = b.r[i] + beta * b.p[i];
+        if (!cg_barrier(b, target, &s_ok))
+            return;
     }
-    pq = block_sum(pq, sh);
-    if (threadIdx.x == 0)
-        b.part[blockIdx.x] = pq;
-}
-
-__global__ void k_cg_update(MpsBufs b, int32_t Ns)
-{
-    __shared__ double sh[32];
-    if (b.cgi[1])
-        return;
-    const double alpha = b.scal[2];
-    double rr = 0.0;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < Ns; i += gridDim.x * blockDim.x) {
-        b.x[i] += alpha * b.p[i];
-        const double ri = b.r[i] - alpha * b.q[i];
-        b.r[i] = ri;
-        rr += ri * ri;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        b.scal[0] = rho;
+        b.scal[1] = bb;
+        b.cgi[0] = it;
+        b.cgi[1] = done;
     }
-    rr = block_sum(rr, sh);
-    if (threadIdx.x == 0)
-        b.part[blockIdx.x] = rr;
-}
-
-__global__ void k_cg_direction(MpsBufs b, int32_t Ns)
-{
-    // the iteration that reached the tolerance has set the flag; its direction
-    // update is not needed
-    if (b.cgi[1])
-        return;
-    const double beta = b.scal[3];
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < Ns; i += gridDim.x * blockDim.x)
-        b.p[i] = b.r[i] + beta * b.p[i];
 }
 
 // ---------------------------------------------------------------- clamp, Eq. 24, Eqs. 25-26
@@ -503,8 +721,83 @@ __global__ void k_mps_clamp(MpsBufs b, int32_t Ns)
     (void)Ns;
 }
 
+// Eqs. 24-26 of one particle from its sums: M, sum P_j r_ij w / d^2, sum r_ij w / d^2
+// and P_hat.
+__device__ __forceinline__ void mps_correct_particle(const MpsBufs &b, const MpsConst &C, int32_t s, double pmin,
+                                                     double m00, double m01, double m02, double m11, double m12,
+                                                     double m22, double vx, double vy, double vz, double ax, double ay,
+                                                     double az)
+{
+    const double v0 = vx - pmin * ax, v1 = vy - pmin * ay, v2 = vz - pmin * az;
+    // M^{-1} v by the adjugate of the symmetric moment matrix
+    const double c00 = m11 * m22 - m12 * m12, c01 = m02 * m12 - m01 * m22, c02 = m01 * m12 - m02 * m11;
+    const double c11 = m00 * m22 - m02 * m02, c12 = m02 * m01 - m00 * m12, c22 = m00 * m11 - m01 * m01;
+    const double det = m00 * c00 + m01 * c01 + m02 * c02;
+    const double scale = (m00 + m11 + m22) / 3.0;
+    double gx = 0.0, gy = 0.0, gz = 0.0;
+    if (fabs(det) > 1e-12 * scale * scale * scale) {
+        gx = (c00 * v0 + c01 * v1 + c02 * v2) / det;
+        gy = (c01 * v0 + c11 * v1 + c12 * v2) / det;
+        gz = (c02 * v0 + c12 * v1 + c22 * v2) / det;
+    }
+    const int32_t id = b.perm[s];
+    const dvec4 us = b.ustar[id];
+    const double k = C.dt / C.rho;
+    const dvec4 un = make_dvec4(us.x - k * gx, us.y - k * gy, us.z - k * gz, 0.0);
+    b.vel[id] = un;
+    const dvec4 p = b.pos[id];
+    b.pos[id] = make_dvec4(p.x + C.dt * (un.x - us.x), p.y + C.dt * (un.y - us.y), p.z + C.dt * (un.z - us.z), 0.0);
+    if (!(un.x == un.x && un.y == un.y && un.z == un.z))
+        atomicOr(&b.misc[2], ST_UNSTABLE);
+}
+
+// Eqs. 24-26 over the rows of the system: a row's columns are the particle's
+// neighbours with a pressure.
+__global__ void __launch_bounds__(256) k_mps_correct_rows(MpsBufs b)
+{
+    if (b.misc[5])
+        return;
+    const MpsConst &C = *b.c;
+    const int32_t n_in = b.misc[0];
+    const double *P = b.q;
+    const double re = C.re;
+    const long long re2 = __double_as_longlong(re * re);
+    for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n_in; s += gridDim.x * blockDim.x) {
+        const dvec4 pi = b.spos[s];
+        if ((int)pi.w != MPS_FLUID)
+            continue;
+        const int cnt = b.ncan[s];
+        long long pmin = __double_as_longlong(P[s]);  // clamped pressures order like their bits
+        double m00 = 0, m01 = 0, m02 = 0, m11 = 0, m12 = 0, m22 = 0, vx = 0, vy = 0, vz = 0, ax = 0, ay = 0, az = 0;
+        for_row(b, C.width, s, cnt, [&](int32_t j, const dvec4 &pj) {
+            const double Pj = P[j];
+            MpsPair p;
+            mps_pair(pi, pj, re, re2, p);
+            // f = w / d^2: M = sum f r r^T, and f r in the other sums
+            const double f = p.w * (p.inv * p.inv);
+            const double fx = f * p.dx, fy = f * p.dy, fz = f * p.dz;
+            m00 += fx * p.dx;
+            m01 += fx * p.dy;
+            m02 += fx * p.dz;
+            m11 += fy * p.dy;
+            m12 += fy * p.dz;
+            m22 += fz * p.dz;
+            vx += Pj * fx;
+            vy += Pj * fy;
+            vz += Pj * fz;
+            ax += fx;
+            ay += fy;
+            az += fz;
+            pmin = min(pmin, __double_as_longlong(Pj));
+        });
+        mps_correct_particle(b, C, s, __longlong_as_double(pmin), m00, m01, m02, m11, m12, m22, vx, vy, vz, ax, ay, az);
+    }
+}
+
 __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_correct(MpsBufs b)
 {
+    if (!b.misc[5])
+        return;
     __shared__ int32_t nbuf[kMpsWarps][64];
     int32_t *buf = nbuf[threadIdx.x >> 5];
     const MpsConst &C = *b.c;
@@ -556,30 +849,8 @@ __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_correct(MpsBufs b)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             pmin = fmin(pmin, __shfl_xor_sync(0xffffffffu, pmin, o));
-        if ((threadIdx.x & 31) == 0) {
-            const double v0 = vx - pmin * ax, v1 = vy - pmin * ay, v2 = vz - pmin * az;
-            // M^{-1} v by the adjugate of the symmetric moment matrix
-            const double c00 = m11 * m22 - m12 * m12, c01 = m02 * m12 - m01 * m22, c02 = m01 * m12 - m02 * m11;
-            const double c11 = m00 * m22 - m02 * m02, c12 = m02 * m01 - m00 * m12, c22 = m00 * m11 - m01 * m01;
-            const double det = m00 * c00 + m01 * c01 + m02 * c02;
-            const double scale = (m00 + m11 + m22) / 3.0;
-            double gx = 0.0, gy = 0.0, gz = 0.0;
-            if (fabs(det) > 1e-12 * scale * scale * scale) {
-                gx = (c00 * v0 + c01 * v1 + c02 * v2) / det;
-                gy = (c01 * v0 + c11 * v1 + c12 * v2) / det;
-                gz = (c02 * v0 + c12 * v1 + c22 * v2) / det;
-            }
-            const int32_t id = b.perm[s];
-            const dvec4 us = b.ustar[id];
-            const double k = C.dt / C.rho;
-            const dvec4 un = make_dvec4(us.x - k * gx, us.y - k * gy, us.z - k * gz, 0.0);
-            b.vel[id] = un;
-            const dvec4 p = b.pos[id];
-            b.pos[id] = make_dvec4(p.x + C.dt * (un.x - us.x), p.y + C.dt * (un.y - us.y), p.z + C.dt * (un.z - us.z),
-                                   0.0);
-            if (!(un.x == un.x && un.y == un.y && un.z == un.z))
-                atomicOr(&b.misc[2], ST_UNSTABLE);
-        }
+        if ((threadIdx.x & 31) == 0)
+            mps_correct_particle(b, C, s, pmin, m00, m01, m02, m11, m12, m22, vx, vy, vz, ax, ay, az);
     }
 }
 
@@ -594,6 +865,20 @@ __global__ void k_mps_finish(MpsBufs b, int64_t N)
         if (b.key[id] == out)
             b.vel[id] = b.ustar[id];
         b.moved[id] = 0;
+    }
+}
+
+// Entries of each row of the last system whose columns are unknowns, into ptmp
+// (free between the cell lists).
+__global__ void k_mps_count(MpsBufs b, int32_t Ns)
+{
+    const int32_t n_in = b.misc[0];
+    for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < Ns; s += gridDim.x * blockDim.x) {
+        int n = 0;
+        const int cnt = s < n_in ? b.ecnt[s] : 0;
+        for (int k = 0; k < cnt; ++k)
+            n += !b.surf[b.ecol[row_entry(b.c->width, s, k)]];
+        b.ptmp[s] = n;
     }
 }
 
@@ -730,18 +1015,18 @@ size_t layout(MpsBufs &b, char *base, int64_t N, int32_t C, int width)
     b.spos = L.take<dvec4>(N);
     b.sposf = L.take<float4>(N);
     b.snd = L.take<double>(N);
-    b.ssig = L.take<double>(N);
+    b.ncan = L.take<int32_t>(N);
     b.surf = L.take<uint8_t>(N);
     b.ecnt = L.take<int32_t>(N);
-    b.ecol = L.take<int32_t>((size_t)N * width);
-    b.eval = L.take<double>((size_t)N * width);
+    b.ecol = L.take<int32_t>(((size_t)N + 31) / 32 * 32 * width);
+    b.eval = L.take<double>(((size_t)N + 31) / 32 * 32 * width);
     b.diag = L.take<double>(N);
     b.rhs = L.take<double>(N);
     b.x = L.take<double>(N);
     b.r = L.take<double>(N);
     b.p = L.take<double>(N);
     b.q = L.take<double>(N);
-    b.part = L.take<double>(kCgBlocks);
+    b.part = L.take<double>(2 * kCgMaxBlocks);
     b.scal = L.take<double>(8);
     b.cgi = L.take<int32_t>(4);
     b.c = L.take<MpsConst>(1);
@@ -788,8 +1073,12 @@ static int flat_grid(int64_t items)
     return (int)std::max<int64_t>(1, std::min<int64_t>((items + 255) / 256, (int64_t)sm_count() * 8));
 }
 
-// Cell list of the current positions.
-static void build_cells(mps_t *s)
+// One thread per particle, all of them resident or queued.
+static int row_grid(int64_t items) { return (int)std::max<int64_t>(1, (items + 255) / 256); }
+
+// Cell list of the current positions and the candidate lists (of every particle, or
+// of the fluid ones).
+static void build_cells(mps_t *s, bool fluid_only)
 {
     const int64_t N = s->g.N;
     const int32_t C = s->g.c.ncells;
@@ -801,6 +1090,8 @@ static void build_cells(mps_t *s)
     k_mps_scan_final<<<nb, kScanThreads, 0, s->st>>>(s->b, C);
     k_mps_scatter<<<flat_grid(N), 256, 0, s->st>>>(s->b, N);
     k_mps_sort<<<warp_grid(std::min<int64_t>(N, C)), 256, 0, s->st>>>(s->b);
+    cudaMemsetAsync(s->b.misc + 5, 0, sizeof(int32_t), s->st);
+    k_mps_list<<<row_grid(N), 256, 0, s->st>>>(s->b, fluid_only ? 1 : 0);
 }
 
 static void mark(mps_t *s, int k)
@@ -814,27 +1105,26 @@ static void mark(mps_t *s, int k)
 static int solve_pressure(mps_t *s)
 {
     const int64_t N = s->g.N;
-    const int32_t Ns = (int32_t)N;
+    k_mps_density_rows<<<row_grid(N), 256, 0, s->st>>>(s->b);
     k_mps_density<<<warp_grid(N), 256, 0, s->st>>>(s->b);
-    k_mps_assemble<<<warp_grid(N), 256, 0, s->st>>>(s->b, Ns);
+    k_mps_assemble<<<warp_grid(N), 256, 0, s->st>>>(s->b);
     mark(s, 2);
-    k_cg_init<<<kCgBlocks, kCgThreads, 0, s->st>>>(s->b, Ns);
-    k_cg_total<<<1, kCgThreads, 0, s->st>>>(s->b, 1, 1);
-    int32_t cgi[2] = {0, 0};
-    for (int it = 0; it < s->p.cg_max; it += kCgChunk) {
-        for (int k = 0; k < kCgChunk; ++k) {
-            k_cg_spmv<<<kCgBlocks, kCgThreads, 0, s->st>>>(s->b, Ns);
-            k_cg_total<<<1, kCgThreads, 0, s->st>>>(s->b, 2, 0);
-            k_cg_update<<<kCgBlocks, kCgThreads, 0, s->st>>>(s->b, Ns);
-            k_cg_total<<<1, kCgThreads, 0, s->st>>>(s->b, 3, 0);
-            k_cg_direction<<<kCgBlocks, kCgThreads, 0, s->st>>>(s->b, Ns);
-        }
-        MCK(cudaGetLastError());
-        MCK(cudaMemcpyAsync(cgi, s->b.cgi, sizeof(cgi), cudaMemcpyDeviceToHost, s->st));
-        MCK(cudaStreamSynchronize(s->st));
-        if (cgi[1])
-            break;
+    {
+        // every CTA resident (a cooperative launch), no more of them than rows to share
+        static int per_sm = 0;
+        if (!per_sm)
+            MCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg_solve, kCgThreads, 0));
+        if (per_sm < 1)
+            return mfail(s, SPH_ECUDA, "the CG kernel does not fit the device");
+        const int64_t most = std::min<int64_t>((int64_t)per_sm * sm_count(), kCgMaxBlocks);
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((N + kCgThreads - 1) / kCgThreads, most));
+        int cap = (int)std::min<int64_t>(((int64_t)s->p.cg_max + kCgChunk - 1) / kCgChunk * kCgChunk, 0x7fffffff);
+        void *args[] = {(void *)&s->b, &cap};
+        MCK(cudaMemsetAsync(s->b.cgi, 0, 4 * sizeof(int32_t), s->st));
+        MCK(cudaLaunchCooperativeKernel((const void *)k_cg_solve, grid, kCgThreads, args, 0, s->st));
     }
+    int32_t cgi[2] = {0, 0};
+    MCK(cudaMemcpyAsync(cgi, s->b.cgi, sizeof(cgi), cudaMemcpyDeviceToHost, s->st));
     double scal[2];
     int32_t misc[4];
     MCK(cudaMemcpyAsync(scal, s->b.scal, sizeof(scal), cudaMemcpyDeviceToHost, s->st));
@@ -842,6 +1132,8 @@ static int solve_pressure(mps_t *s)
     MCK(cudaStreamSynchronize(s->st));
     s->last_it = cgi[0];
     s->last_res = scal[1] > 0.0 ? std::sqrt(scal[0] / scal[1]) : 0.0;
+    if (misc[2] & ST_TIMEOUT)
+        return mfail(s, SPH_ETIMEOUT, "a bounded device wait ran out");
     if (misc[2] & ST_OVERFLOW)
         return mfail(s, SPH_ESTATE, "a row of the pressure system has more entries than row_width");
     if (!cgi[1] || !(s->last_res <= s->p.cg_tol))
@@ -996,15 +1288,17 @@ int mps_step(mps_t *s, int32_t nsteps)
     const int64_t N = s->g.N;
     for (int32_t k = 0; k < nsteps; ++k) {
         mark(s, 0);
-        build_cells(s);
+        build_cells(s, true);
+        k_mps_predict_rows<<<row_grid(N), 256, 0, s->st>>>(s->b);
         k_mps_predict<<<warp_grid(N), 256, 0, s->st>>>(s->b);
-        build_cells(s);
+        build_cells(s, false);
         mark(s, 1);
         int rc = solve_pressure(s);
         if (rc)
             return rc;
         mark(s, 3);
         k_mps_clamp<<<flat_grid(N), 256, 0, s->st>>>(s->b, (int32_t)N);
+        k_mps_correct_rows<<<row_grid(N), 256, 0, s->st>>>(s->b);
         k_mps_correct<<<warp_grid(N), 256, 0, s->st>>>(s->b);
         k_mps_finish<<<flat_grid(N), 256, 0, s->st>>>(s->b, N);
         mark(s, 4);
@@ -1032,7 +1326,7 @@ int mps_pressure(mps_t *s, double *P, double *nd, int32_t *surf, int64_t *iterat
     if (!s)
         return SPH_EINVAL;
     const int64_t N = s->g.N;
-    build_cells(s);
+    build_cells(s, false);
     int rc = solve_pressure(s);
     if (rc)
         return rc;
@@ -1141,8 +1435,11 @@ int mps_system_size(mps_t *s, int64_t out[2])
     if (!s || !out)
         return SPH_EINVAL;
     const int64_t N = s->g.N;
+    // the rows may hold columns of free-surface particles, which are no unknowns
+    k_mps_count<<<row_grid(N), 256, 0, s->st>>>(s->b, (int32_t)N);
+    MCK(cudaGetLastError());
     std::vector<int32_t> cnt((size_t)N);
-    MCK(cudaMemcpyAsync(cnt.data(), s->b.ecnt, sizeof(int32_t) * (size_t)N, cudaMemcpyDeviceToHost, s->st));
+    MCK(cudaMemcpyAsync(cnt.data(), s->b.ptmp, sizeof(int32_t) * (size_t)N, cudaMemcpyDeviceToHost, s->st));
     MCK(cudaStreamSynchronize(s->st));
     int64_t nnz = 0;
     for (int64_t i = 0; i < N; ++i)
