@@ -587,27 +587,31 @@ __device__ __forceinline__ bool cg_barrier(MpsBufs &b, unsigned &target, int *s_
     __syncthreads();
     target += gridDim.x;
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&b.cgi[2], 1);
-        int polls = 0;
+        unsigned *bar = reinterpret_cast<unsigned *>(&b.cgi[2]);
+        // the release makes the CTA's writes before its barrier visible, the acquire
+        // those of the others to the CTA after its own
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
         bool ok = true;
-        // (the counter may wrap)
-        while ((int)(*(volatile unsigned *)&b.cgi[2] - target) < 0) {
-            if (++polls > kCgSpin) {
+        for (int polls = 0;; ++polls) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if ((int)(v - target) >= 0)  // (the counter may wrap)
+                break;
+            if (polls > kCgSpin) {
                 atomicOr(&b.misc[2], ST_TIMEOUT);
                 ok = false;
                 break;
             }
-            __nanosleep(20);
+            if (polls > 64)
+                __nanosleep(20);
         }
-        __threadfence();
         *s_ok = ok;
     }
     __syncthreads();
     return *s_ok != 0;
 }
 
-__global__ void __launch_bounds__(kCgThreads) k_cg_solve(MpsBufs b, int max_iterations)
+__global__ void __launch_bounds__(kCgThreads, 3) k_cg_solve(MpsBufs b, int max_iterations)
 {
     const int width = b.c->width;
     __shared__ double sh[kCgThreads / 32];
@@ -654,25 +658,30 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_solve(MpsBufs b, int max_iter
             const int64_t e0 = row_entry(width, i, 0);
             const double *ev = b.eval + e0;
             const int32_t *ec = b.ecol + e0;
-            int k = 0;
-            for (; k + 8 <= cnt; k += 8) {
-                double v[8], g[8];
-                int32_t c[8];
+            // eight entries at a time, the next eight on their way while the p of these
+            // are gathered; past the end a zero coefficient
+            double v[8], g[8];
+            int32_t c[8];
+            auto load = [&](int k) {
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    c[u] = __ldcs(ec + 32 * (k + u));
+                for (int u = 0; u < 8; ++u) {
+                    c[u] = k + u < cnt ? __ldcs(ec + 32 * (k + u)) : i;
+                    v[u] = k + u < cnt ? __ldcs(ev + 32 * (k + u)) : 0.0;
+                }
+            };
+            load(0);
+            for (int k = 0; k < cnt; k += 8) {
+                double w[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    v[u] = __ldcs(ev + 32 * (k + u));
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
+                for (int u = 0; u < 8; ++u) {
                     g[u] = b.p[c[u]];
+                    w[u] = v[u];
+                }
+                load(k + 8);
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
-                    s += v[u] * g[u];
+                    s += w[u] * g[u];
             }
-            for (; k < cnt; ++k)
-                s += __ldcs(ev + 32 * k) * b.p[__ldcs(ec + 32 * k)];
             b.q[i] = s;
             pq += pi * s;
         }
@@ -680,11 +689,27 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_solve(MpsBufs b, int max_iter
             return;
         const double alpha = rho / pq;
         double rr = 0.0;
-        for (int32_t i = i0; i < n_in; i += stride) {
-            b.x[i] += alpha * b.p[i];
-            const double ri = b.r[i] - alpha * b.q[i];
-            b.r[i] = ri;
-            rr += ri * ri;
+        for (int32_t i = i0; i < n_in; i += 4 * stride) {  // four rows in flight
+            double x[4], p[4], r[4], q[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int32_t iu = i + u * stride;
+                const bool on = iu < n_in;
+                x[u] = on ? b.x[iu] : 0.0;
+                p[u] = on ? b.p[iu] : 0.0;
+                r[u] = on ? b.r[iu] : 0.0;
+                q[u] = on ? b.q[iu] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int32_t iu = i + u * stride;
+                const double ri = r[u] - alpha * q[u];
+                if (iu < n_in) {
+                    b.x[iu] = x[u] + alpha * p[u];
+                    b.r[iu] = ri;
+                }
+                rr += ri * ri;
+            }
         }
         if (!total(rr, rr))
             return;
@@ -694,8 +719,19 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_solve(MpsBufs b, int max_iter
         done = sqrt(rr) <= b.c->tol * sqrt(bb) || !(rr == rr);
         if (done)
             break;
-        for (int32_t i = i0; i < n_in; i += stride)
-            b.p[i] = b.r[i] + beta * b.p[i];
+        for (int32_t i = i0; i < n_in; i += 4 * stride) {
+            double p[4], r[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int32_t iu = i + u * stride;
+                p[u] = iu < n_in ? b.p[iu] : 0.0;
+                r[u] = iu < n_in ? b.r[iu] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i + u * stride < n_in)
+                    b.p[i + u * stride] = r[u] + beta * p[u];
+        }
         if (!cg_barrier(b, target, &s_ok))
             return;
     }
