@@ -11,21 +11,25 @@
 
 namespace sph {
 
+// Cell along one axis from the coordinate in cells; false outside [0, n).  One FP64
+// conversion (rounding down) instead of a floor, two comparisons and a conversion:
+// the kernels that bin every particle are bound by the FP64 pipe (mixed update of
+// 0.9 M particles 69 -> 54 us, of 1.77 M 140 -> 107 us).  The conversion saturates;
+// a NaN, which it would turn into 0, is told by its bits.
+__device__ __forceinline__ bool cell_of(double f, int n, int &c)
+{
+    c = __double2int_rd(f);
+    return (unsigned)c < (unsigned)n && (__double2hiint(f) & 0x7ff00000) != 0x7ff00000;
+}
+
 // Cell coordinates with the exact IEEE division (x - lo) / cs, as the
 // definition of the grid states it; false when outside the grid.
 __device__ __forceinline__ bool cell_coords_exact(const Inst &I, double x, double y, double z, int &cx, int &cy,
                                                   int &cz)
 {
-    double fx = floor((x - I.lo[0]) / I.cs);
-    double fy = floor((y - I.lo[1]) / I.cs);
-    double fz = floor((z - I.lo[2]) / I.cs);
-    if (!(fx >= 0.0) || fx >= (double)I.n[0] || !(fy >= 0.0) || fy >= (double)I.n[1] || !(fz >= 0.0) ||
-        fz >= (double)I.n[2])
-        return false;
-    cx = (int)fx;
-    cy = (int)fy;
-    cz = (int)fz;
-    return true;
+    const bool ix = cell_of((x - I.lo[0]) / I.cs, I.n[0], cx), iy = cell_of((y - I.lo[1]) / I.cs, I.n[1], cy),
+               iz = cell_of((z - I.lo[2]) / I.cs, I.n[2], cz);
+    return ix && iy && iz;
 }
 
 // The same with a multiplication by 1/cs (mixed form: cell assignment only
@@ -33,16 +37,9 @@ __device__ __forceinline__ bool cell_coords_exact(const Inst &I, double x, doubl
 __device__ __forceinline__ bool cell_coords_fast(const Inst &I, double x, double y, double z, int &cx, int &cy,
                                                  int &cz)
 {
-    double fx = floor((x - I.lo[0]) * I.inv_cs);
-    double fy = floor((y - I.lo[1]) * I.inv_cs);
-    double fz = floor((z - I.lo[2]) * I.inv_cs);
-    if (!(fx >= 0.0) || fx >= (double)I.n[0] || !(fy >= 0.0) || fy >= (double)I.n[1] || !(fz >= 0.0) ||
-        fz >= (double)I.n[2])
-        return false;
-    cx = (int)fx;
-    cy = (int)fy;
-    cz = (int)fz;
-    return true;
+    const bool ix = cell_of((x - I.lo[0]) * I.inv_cs, I.n[0], cx), iy = cell_of((y - I.lo[1]) * I.inv_cs, I.n[1], cy),
+               iz = cell_of((z - I.lo[2]) * I.inv_cs, I.n[2], cz);
+    return ix && iy && iz;
 }
 
 // x offset of a particle from the origin of its cell (mixed form).
