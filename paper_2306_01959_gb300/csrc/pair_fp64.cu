@@ -121,10 +121,37 @@ __device__ __forceinline__ long long fixed_t3(unsigned long long R, unsigned lon
     return (long long)__umul64hi(__umul64hi(t1, t1) << 1, t1);
 }
 
+// 1 / (V d) for an integer 2^49 <= V < 2^63 and d = (1 + f) 2^(ex - 1023), ex in [128, 1792),
+// from d's bits: the product of the two mantissas, W in [1/4, 1), its reciprocal by
+// one third-order step from the FP32 approximation (as rcp3), rounded once.  Error
+// 1.11e-16, against 2.8e-16 for the FP64 operations it replaces (a conversion, a
+// product and three more).
+__device__ __forceinline__ double fixed_rcp(unsigned long long V, double d)
+{
+    const int ex = __double2hiint(d) >> 20;
+    const int n = __clzll((long long)V);
+    const unsigned long long m = ((unsigned long long)__double_as_longlong(d) << 11) | 1ull << 63;
+    const unsigned long long w = __umul64hi(V << n, m);  // W, 64 fraction bits
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((float)(unsigned)(w >> 32)));
+    const unsigned Y = __float2uint_rz(y * 4611686018427387904.f);  // 2^30 / W, saturating
+    const long long E = (1ll << 62) - (long long)((w >> 32) * Y + __umulhi((unsigned)w, Y));  // 1 - W Y
+    const int e = (int)(E >> 12);
+    const long long g = E + (((long long)e * e) >> 38);  // E + E^2
+    const unsigned long long z = ((unsigned long long)Y << 31) +
+                                 (unsigned long long)(__mul64hi((long long)Y << 30, g << 21) >> 18);  // 2^61 / W
+    const int k = __clzll((long long)z);
+    const unsigned long long u = z << k;
+    return __longlong_as_double((long long)((u >> 11) + ((u >> 10) & 1) +
+                                            ((unsigned long long)(1085 - k + n + 897 - ex) << 52)));
+}
+
 // Geometry of a pair: r_ij, |r_ij|^2 + eta^2 and t^3, in the units of k.  The
-// positions are doubles, or (FIX) 64-bit integers in the same registers.
+// positions are doubles, or (FIX) 64-bit integers in the same registers, and so is
+// |r_ij|^2 + eta^2 (V in place of re).
 struct PairGeoD {
     double rx, ry, rz, re, t3;
+    unsigned long long V;
 };
 template <bool FIX>
 __device__ __forceinline__ PairGeoD pair_geo_d(const PairConstD &k, double xi, double yi, double zi, double xj,
@@ -143,13 +170,13 @@ __device__ __forceinline__ PairGeoD pair_geo_d(const PairConstD &k, double xi, d
         p.ry = int_to_double(dy);
         p.rz = int_to_double(dz);
         if (R >= (1ull << 48)) {
-            p.re = int_to_double((long long)(R + k.eta));
+            p.V = R + k.eta;
             // (a pair just within 2h can round to 2h, at most 2^62)
             p.t3 = int_to_double(fixed_t3(min(R, (1ull << 62) - 1), k.kh));
         } else {
             const double r2 = p.rx * p.rx + p.ry * p.ry + p.rz * p.rz;
             const double t = 1.0 - sqrt3(r2) * k.half_inv_h;
-            p.re = fma(r2, 0x1p-44, k.eta2);
+            p.V = (unsigned long long)__double2ll_rn(fma(r2, 0x1p-44, k.eta2));
             p.t3 = t * t * t * 0x1p62;
         }
     } else {
@@ -162,6 +189,18 @@ __device__ __forceinline__ PairGeoD pair_geo_d(const PairConstD &k, double xi, d
         p.t3 = t * t * t;  // m_j F / (-kF m)
     }
     return p;
+}
+
+// 1 / ((|r_ij|^2 + eta^2) (rho_i + rho_j)).
+template <bool FIX>
+__device__ __forceinline__ double pair_rcp(const PairGeoD &p, double rsum)
+{
+    if (!FIX)
+        return rcp3(p.re * rsum);
+    // densities whose sum is not positive, or no number, take the FP64 operations
+    if ((unsigned)((__double2hiint(rsum) >> 20) - 128) < 1664u)
+        return fixed_rcp(p.V, rsum);
+    return rcp3(int_to_double((long long)p.V) * rsum);
 }
 
 // Contribution of neighbour j to particle i (Eqs. 3-7), in double.
@@ -199,11 +238,13 @@ __device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, doub
     // Eqs. 4-5: Pi_ij = -alpha c_bar mu / rho_bar, c_bar / rho_bar = (c_i + c_j) / (rho_i + rho_j),
     // mu = h (u_ij . r_ij) / (|r_ij|^2 + eta^2) = h muh, muh = mur (rho_i + rho_j)
     double rsum = rhoi + rhoj;
-    double mur = udotr * rcp3(p.re * rsum);
-    double muh = mur * rsum;
-    double visc = 0.0;
-    if (__double2hiint(udotr) < 0)  // u_ij . r_ij < 0 (a -0.0 gives a zero term)
-        visc = fma(k.nah, cj, k.nah * ci) * mur;
+    double mur = udotr * pair_rcp<FIX>(p, rsum);
+    // u_ij . r_ij < 0 (a -0.0 gives a zero term): the viscosity; else muh, whose
+    // maximum starts at 0: one product for both
+    const bool app = __double2hiint(udotr) < 0;
+    const double cs = fma(k.nah, cj, k.nah * ci);
+    const double prod = mur * (app ? cs : rsum);
+    const double visc = app ? prod : 0.0, muh = app ? 0.0 : prod;
     // Eq. 3: a_i -= m_j (...) grad_i W_ij = m_j (...) F r_ij, with
     // (P_i + P_j) / (rho_i rho_j) = (P_i / rho_i + P_j / rho_i) / rho_j
     double coef = fma(fma(Pj, inv_rhoi, Pi * inv_rhoi), inv_rhoj, visc) * t3;
@@ -237,11 +278,11 @@ __device__ __forceinline__ void pair_share_j(const PairConstD &k, double xi, dou
     double gj = ff ? fma(-k.dfac * rhoj, inv_rhoi, k.dfac) : 0.0;
     a.drho = fma(t3, udotr - g, a.drho);
     double rsum = rhoi + rhoj;
-    double mur = udotr * rcp3(p.re * rsum);
-    double muh = mur * rsum;
-    double visc = 0.0;
-    if (__double2hiint(udotr) < 0)
-        visc = fma(k.nah, cj, k.nah * ci) * mur;
+    double mur = udotr * pair_rcp<FIX>(p, rsum);
+    const bool app = __double2hiint(udotr) < 0;
+    const double cs = fma(k.nah, cj, k.nah * ci);
+    const double prod = mur * (app ? cs : rsum);
+    const double visc = app ? prod : 0.0, muh = app ? 0.0 : prod;
     double coef = fma(fma(Pj, inv_rhoi, Pi * inv_rhoi), inv_rhoj, visc) * t3;
     a.ax += coef * rx;
     a.ay += coef * ry;
