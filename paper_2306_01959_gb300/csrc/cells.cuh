@@ -219,7 +219,7 @@ __device__ __forceinline__ void sort_reorder_range(const Bufs &b, int32_t ninst,
                      : make_dvec4(p.x, p.y, p.z, v.w);
             reinterpret_cast<dvec4 *>(b.sB)[s] = make_dvec4(v.x, v.y, v.z, tait_d(I, v.w));
             b.sC[s] = make_double2(1.0 / v.w, sound_d(I, v.w));
-            b.sD[s] = make_float4((float)p.x, (float)p.y, (float)p.z, 0.f);
+            b.sD[s] = make_float4((float)p.x, (float)p.y, (float)p.z, type == T_FLUID ? 1.f : 0.f);
         } else {
             const float4 v = reinterpret_cast<const float4 *>(b.vel)[id];
             // offsets from the origin of the cell

@@ -106,7 +106,7 @@ struct Bufs {
     void *sA;                // FP64: dvec4 (x, y, z, rho), x, y, z the bits of 64-bit integers with Inst::fx; mixed: float4 (offset to cell origin, rho - rho0)
     void *sB;                // FP64: dvec4 (u, P); mixed: float4 (u, P)
     double2 *sC;             // FP64 form: (1 / rho, c) per sorted particle; unused by the mixed form
-    float4 *sD;              // FP64 form: FP32 copies of the sorted positions, for the pre-test
+    float4 *sD;              // FP64 form: FP32 copies of the sorted positions, for the pre-test; w: 1 for fluid
     uint8_t *sflag;          // type per sorted index
     // pair outputs (sorted)
     void *deriv;             // FP64: dvec4 (a, Drho); mixed: float4

@@ -30,15 +30,28 @@ struct AccD {
 
 // Constants of an instance used by every pair.
 struct PairConstD {
-    double half_inv_h, dfac, nah, eta2;  // dfac = 2 delta h c0, nah = -alpha h
+    double half_inv_h, eta2, dfac, nah;  // dfac = 2 delta h c0, nah = -alpha h
     unsigned long long kh, eta;          // fixed-point positions only
 };
 
 template <bool FIX>
 __device__ __forceinline__ PairConstD pair_const_d(const Inst &I)
 {
-    return FIX ? PairConstD{I.fx_hinv, I.fx_dfac, I.fx_nah, (double)I.fx_eta, I.fx_kh, I.fx_eta}
-               : PairConstD{I.half_inv_h, I.dfac_d, I.nah, I.eta2, 0ull, 0ull};
+    return FIX ? PairConstD{I.fx_hinv, (double)I.fx_eta, I.fx_dfac, I.fx_nah, I.fx_kh, I.fx_eta}
+               : PairConstD{I.half_inv_h, I.eta2, I.dfac_d, I.nah, 0ull, 0ull};
+}
+
+// Particle i of a pair, with the products that all its pairs share, and the constants.
+struct __align__(16) OwnD {
+    double x, y, z, rho;
+    double ux, uy, uz, inv_rho;
+    double drho, prho, nac;  // -dfac rho, P / rho, nah c
+    PairConstD k;
+};
+__device__ __forceinline__ OwnD own_d(const PairConstD &k, double x, double y, double z, double ux, double uy,
+                                      double uz, double rho, double inv_rho, double P, double c)
+{
+    return OwnD{x, y, z, rho, ux, uy, uz, inv_rho, -k.dfac * rho, P * inv_rho, k.nah * c, k};
 }
 
 // The FP64 pipe of this GPU issues one warp operation every 64 cycles per
@@ -154,14 +167,13 @@ struct PairGeoD {
     unsigned long long V;
 };
 template <bool FIX>
-__device__ __forceinline__ PairGeoD pair_geo_d(const PairConstD &k, double xi, double yi, double zi, double xj,
-                                               double yj, double zj)
+__device__ __forceinline__ PairGeoD pair_geo_d(const OwnD &o, double xj, double yj, double zj)
 {
     PairGeoD p;
     if (FIX) {
-        const long long dx = __double_as_longlong(xj) - __double_as_longlong(xi);
-        const long long dy = __double_as_longlong(yj) - __double_as_longlong(yi);
-        const long long dz = __double_as_longlong(zj) - __double_as_longlong(zi);
+        const long long dx = __double_as_longlong(xj) - __double_as_longlong(o.x);
+        const long long dy = __double_as_longlong(yj) - __double_as_longlong(o.y);
+        const long long dz = __double_as_longlong(zj) - __double_as_longlong(o.z);
         const unsigned long long ax = (unsigned long long)(dx < 0 ? -dx : dx) << 10;
         const unsigned long long ay = (unsigned long long)(dy < 0 ? -dy : dy) << 10;
         const unsigned long long az = (unsigned long long)(dz < 0 ? -dz : dz) << 10;
@@ -170,22 +182,22 @@ __device__ __forceinline__ PairGeoD pair_geo_d(const PairConstD &k, double xi, d
         p.ry = int_to_double(dy);
         p.rz = int_to_double(dz);
         if (R >= (1ull << 48)) {
-            p.V = R + k.eta;
+            p.V = R + o.k.eta;
             // (a pair just within 2h can round to 2h, at most 2^62)
-            p.t3 = int_to_double(fixed_t3(min(R, (1ull << 62) - 1), k.kh));
+            p.t3 = int_to_double(fixed_t3(min(R, (1ull << 62) - 1), o.k.kh));
         } else {
             const double r2 = p.rx * p.rx + p.ry * p.ry + p.rz * p.rz;
-            const double t = 1.0 - sqrt3(r2) * k.half_inv_h;
-            p.V = (unsigned long long)__double2ll_rn(fma(r2, 0x1p-44, k.eta2));
+            const double t = 1.0 - sqrt3(r2) * o.k.half_inv_h;
+            p.V = (unsigned long long)__double2ll_rn(fma(r2, 0x1p-44, o.k.eta2));
             p.t3 = t * t * t * 0x1p62;
         }
     } else {
-        p.rx = xj - xi;
-        p.ry = yj - yi;
-        p.rz = zj - zi;
+        p.rx = xj - o.x;
+        p.ry = yj - o.y;
+        p.rz = zj - o.z;
         const double r2 = p.rx * p.rx + p.ry * p.ry + p.rz * p.rz;
-        const double t = 1.0 - sqrt3(r2) * k.half_inv_h;
-        p.re = r2 + k.eta2;
+        const double t = 1.0 - sqrt3(r2) * o.k.half_inv_h;
+        p.re = r2 + o.k.eta2;
         p.t3 = t * t * t;  // m_j F / (-kF m)
     }
     return p;
@@ -215,20 +227,18 @@ __device__ __forceinline__ double pair_rcp(const PairGeoD &p, double rsum)
 // delta term is summed apart (the caller drops it for a fluid particle that
 // has a boundary neighbour).
 template <bool DFS, bool FIX>
-__device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, double yi, double zi, double uxi,
-                                            double uyi, double uzi, double rhoi, double inv_rhoi, double Pi,
-                                            double ci, bool fluid_i, double xj, double yj, double zj, double uxj,
+__device__ __forceinline__ void pair_term_d(const OwnD &o, bool fluid_i, double xj, double yj, double zj, double uxj,
                                             double uyj, double uzj, double rhoj, double inv_rhoj, double Pj,
                                             double cj, bool fluid_j, AccD &a)
 {
-    const PairGeoD p = pair_geo_d<FIX>(k, xi, yi, zi, xj, yj, zj);
+    const PairGeoD p = pair_geo_d<FIX>(o, xj, yj, zj);
     const double rx = p.rx, ry = p.ry, rz = p.rz, t3 = p.t3;  // r_ij = r_j - r_i; grad_i W_ij = F (r_i - r_j) = -F r_ij
-    double ux = uxj - uxi, uy = uyj - uyi, uz = uzj - uzi;  // u_ij = u_j - u_i
+    double ux = uxj - o.ux, uy = uyj - o.uy, uz = uzj - o.uz;  // u_ij = u_j - u_i
     double udotr = ux * rx + uy * ry + uz * rz;  // u_ij . r_ij
     // Eq. 7: sum_j m_j (u_i - u_j) . grad_i W_ij = m_j F (u_ij . r_ij), plus the delta term
     // 2 delta h c0 (rho_j - rho_i) (r_ij . grad_i W_ij) / |r_ij|^2 m_j / rho_j, where
     // (r_ij . grad_i W_ij) / |r_ij|^2 = -F and (rho_j - rho_i) / rho_j = 1 - rho_i / rho_j
-    double g = (fluid_i && fluid_j) ? fma(-k.dfac * rhoi, inv_rhoj, k.dfac) : 0.0;
+    double g = (fluid_i && fluid_j) ? fma(o.drho, inv_rhoj, o.k.dfac) : 0.0;
     if (DFS) {
         a.drho = fma(t3, udotr, a.drho);
         a.dd = fma(t3, g, a.dd);
@@ -237,17 +247,17 @@ __device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, doub
     }
     // Eqs. 4-5: Pi_ij = -alpha c_bar mu / rho_bar, c_bar / rho_bar = (c_i + c_j) / (rho_i + rho_j),
     // mu = h (u_ij . r_ij) / (|r_ij|^2 + eta^2) = h muh, muh = mur (rho_i + rho_j)
-    double rsum = rhoi + rhoj;
+    double rsum = o.rho + rhoj;
     double mur = udotr * pair_rcp<FIX>(p, rsum);
     // u_ij . r_ij < 0 (a -0.0 gives a zero term): the viscosity; else muh, whose
     // maximum starts at 0: one product for both
     const bool app = __double2hiint(udotr) < 0;
-    const double cs = fma(k.nah, cj, k.nah * ci);
+    const double cs = fma(o.k.nah, cj, o.nac);
     const double prod = mur * (app ? cs : rsum);
     const double visc = app ? prod : 0.0, muh = app ? 0.0 : prod;
     // Eq. 3: a_i -= m_j (...) grad_i W_ij = m_j (...) F r_ij, with
     // (P_i + P_j) / (rho_i rho_j) = (P_i / rho_i + P_j / rho_i) / rho_j
-    double coef = fma(fma(Pj, inv_rhoi, Pi * inv_rhoi), inv_rhoj, visc) * t3;
+    double coef = fma(fma(Pj, o.inv_rho, o.prho), inv_rhoj, visc) * t3;
     a.ax += coef * rx;
     a.ay += coef * ry;
     a.az += coef * rz;
@@ -262,28 +272,26 @@ __device__ __forceinline__ void pair_term_d(const PairConstD &k, double xi, doub
 // 2 delta h c0 (1 - rho_j / rho_i), mu is the same; units as pair_term_d
 // (t^3 in place of m F, mu / h).  i's own share is accumulated in a.
 template <bool FIX>
-__device__ __forceinline__ void pair_share_j(const PairConstD &k, double xi, double yi, double zi, double uxi,
-                                             double uyi, double uzi, double rhoi, double inv_rhoi, double Pi,
-                                             double ci, bool fluid_i, double xj, double yj, double zj, double uxj,
+__device__ __forceinline__ void pair_share_j(const OwnD &o, bool fluid_i, double xj, double yj, double zj, double uxj,
                                              double uyj, double uzj, double rhoj, double inv_rhoj, double Pj,
                                              double cj, bool fluid_j, dvec4 *jacc, long long *jmu, int32_t j,
                                              AccD &a)
 {
-    const PairGeoD p = pair_geo_d<FIX>(k, xi, yi, zi, xj, yj, zj);
+    const PairGeoD p = pair_geo_d<FIX>(o, xj, yj, zj);
     const double rx = p.rx, ry = p.ry, rz = p.rz, t3 = p.t3;
-    double ux = uxj - uxi, uy = uyj - uyi, uz = uzj - uzi;
+    double ux = uxj - o.ux, uy = uyj - o.uy, uz = uzj - o.uz;
     double udotr = ux * rx + uy * ry + uz * rz;
     const bool ff = fluid_i && fluid_j;
-    double g = ff ? fma(-k.dfac * rhoi, inv_rhoj, k.dfac) : 0.0;
-    double gj = ff ? fma(-k.dfac * rhoj, inv_rhoi, k.dfac) : 0.0;
+    double g = ff ? fma(o.drho, inv_rhoj, o.k.dfac) : 0.0;
+    double gj = ff ? fma(-o.k.dfac * rhoj, o.inv_rho, o.k.dfac) : 0.0;
     a.drho = fma(t3, udotr - g, a.drho);
-    double rsum = rhoi + rhoj;
+    double rsum = o.rho + rhoj;
     double mur = udotr * pair_rcp<FIX>(p, rsum);
     const bool app = __double2hiint(udotr) < 0;
-    const double cs = fma(k.nah, cj, k.nah * ci);
+    const double cs = fma(o.k.nah, cj, o.nac);
     const double prod = mur * (app ? cs : rsum);
     const double visc = app ? prod : 0.0, muh = app ? 0.0 : prod;
-    double coef = fma(fma(Pj, inv_rhoi, Pi * inv_rhoi), inv_rhoj, visc) * t3;
+    double coef = fma(fma(Pj, o.inv_rho, o.prho), inv_rhoj, visc) * t3;
     a.ax += coef * rx;
     a.ay += coef * ry;
     a.az += coef * rz;
@@ -309,13 +317,19 @@ __device__ __forceinline__ double dist2_rn(double xi, double yi, double zi, doub
 // CNT (with SYM): also count the partners' neighbours (nneigh is read by
 // sph_derivatives and the work counts, not by a time step).
 // FIX: fixed-point sorted positions.
+// No unit is full (FP64 pipe about 70 %, of the 84 % that FMAs alone reach): the
+// gathers and the serial integer chains of a batch are covered by warps, so what
+// the lanes of a warp share lies in shared memory and 24 warps of 80 registers fit
+// on an SM instead of 16 of 124.  0.9 M particles: 12.5 -> 10.7 ms, 11 k: 200 -> 163 us
+// (the register bound alone 12.6 ms and 186 us).
 template <bool FIX, bool DFS, bool SYM, bool CNT = true>
-__global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
+__global__ void __launch_bounds__(256, 3) k_pair_fp64(Bufs b, int ninst, int kdiv)
 {
     extern __shared__ int32_t smem_q[];
+    __shared__ OwnD own[8];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    int32_t *q = smem_q + wib * kQ;
+    int32_t *q = smem_q + wib * kQ;  // neighbours; the sign bit marks a fluid particle
     const unsigned lt = (1u << lane) - 1u;
     const int32_t n_in = b.misc[0];
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -327,11 +341,14 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
         const Inst &I = b.inst[inst_of_cell(b.inst, ninst, ci_cell)];
         int cx, cy, cz;
         decompose(I, ci_cell, cx, cy, cz);
-        const dvec4 Ai = sA[i], Bi = sB[i];
-        const double2 Ci = b.sC[i];
         const float4 Di = b.sD[i];
-        const bool fluid_i = b.sflag[i] == T_FLUID;
-        const PairConstD kc = pair_const_d<FIX>(I);
+        const bool fluid_i = Di.w != 0.f;
+        if (lane == 0) {
+            const dvec4 A = sA[i], B = sB[i];
+            const double2 C = b.sC[i];
+            own[wib] = own_d(pair_const_d<FIX>(I), A.x, A.y, A.z, B.x, B.y, B.z, A.w, C.x, B.w, C.y);
+        }
+        __syncwarp();
         AccD acc = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
         bool touches_boundary = false;  // DFS: some neighbour j is a boundary particle
         int nn = 0;
@@ -340,16 +357,16 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
 
         auto flush = [&](int cnt) {
             if (lane < cnt) {
-                int32_t j = q[lane];
-                dvec4 Aj = sA[j], Bj = sB[j];
-                double2 Cj = b.sC[j];
+                const int32_t qj = q[lane], j = qj & 0x7fffffff;
+                const bool fluid_j = qj < 0;
+                const dvec4 Aj = sA[j], Bj = sB[j];
+                const double2 Cj = b.sC[j];
                 if (SYM)
-                    pair_share_j<FIX>(kc, Ai.x, Ai.y, Ai.z, Bi.x, Bi.y, Bi.z, Ai.w, Ci.x, Bi.w, Ci.y, fluid_i, Aj.x, Aj.y,
-                                 Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, b.sflag[j] == T_FLUID, b.fjacc, b.fjmu,
-                                 j, acc);
+                    pair_share_j<FIX>(own[wib], fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, fluid_j,
+                                      b.fjacc, b.fjmu, j, acc);
                 else
-                    pair_term_d<DFS, FIX>(kc, Ai.x, Ai.y, Ai.z, Bi.x, Bi.y, Bi.z, Ai.w, Ci.x, Bi.w, Ci.y, fluid_i, Aj.x,
-                                     Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, b.sflag[j] == T_FLUID, acc);
+                    pair_term_d<DFS, FIX>(own[wib], fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y,
+                                          fluid_j, acc);
             }
         };
 
@@ -368,7 +385,7 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
                     s0 = i + 1;  // the home row from the home cell on (cells hold ascending ids), after i
                 for (int32_t base = s0; base < s1; base += 32) {
                     int32_t j = base + lane;
-                    bool take = false;
+                    bool take = false, fluid_j = false;
                     if (j < s1 && j != i) {
                         // FP32 pre-test with radii that cover every rounding of the
                         // FP32 copies: certainly inside, certainly outside, or (in a
@@ -385,7 +402,7 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
                             ++nn;
                             if (SYM && CNT)
                                 atomicAdd(b.fjnn + j, 1);
-                            const bool fluid_j = b.sflag[j] == T_FLUID;
+                            fluid_j = Dj.w != 0.f;
                             take = fluid_i || fluid_j;
                             if (DFS)
                                 touches_boundary = touches_boundary || !fluid_j;
@@ -393,7 +410,7 @@ __global__ void __launch_bounds__(256) k_pair_fp64(Bufs b, int ninst, int kdiv)
                     }
                     unsigned m = __ballot_sync(0xffffffffu, take);
                     if (take)
-                        q[qn + __popc(m & lt)] = j;
+                        q[qn + __popc(m & lt)] = fluid_j ? j | (int32_t)0x80000000 : j;
                     qn += __popc(m);
                     npair += __popc(m);
                     ncand += min(32, s1 - base);
@@ -540,7 +557,8 @@ __global__ void k_probe_force(Bufs b, int inst, int kdiv)
         double xb, yb, zb, uxb, uyb, uzb, rhob;
         load_state<MODE>(b, I, idb, xb, yb, zb, uxb, uyb, uzb, rhob);
         double Pb = tait_d(I, rhob), cb = sound_d(I, rhob);
-        const PairConstD kc = pair_const_d<false>(I);
+        const OwnD own =
+            own_d(pair_const_d<false>(I), xb, yb, zb, uxb, uyb, uzb, rhob, 1.0 / rhob, Pb, cb);
         int cx, cy, cz;
         decompose(I, b.scell[s], cx, cy, cz);
         AccD acc = {0, 0, 0, 0, 0};
@@ -562,8 +580,8 @@ __global__ void k_probe_force(Bufs b, int inst, int kdiv)
                     double xj, yj, zj, uxj, uyj, uzj, rhoj;
                     load_state<MODE>(b, I, idj, xj, yj, zj, uxj, uyj, uzj, rhoj);
                     if (dist2_rn(xb, yb, zb, xj, yj, zj) < I.sup2)
-                        pair_term_d<false, false>(kc, xb, yb, zb, uxb, uyb, uzb, rhob, 1.0 / rhob, Pb, cb, false, xj, yj, zj, uxj,
-                                    uyj, uzj, rhoj, 1.0 / rhoj, tait_d(I, rhoj), sound_d(I, rhoj), true, acc);
+                        pair_term_d<false, false>(own, false, xj, yj, zj, uxj, uyj, uzj, rhoj, 1.0 / rhoj,
+                                                  tait_d(I, rhoj), sound_d(I, rhoj), true, acc);
                 }
             }
         }
