@@ -311,24 +311,37 @@ __device__ __forceinline__ double dist2_rn(double xi, double yi, double zi, doub
     return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
+// What the lanes of a warp share while they work on particle i.
+constexpr int kRowsD = 49;  // rows of cells around one, cell_div <= 3
+struct WarpD {
+    OwnD own;
+    double sup2, sF, hmu, g;
+    float4 d;  // FP32 copy of the position, and the radius certainly inside, squared
+    float filter;
+    int2 rows[kRowsD];
+};
+
 // SYM: each interacting pair once (the forward half of i's neighbourhood:
 // rows with dz > 0, rows with dz = 0 and dy > 0, and the home row after i),
 // the partner's share by pair_share_j; k_pair_fp64_finish adds the shares.
 // CNT (with SYM): also count the partners' neighbours (nneigh is read by
 // sph_derivatives and the work counts, not by a time step).
 // FIX: fixed-point sorted positions.
-// No unit is full (FP64 pipe about 70 %, of the 84 % that FMAs alone reach): the
-// gathers and the serial integer chains of a batch are covered by warps, so what
-// the lanes of a warp share lies in shared memory and 24 warps of 80 registers fit
-// on an SM instead of 16 of 124.  0.9 M particles: 12.5 -> 10.7 ms, 11 k: 200 -> 163 us
-// (the register bound alone 12.6 ms and 186 us).
+// Bound by the FP64 pipe (82 % busy on 0.9 M particles, of the 84 % that FMAs alone
+// reach) as long as enough warps cover the gathers and the serial integer chains of
+// a batch: what the lanes of a warp share, the row ranges too, lies in shared memory,
+// so that 32 warps of 64 registers fit on an SM.  0.9 M particles (11 k): 12.5 ms
+// (200 us) with all of it in 124 registers and 16 warps, 10.7 (163) without the rows
+// and 24 warps, 9.8 (145) with the rows and 24 warps, 8.9 (146) with 32, 9.9 (154)
+// with 40, which spill.
 template <bool FIX, bool DFS, bool SYM, bool CNT = true>
-__global__ void __launch_bounds__(256, 3) k_pair_fp64(Bufs b, int ninst, int kdiv)
+__global__ void __launch_bounds__(256, 4) k_pair_fp64(Bufs b, int ninst, int kdiv)
 {
     extern __shared__ int32_t smem_q[];
-    __shared__ OwnD own[8];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
+    __shared__ WarpD warps[8];
+    WarpD &W = warps[wib];
     int32_t *q = smem_q + wib * kQ;  // neighbours; the sign bit marks a fluid particle
     const unsigned lt = (1u << lane) - 1u;
     const int32_t n_in = b.misc[0];
@@ -337,23 +350,57 @@ __global__ void __launch_bounds__(256, 3) k_pair_fp64(Bufs b, int ninst, int kdi
     const dvec4 *sB = reinterpret_cast<const dvec4 *>(b.sB);
 
     for (int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_in; i += nwarps) {
-        const int32_t ci_cell = b.scell[i];
-        const Inst &I = b.inst[inst_of_cell(b.inst, ninst, ci_cell)];
-        int cx, cy, cz;
-        decompose(I, ci_cell, cx, cy, cz);
-        const float4 Di = b.sD[i];
-        const bool fluid_i = Di.w != 0.f;
-        if (lane == 0) {
-            const dvec4 A = sA[i], B = sB[i];
-            const double2 C = b.sC[i];
-            own[wib] = own_d(pair_const_d<FIX>(I), A.x, A.y, A.z, B.x, B.y, B.z, A.w, C.x, B.w, C.y);
+        int nrows = 0;
+        {
+            const int32_t ci_cell = b.scell[i];
+            const Inst &I = b.inst[inst_of_cell(b.inst, ninst, ci_cell)];
+            int cx, cy, cz;
+            decompose(I, ci_cell, cx, cy, cz);
+            if (lane == 0) {
+                const dvec4 A = sA[i], B = sB[i];
+                const double2 C = b.sC[i];
+                const float4 D = b.sD[i];
+                W.own = own_d(pair_const_d<FIX>(I), A.x, A.y, A.z, B.x, B.y, B.z, A.w, C.x, B.w, C.y);
+                W.d = make_float4(D.x, D.y, D.z, I.sup2_inner);
+                W.filter = I.sup2_filter;
+                W.sup2 = I.sup2;
+                W.sF = I.pair_sF;
+                W.hmu = I.pair_hmu;
+                W.g = I.g;
+            }
+            // a lane per row of cells reads its range, so that the loads of all rows are in
+            // flight together
+            const int side = 2 * kdiv + 1;
+            int ncand = 0;
+            for (int r0 = 0; r0 < side * side; r0 += 32) {
+                int32_t s0 = 0, s1 = 0;
+                const int r = r0 + lane, dz = r / side - kdiv, dy = r % side - kdiv, z = cz + dz, y = cy + dy;
+                if (dz <= kdiv && z >= 0 && z < I.n[2] && y >= 0 && y < I.n[1] &&
+                    (!SYM || dz > 0 || (dz == 0 && dy >= 0))) {
+                    const int32_t row = I.cell_base + (z * I.n[1] + y) * I.n[0];
+                    s0 = b.cell_start[row + max(cx - kdiv, 0)];
+                    s1 = b.cell_start[row + min(cx + kdiv, I.n[0] - 1) + 1];
+                    if (SYM && dz == 0 && dy == 0)
+                        s0 = i + 1;  // the home row from the home cell on (cells hold ascending ids), after i
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, s0 < s1);
+                if (s0 < s1) {
+                    W.rows[nrows + __popc(m & lt)] = make_int2(s0, s1);
+                    ncand += s1 - s0;
+                }
+                nrows += __popc(m);
+            }
+            ncand = warp_sum(ncand);
+            if (lane == 0)
+                b.ncand[i] = ncand;
         }
         __syncwarp();
+        const bool fluid_i = b.sflag[i] == T_FLUID;
         AccD acc = {0.0, 0.0, 0.0, 0.0, 0.0, 0};
         bool touches_boundary = false;  // DFS: some neighbour j is a boundary particle
         int nn = 0;
         int qn = 0;
-        int npair = 0, ncand = 0;
+        int npair = 0;
 
         auto flush = [&](int cnt) {
             if (lane < cnt) {
@@ -362,73 +409,60 @@ __global__ void __launch_bounds__(256, 3) k_pair_fp64(Bufs b, int ninst, int kdi
                 const dvec4 Aj = sA[j], Bj = sB[j];
                 const double2 Cj = b.sC[j];
                 if (SYM)
-                    pair_share_j<FIX>(own[wib], fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, fluid_j,
+                    pair_share_j<FIX>(W.own, fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, fluid_j,
                                       b.fjacc, b.fjmu, j, acc);
                 else
-                    pair_term_d<DFS, FIX>(own[wib], fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y,
+                    pair_term_d<DFS, FIX>(W.own, fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y,
                                           fluid_j, acc);
             }
         };
 
-        for (int dz = SYM ? 0 : -kdiv; dz <= kdiv; ++dz) {
-            int z = cz + dz;
-            if (z < 0 || z >= I.n[2])
-                continue;
-            for (int dy = (SYM && dz == 0) ? 0 : -kdiv; dy <= kdiv; ++dy) {
-                int y = cy + dy;
-                if (y < 0 || y >= I.n[1])
-                    continue;
-                int x0 = max(cx - kdiv, 0), x1 = min(cx + kdiv, I.n[0] - 1);
-                int32_t row = I.cell_base + (z * I.n[1] + y) * I.n[0];
-                int32_t s0 = b.cell_start[row + x0], s1 = b.cell_start[row + x1 + 1];
-                if (SYM && dz == 0 && dy == 0)
-                    s0 = i + 1;  // the home row from the home cell on (cells hold ascending ids), after i
-                for (int32_t base = s0; base < s1; base += 32) {
-                    int32_t j = base + lane;
-                    bool take = false, fluid_j = false;
-                    if (j < s1 && j != i) {
-                        // FP32 pre-test with radii that cover every rounding of the
-                        // FP32 copies: certainly inside, certainly outside, or (in a
-                        // thin shell around 2h) decided by the exact FP64 test
-                        const float4 Dj = b.sD[j];
-                        const float fx = Dj.x - Di.x, fy = Dj.y - Di.y, fz = Dj.z - Di.z;
-                        const float d2f = fx * fx + fy * fy + fz * fz;
-                        bool hit = d2f < I.sup2_inner;
-                        if (!hit && d2f < I.sup2_filter) {
-                            const dvec4 ri = b.pos[b.perm[i]], rj = b.pos[b.perm[j]];
-                            hit = dist2_rn(ri.x, ri.y, ri.z, rj.x, rj.y, rj.z) < I.sup2;
-                        }
-                        if (hit) {
-                            ++nn;
-                            if (SYM && CNT)
-                                atomicAdd(b.fjnn + j, 1);
-                            fluid_j = Dj.w != 0.f;
-                            take = fluid_i || fluid_j;
-                            if (DFS)
-                                touches_boundary = touches_boundary || !fluid_j;
-                        }
+        for (int k = 0; k < nrows; ++k) {
+            const int2 row = W.rows[k];
+            for (int32_t base = row.x; base < row.y; base += 32) {
+                int32_t j = base + lane;
+                bool take = false, fluid_j = false;
+                if (j < row.y && j != i) {
+                    // FP32 pre-test with radii that cover every rounding of the
+                    // FP32 copies: certainly inside, certainly outside, or (in a
+                    // thin shell around 2h) decided by the exact FP64 test
+                    const float4 Dj = b.sD[j], Di = W.d;
+                    const float fx = Dj.x - Di.x, fy = Dj.y - Di.y, fz = Dj.z - Di.z;
+                    const float d2f = fx * fx + fy * fy + fz * fz;
+                    bool hit = d2f < Di.w;
+                    if (!hit && d2f < W.filter) {
+                        const dvec4 ri = b.pos[b.perm[i]], rj = b.pos[b.perm[j]];
+                        hit = dist2_rn(ri.x, ri.y, ri.z, rj.x, rj.y, rj.z) < W.sup2;
                     }
-                    unsigned m = __ballot_sync(0xffffffffu, take);
-                    if (take)
-                        q[qn + __popc(m & lt)] = fluid_j ? j | (int32_t)0x80000000 : j;
-                    qn += __popc(m);
-                    npair += __popc(m);
-                    ncand += min(32, s1 - base);
+                    if (hit) {
+                        ++nn;
+                        if (SYM && CNT)
+                            atomicAdd(b.fjnn + j, 1);
+                        fluid_j = Dj.w != 0.f;
+                        take = fluid_i || fluid_j;
+                        if (DFS)
+                            touches_boundary = touches_boundary || !fluid_j;
+                    }
+                }
+                unsigned m = __ballot_sync(0xffffffffu, take);
+                if (take)
+                    q[qn + __popc(m & lt)] = fluid_j ? j | (int32_t)0x80000000 : j;
+                qn += __popc(m);
+                npair += __popc(m);
+                __syncwarp();
+                if (qn >= 32) {
+                    flush(32);
                     __syncwarp();
-                    if (qn >= 32) {
-                        flush(32);
-                        __syncwarp();
-                        if (lane < qn - 32)
-                            q[lane] = q[lane + 32];
-                        qn -= 32;
-                        __syncwarp();
-                    }
+                    if (lane < qn - 32)
+                        q[lane] = q[lane + 32];
+                    qn -= 32;
+                    __syncwarp();
                 }
             }
         }
         flush(qn);
         __syncwarp();
-        const double sF = I.pair_sF;  // t^3 -> m_j F
+        const double sF = W.sF;  // t^3 -> m_j F
         constexpr int K = DFS ? 8 : 4;
         double tot[K] = {acc.drho, acc.ax, acc.ay, acc.az};
         if (DFS)
@@ -440,17 +474,17 @@ __global__ void __launch_bounds__(256, 3) k_pair_fp64(Bufs b, int ninst, int kdi
         if (DFS && !__any_sync(0xffffffffu, touches_boundary))
             drho -= tot[K > 4 ? 4 : 0];
         double ax = tot[1], ay = tot[2], az = tot[3];
-        double mumax = I.pair_hmu * __longlong_as_double(warp_max_bits(acc.mumax_bits));
+        double mumax = W.hmu * __longlong_as_double(warp_max_bits(acc.mumax_bits));
         int nsum = warp_sum(nn);
         if (lane == 0) {
             if (fluid_i)
-                az -= I.g;
+                az -= W.g;
             reinterpret_cast<dvec4 *>(b.deriv)[i] = make_dvec4(ax, ay, az, drho);
             reinterpret_cast<double *>(b.mumax)[i] = mumax;
             b.nneigh[i] = nsum;
             b.npair[i] = npair;
-            b.ncand[i] = ncand;
         }
+        __syncwarp();
     }
 }
 
