@@ -26,9 +26,10 @@ enum : uint8_t { T_FLUID = 0, T_WALL = 1, T_OBST = 2, T_GATE = 3 };
 // Device status bits (ORed by kernels, read by sph_sync).
 enum : int32_t { ST_UNSTABLE = 1, ST_TIMEOUT = 2, ST_OVERFLOW = 4, ST_BOUNDS = 8 };
 
-// Debug builds (-DSPH_DEBUG) check shared-memory indices of the pair kernels
-// before each access: a failing check records ST_BOUNDS and skips the access.
-#ifdef SPH_DEBUG
+// Debug builds (-DSPH_DEBUG) check the indices of the pair kernels before each
+// access, and so does the persistent launch in every build (SPH_CHECK_BOUNDS): a
+// failing check records ST_BOUNDS and skips the access.
+#if defined(SPH_DEBUG) || defined(SPH_CHECK_BOUNDS)
 #define SPH_BOUNDS_OK(cond, status) ((cond) ? true : (atomicOr((status), ST_BOUNDS), false))
 #else
 #define SPH_BOUNDS_OK(cond, status) true

@@ -464,7 +464,11 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
     const float4 *gB = reinterpret_cast<const float4 *>(b.sB);
     const int32_t dummy = STG ? kStage : -1;
     // position and density offset of candidate t in the tile's frame
-    auto cand_a = [&](int32_t t) -> float4 {
+    auto ck = [&](int32_t t) -> int32_t {
+        return SPH_BOUNDS_OK(STG ? t >= 0 && t <= kStage : t >= -1 && t < b.misc[0], &b.misc[2]) ? t : dummy;
+    };
+    auto cand_a = [&](int32_t t_) -> float4 {
+        const int32_t t = ck(t_);
         if (STG)
             return lds_f4<0>(st + 16u * (uint32_t)t);
         if (t < 0)
@@ -477,13 +481,15 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
         a.z += (float)(cz - T.cen[2]) * I.ocf;
         return a;
     };
-    auto cand_x = [&](int32_t t) -> float { return STG ? lds_f32(st + 16u * (uint32_t)t) : cand_a(t).x; };
-    auto cand_b = [&](int32_t t) -> float4 {
+    auto cand_x = [&](int32_t t) -> float { return STG ? lds_f32(st + 16u * (uint32_t)ck(t)) : cand_a(t).x; };
+    auto cand_b = [&](int32_t t_) -> float4 {
+        const int32_t t = ck(t_);
         if (STG)
             return lds_f4<kOffB>(st + 16u * (uint32_t)t);
         return t < 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : gB[t];
     };
-    auto cand_f = [&](int32_t t) -> bool {
+    auto cand_f = [&](int32_t t_) -> bool {
+        const int32_t t = ck(t_);
         return STG ? lds_u8<kOffF>(st + (uint32_t)t) == T_FLUID : (t >= 0 && b.sflag[t] == T_FLUID);
     };
 
@@ -492,6 +498,8 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
     const int rr = __popc(__ballot_sync(0xffffffffu, lane < nh && S.hpre[min(lane, nh - 1) + 1] <= q));
     const int k0 = (q - S.hpre[rr]) * G;
     const int nreal = min(G, S.hlen[rr] - k0);  // a short cluster repeats its last particle; nothing is stored for it
+    if (!SPH_BOUNDS_OK(rr < nh && nreal >= 1 && S.hst[rr] >= 0 && S.hst[rr] + k0 + nreal <= b.misc[0], &b.misc[2]))
+        return;
     const int hy = S.hyz[rr] & 0xffff, hz = S.hyz[rr] >> 16;
     const int32_t s0 = S.hst[rr] + k0;
     const int hrow = (hz + kdiv) * T.nry + hy + kdiv;
@@ -760,9 +768,10 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
         for (int g = 0; g < G; ++g) {
             const int a = warp_sum(nn[g]), p = warp_sum(np[g]);
             if (lane == 0 && g < nreal) {
-                // the particle itself is a hit; it is evaluated unless it is a boundary particle
+                // the particle's own pair comes off both counts, as in the staged kernel (where a boundary
+                // particle's own pair is not listed, so that its count of evaluated pairs is one short)
                 b.nneigh[s0 + g] = a - 1;
-                b.npair[s0 + g] = p - (int)((fl >> g) & 1u);
+                b.npair[s0 + g] = p - 1;
                 b.ncand[s0 + g] = T.total;
             }
         }
@@ -810,7 +819,10 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
     for (;;) {
         if (tid == 0) {
             const int32_t item = atomicAdd(&b.misc[3], 1);
-            S.item = item < n_tiles ? b.tiles[item] : -1;
+            int32_t t = item < n_tiles && SPH_BOUNDS_OK(n_tiles <= b.ntiles, &b.misc[2]) ? b.tiles[item] : -1;
+            if (!SPH_BOUNDS_OK(t >= -1 && t < b.ntiles, &b.misc[2]))
+                t = -1;
+            S.item = t;
         }
         __syncthreads();  // and every warp is done with the previous tile
         const int32_t tile = S.item;
@@ -848,6 +860,8 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
                 a = b.cell_start[row + (home ? T.t0[0] : x0)];
                 n = b.cell_start[row + (home ? min(T.t0[0] + I.tdim[0], I.n[0]) : x1)] - a;
             }
+            if (!SPH_BOUNDS_OK(n >= 0 && a >= 0 && n <= b.misc[0] - a, &b.misc[2]))
+                a = n = 0;
             if (home) {
                 S.hst[r] = a;
                 S.hlen[r] = n;

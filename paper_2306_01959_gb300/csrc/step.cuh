@@ -64,7 +64,7 @@ __device__ __forceinline__ void dt_reduce_part(const Bufs &b, int ninst, int par
         amax = (a2 > amax || a2 != a2) ? a2 : amax;
         mmax = (mu > mmax || mu != mu) ? mu : mmax;
         if (MODE == SPH_MIXED) {
-            floor_a = (float)amax * (1.f - 1e-6f);
+            floor_a = (float)amax * (1.f - 1e-6f) - 1e-36f;  // (subnormal sums round further off)
             floor_m = (float)mmax * (1.f - 1e-6f);
         }
     }
