@@ -67,3 +67,31 @@ def test_long_tank_takes_the_double_positions():
         assert np.array_equal(got[3], ref[3])
         out.append([g[:nf] for g in got])
     assert not np.array_equal(out[0][1], out[1][1])  # two different paths
+
+
+# 9, 25 and 49 rows of cells: up to two loads of row ranges by the 32 lanes, and
+# rows that are empty or outside the grid (the column fills a part of the tank)
+@pytest.mark.parametrize("cell_div", [1, 2, 3])
+@pytest.mark.parametrize("kw", [{}, {"pair_symmetric": 1}])
+def test_rows_of_every_cell_size(cell_div, kw):
+    c = wl.small_dambreak()
+    case = oracle_case(c)
+    st = jittered(c, seed=5, case=case)
+    got, ref = _derivatives(c, st.r, st.u, st.rho, st.type, cell_div=cell_div, **kw), oracle.derivatives(case, st)
+    assert max(normwise(got[k], ref[k]) for k in range(3)) <= TOL
+    assert np.array_equal(got[3], ref[3])
+
+
+def test_density_sums_that_are_not_positive():
+    # rho_i + rho_j negative, or positive from two signs: the integer reciprocal
+    # leaves the former to the FP64 operations
+    c = wl.small_dambreak()
+    case = oracle_case(c)
+    st = jittered(c, seed=8, case=case)
+    rho = st.rho.copy()
+    f = np.flatnonzero(st.type == oracle.FLUID)
+    rho[f[::3]] *= -1.3
+    got = _derivatives(c, st.r, st.u, rho, st.type)
+    ref = oracle.derivatives(case, oracle.State(st.r, st.u, rho, st.type))
+    assert max(normwise(got[k], ref[k]) for k in range(3)) <= TOL
+    assert np.array_equal(got[3], ref[3])
