@@ -80,11 +80,12 @@ int mps_create(mps_t **out, const double tank[3], const double column[3], double
 
 void mps_destroy(mps_t *s);
 
-/* Advance nsteps steps.  Each step waits for its CG solve (the convergence
- * test reads one flag back every 16 iterations).  Errors: SPH_EINVAL,
+/* Advance nsteps steps.  Each step waits for its CG solve (one launch; its
+ * convergence flag is read back when it ends).  Errors: SPH_EINVAL,
  * SPH_ECUDA, SPH_ESTATE (a row of Eq. 23 with more than row_width entries),
- * SPH_EUNSTABLE (the solve did not reach cg_tol within cg_max iterations, or a
- * non-finite state). */
+ * SPH_ETIMEOUT (a grid-wide wait of the solve ran out), SPH_EUNSTABLE (the
+ * solve did not reach cg_tol within cg_max iterations, or a non-finite
+ * state). */
 int mps_step(mps_t *s, int32_t nsteps);
 
 /* The pressure system of the current state without advancing it (test seam):
