@@ -99,6 +99,41 @@ __device__ __forceinline__ double sound_d(const Inst &I, double rho)
     return I.c0 * pow(x, 0.5 * (I.gamma - 1.0));
 }
 
+// Barrier of a cooperative grid (every CTA resident): a counter that each CTA
+// raises once per barrier, waited on until it reaches (barriers passed) x (CTAs).
+// The release makes the CTA's writes before its barrier visible, the acquire those
+// of the others to the CTA after its own; both stand for the whole CTA, whose
+// threads are ordered with thread 0 by the CTA barriers around it.  The wait is
+// bounded: after `limit` polls thread 0 records ST_TIMEOUT in *status, and the
+// barrier returns false to every thread of the CTA; the caller returns then, and
+// every other CTA runs out at its next barrier.
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &target, long long limit, int32_t *status,
+                                             int *s_ok)
+{
+    __syncthreads();
+    target += gridDim.x;
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        bool ok = true;
+        for (long long polls = 0;; ++polls) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if ((int)(v - target) >= 0)  // (the counter may wrap)
+                break;
+            if (polls >= limit) {
+                atomicOr(status, ST_TIMEOUT);
+                ok = false;
+                break;
+            }
+            if (polls > 64)
+                __nanosleep(20);
+        }
+        *s_ok = ok;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+}
+
 // Max of a non-negative double through its bit pattern (order preserving for
 // x >= 0; a NaN result propagates as the largest pattern).
 __device__ __forceinline__ void atomic_max_pos(unsigned long long *addr, double x)

@@ -581,36 +581,6 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
     return t;
 }
 
-// Grid barrier (every CTA is resident); false when the wait ran out.
-__device__ __forceinline__ bool cg_barrier(MpsBufs &b, unsigned &target, int *s_ok)
-{
-    __syncthreads();
-    target += gridDim.x;
-    if (threadIdx.x == 0) {
-        unsigned *bar = reinterpret_cast<unsigned *>(&b.cgi[2]);
-        // the release makes the CTA's writes before its barrier visible, the acquire
-        // those of the others to the CTA after its own
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-        bool ok = true;
-        for (int polls = 0;; ++polls) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if ((int)(v - target) >= 0)  // (the counter may wrap)
-                break;
-            if (polls > kCgSpin) {
-                atomicOr(&b.misc[2], ST_TIMEOUT);
-                ok = false;
-                break;
-            }
-            if (polls > 64)
-                __nanosleep(20);
-        }
-        *s_ok = ok;
-    }
-    __syncthreads();
-    return *s_ok != 0;
-}
-
 __global__ void __launch_bounds__(kCgThreads, 3) k_cg_solve(MpsBufs b, int max_iterations)
 {
     const int width = b.c->width;
@@ -620,6 +590,9 @@ __global__ void __launch_bounds__(kCgThreads, 3) k_cg_solve(MpsBufs b, int max_i
     int phase = 0;
     const int32_t n_in = b.misc[0];
     const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    auto barrier = [&]() {
+        return grid_barrier(reinterpret_cast<unsigned *>(&b.cgi[2]), target, kCgSpin, &b.misc[2], &s_ok);
+    };
     // the sum of v over the grid (a barrier); the two halves of part alternate
     auto total = [&](double v, double &sum) {
         double *part = b.part + (phase & 1) * kCgMaxBlocks;
@@ -627,7 +600,7 @@ __global__ void __launch_bounds__(kCgThreads, 3) k_cg_solve(MpsBufs b, int max_i
         v = block_sum(v, sh);
         if (threadIdx.x == 0)
             part[blockIdx.x] = v;
-        if (!cg_barrier(b, target, &s_ok))
+        if (!barrier())
             return false;
         double t = 0.0;
         for (int k = threadIdx.x; k < (int)gridDim.x; k += kCgThreads)
@@ -732,7 +705,7 @@ __global__ void __launch_bounds__(kCgThreads, 3) k_cg_solve(MpsBufs b, int max_i
                 if (i + u * stride < n_in)
                     b.p[i + u * stride] = r[u] + beta * p[u];
         }
-        if (!cg_barrier(b, target, &s_ok))
+        if (!barrier())
             return;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {

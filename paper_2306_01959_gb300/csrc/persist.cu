@@ -8,12 +8,11 @@
 // (pair_mixed.cuh, step.cuh, cells.cuh), so a persistent step computes what a
 // launched step computes, bit for bit.
 //
-// The barrier is a counter in the workspace that every CTA increments once per
-// barrier; a CTA waits until it reaches (barriers passed) x (CTAs).  Every wait
-// is bounded: after spin_limit polls the CTA records ST_TIMEOUT in the device
-// status (reported as SPH_ETIMEOUT) and returns, and every other CTA then runs
-// out at its next barrier, so the launch always ends.  A cooperative launch
-// guarantees that all CTAs are resident at once.
+// The barrier (grid_barrier, device.cuh) counts in the workspace.  Every wait is
+// bounded: after spin_limit polls the CTA records ST_TIMEOUT in the device status
+// (reported as SPH_ETIMEOUT) and returns, and every other CTA then runs out at its
+// next barrier, so the launch always ends.  A cooperative launch guarantees that
+// all CTAs are resident at once.
 #define SPH_CHECK_BOUNDS  // a launch of many steps must not run on after one of its waits or counts went wrong
 #include "cells.cuh"
 #include "pair_wide.cuh"
@@ -25,33 +24,6 @@ namespace {
 
 constexpr int kPersistWarps = 8;  // the pair pass's default shape: 8 warps,
 constexpr int kPersistGroup = 4;  // 4 particles per warp
-
-// Grid barrier with a bounded wait; returns false (for every thread of the
-// CTA) when the wait ran out.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &target, long long spin_limit, int32_t *status,
-                                             int *s_ok)
-{
-    __syncthreads();
-    target += gridDim.x;
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        __threadfence();
-        atomicAdd(bar, 1u);
-        long long polls = 0;
-        while (*((volatile unsigned *)bar) < target) {
-            if (++polls > spin_limit) {
-                atomicOr(status, ST_TIMEOUT);
-                ok = 0;
-                break;
-            }
-            __nanosleep(100);
-        }
-        __threadfence();
-        *s_ok = ok;
-    }
-    __syncthreads();
-    return *s_ok != 0;
-}
 
 template <bool TILED, bool DFS>
 __global__ void __launch_bounds__(kPersistWarps * 32, 2)
