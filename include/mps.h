@@ -63,7 +63,8 @@ typedef struct mps_params {
     double cg_tol;      /* relative residual |r| <= cg_tol |b| of the CG solve (1e-6) */
     int32_t cg_max;     /* iteration cap of the CG solve (20000) */
     int32_t row_width;  /* stored off-diagonal entries per row of Eq. 23, at most (64) */
-    int32_t reserved[6];
+    int32_t spin_limit; /* polls before a grid-wide wait of the CG solve gives up (SPH_ETIMEOUT); 0 = default 2e7 */
+    int32_t reserved[5];
 } mps_params;
 
 void mps_params_default(mps_params *p);
@@ -100,7 +101,9 @@ int mps_pressure(mps_t *s, double *P, double *nd, int32_t *surf, int64_t *iterat
 int mps_get_state(mps_t *s, double *r, double *u, double *P, int32_t *type, int64_t *step);
 
 /* Load positions and velocities (id order; wall and dummy velocities are held
- * at zero).  Synchronous. */
+ * at zero).  Clears what a failed step left behind, its status too: until then
+ * every step after SPH_ETIMEOUT, SPH_ESTATE or a non-finite state reports that
+ * error again.  Synchronous. */
 int mps_set_state(mps_t *s, const double *r, const double *u);
 
 /* CG iterations and final relative residual of the last solve. */

@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(kMpsWarps * 32) k_mps_assemble(MpsBufs b)
 // every CTA adds for itself.
 constexpr int kCgThreads = 256;
 constexpr int kCgMaxBlocks = 2048;  // partial sums held per dot product
-constexpr int kCgSpin = 20000000;   // polls of a barrier wait before it gives up
+constexpr int kCgSpin = 20000000;   // polls of a barrier wait before it gives up (mps_params.spin_limit = 0)
 
 __device__ __forceinline__ double block_sum(double v, double *sh)
 {
@@ -581,7 +581,7 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
     return t;
 }
 
-__global__ void __launch_bounds__(kCgThreads, 3) k_cg_solve(MpsBufs b, int max_iterations)
+__global__ void __launch_bounds__(kCgThreads, 3) k_cg_solve(MpsBufs b, int max_iterations, int spin_limit)
 {
     const int width = b.c->width;
     __shared__ double sh[kCgThreads / 32];
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kCgThreads, 3) k_cg_solve(MpsBufs b, int max_i
     const int32_t n_in = b.misc[0];
     const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     auto barrier = [&]() {
-        return grid_barrier(reinterpret_cast<unsigned *>(&b.cgi[2]), target, kCgSpin, &b.misc[2], &s_ok);
+        return grid_barrier(reinterpret_cast<unsigned *>(&b.cgi[2]), target, spin_limit, &b.misc[2], &s_ok);
     };
     // the sum of v over the grid (a barrier); the two halves of part alternate
     auto total = [&](double v, double &sum) {
@@ -1128,7 +1128,8 @@ static int solve_pressure(mps_t *s)
         const int64_t most = std::min<int64_t>((int64_t)per_sm * sm_count(), kCgMaxBlocks);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((N + kCgThreads - 1) / kCgThreads, most));
         int cap = (int)std::min<int64_t>(((int64_t)s->p.cg_max + kCgChunk - 1) / kCgChunk * kCgChunk, 0x7fffffff);
-        void *args[] = {(void *)&s->b, &cap};
+        int spin = s->p.spin_limit > 0 ? s->p.spin_limit : kCgSpin;
+        void *args[] = {(void *)&s->b, &cap, &spin};
         MCK(cudaMemsetAsync(s->b.cgi, 0, 4 * sizeof(int32_t), s->st));
         MCK(cudaLaunchCooperativeKernel((const void *)k_cg_solve, grid, kCgThreads, args, 0, s->st));
     }
@@ -1424,6 +1425,9 @@ int mps_set_state(mps_t *s, const double *r, const double *u)
     }
     MCK(cudaMemcpyAsync(s->b.pos, pos.data(), sizeof(dvec4) * N, cudaMemcpyHostToDevice, s->st));
     MCK(cudaMemcpyAsync(s->b.vel, vel.data(), sizeof(dvec4) * N, cudaMemcpyHostToDevice, s->st));
+    // a step that failed in its solve leaves its status and its predicted particles marked
+    MCK(cudaMemsetAsync(s->b.misc + 2, 0, sizeof(int32_t), s->st));
+    MCK(cudaMemsetAsync(s->b.moved, 0, (size_t)N, s->st));
     MCK(cudaStreamSynchronize(s->st));
     return SPH_OK;
 }

@@ -28,7 +28,8 @@ class Params(ctypes.Structure):
         ("cg_tol", ctypes.c_double),
         ("cg_max", ctypes.c_int32),
         ("row_width", ctypes.c_int32),
-        ("reserved", ctypes.c_int32 * 6),
+        ("spin_limit", ctypes.c_int32),
+        ("reserved", ctypes.c_int32 * 5),
     ]
 
 
