@@ -105,6 +105,7 @@ static size_t layout(Bufs &b, char *base, int64_t N, int32_t C, int32_t ninst, i
     Layout L;
     L.base = base;
     const size_t vsz = mode == SPH_FP64 ? sizeof(dvec4) : sizeof(float4);
+    b.N = (int32_t)N;
     b.pos = L.take<dvec4>(N);
     b.vel = L.take<char>(N * vsz);
     b.velp = L.take<char>(N * vsz);

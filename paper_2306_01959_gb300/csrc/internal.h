@@ -26,11 +26,21 @@ enum : uint8_t { T_FLUID = 0, T_WALL = 1, T_OBST = 2, T_GATE = 3 };
 // Device status bits (ORed by kernels, read by sph_sync).
 enum : int32_t { ST_UNSTABLE = 1, ST_TIMEOUT = 2, ST_OVERFLOW = 4, ST_BOUNDS = 8 };
 
-// Debug builds (-DSPH_DEBUG) check the indices of the pair kernels before each
-// access, and so does the persistent launch in every build (SPH_CHECK_BOUNDS): a
-// failing check records ST_BOUNDS and skips the access.
-#if defined(SPH_DEBUG) || defined(SPH_CHECK_BOUNDS)
-#define SPH_BOUNDS_OK(cond, status) ((cond) ? true : (atomicOr((status), ST_BOUNDS), false))
+// A check that every build makes: a failing one records ST_BOUNDS in the device
+// status (SPH_ESTATE) and the caller skips what it guards.
+#ifdef __CUDACC__
+__device__ __forceinline__ bool check_ok(bool ok, int32_t *status)
+{
+    if (!ok)
+        atomicOr(status, ST_BOUNDS);
+    return ok;
+}
+#endif
+
+// Debug builds (-DSPH_DEBUG) also check single indices of the inner loops before
+// each access.
+#ifdef SPH_DEBUG
+#define SPH_BOUNDS_OK(cond, status) check_ok(cond, status)
 #else
 #define SPH_BOUNDS_OK(cond, status) true
 #endif
@@ -91,6 +101,7 @@ struct Bufs {
     uint8_t *type;           // SPH_FLUID / SPH_WALL / SPH_OBSTACLE
     uint16_t *inst_of;       // instance of each particle
     uint32_t *key;           // cell of each particle (C = out of domain)
+    int32_t N;               // particles
     // neighbour structure
     uint32_t *count;         // C + 1 per-cell counters (zero between steps)
     int32_t *cell_start;     // C + 2 lower bounds into the sorted order

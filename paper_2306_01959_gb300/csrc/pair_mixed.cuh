@@ -48,6 +48,7 @@
 #include <type_traits>
 
 #include "device.cuh"
+#include "rows.h"
 
 namespace sph {
 
@@ -67,13 +68,14 @@ __host__ __device__ __forceinline__ size_t mixed_dyn_smem(int NW) { return kOffW
 struct PairSmem {
     int32_t item;   // tile, -1 when the queue is exhausted
     int32_t next;   // next cluster of the tile
+    int32_t fit;    // the tile's neighbourhood fits the staging buffer
     int32_t wild;   // a staged value is not finite or huge: take the masked path
     unsigned long long st_ff, st_visc, st_cand;  // work counts of this CTA
     int32_t pre[kMaxRowsM + 1];  // staged index of each row's first particle
     int32_t gs[kMaxRowsM];       // its sorted index
-    int32_t hst[kMaxHome], hlen[kMaxHome];  // the tile's own particles of each home row
-    int32_t hyz[kMaxHome];                  // y | z << 16 of the home row in the tile
-    int32_t hpre[kMaxHome + 1];             // clusters before each home row
+    int32_t hoff[kMaxHome], hlen[kMaxHome + 1];  // the tile's own run of each home row, from the staged run's start
+    int32_t hyz[kMaxHome];                   // y | z << 16 of the home row in the tile
+    int32_t hpre[kMaxHome + 1];              // clusters before each home row
 };
 
 __device__ __forceinline__ void two_sum(float &s, float &e, float x)
@@ -498,12 +500,13 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
     const int rr = __popc(__ballot_sync(0xffffffffu, lane < nh && S.hpre[min(lane, nh - 1) + 1] <= q));
     const int k0 = (q - S.hpre[rr]) * G;
     const int nreal = min(G, S.hlen[rr] - k0);  // a short cluster repeats its last particle; nothing is stored for it
-    if (!SPH_BOUNDS_OK(rr < nh && nreal >= 1 && S.hst[rr] >= 0 && S.hst[rr] + k0 + nreal <= b.misc[0], &b.misc[2]))
+    if (!check_ok(rr < nh && k0 >= 0 && nreal > 0, &b.misc[2]))
         return;
     const int hy = S.hyz[rr] & 0xffff, hz = S.hyz[rr] >> 16;
-    const int32_t s0 = S.hst[rr] + k0;
     const int hrow = (hz + kdiv) * T.nry + hy + kdiv;
-    const int32_t i0 = STG ? S.pre[hrow] + (s0 - S.gs[hrow]) : s0;
+    // staged slot and sorted index, both from the row's one staged run
+    const int32_t s0 = S.gs[hrow] + S.hoff[rr] + k0;
+    const int32_t i0 = STG ? S.pre[hrow] + S.hoff[rr] + k0 : s0;
     float2 nx[P], ny[P], nz[P];
     unsigned fl = 0;  // bit g: particle g is fluid
 #pragma unroll
@@ -819,8 +822,8 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
     for (;;) {
         if (tid == 0) {
             const int32_t item = atomicAdd(&b.misc[3], 1);
-            int32_t t = item < n_tiles && SPH_BOUNDS_OK(n_tiles <= b.ntiles, &b.misc[2]) ? b.tiles[item] : -1;
-            if (!SPH_BOUNDS_OK(t >= -1 && t < b.ntiles, &b.misc[2]))
+            int32_t t = item < n_tiles && check_ok(n_tiles <= b.ntiles, &b.misc[2]) ? b.tiles[item] : -1;
+            if (!check_ok(t >= -1 && t < b.ntiles, &b.misc[2]))
                 t = -1;
             S.item = t;
         }
@@ -849,26 +852,25 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
         T.dz0 = (float)(T.cen[2] * (I.cs - I.oc));
         const int nrow = T.nry * (I.tdim[2] + 2 * kdiv), nh = I.tdim[1] * I.tdim[2];
         const int x0 = max(T.t0[0] - kdiv, 0), x1 = min(T.t0[0] + I.tdim[0] + kdiv, I.n[0]);
-        // the staged rows (one thread per row) and the tile's own runs of them
-        for (int u = tid; u < nrow + nh; u += blockDim.x) {
-            const bool home = u >= nrow;
-            const int r = home ? u - nrow : u, ny = home ? I.tdim[1] : T.nry, k = home ? 0 : kdiv;
-            const int z = T.t0[2] + r / ny - k, y = T.t0[1] + r % ny - k;
-            int32_t a = 0, n = 0;
+        // the staged rows, one thread per row: the only reads of the cell starts
+        for (int r = tid; r < nrow; r += blockDim.x) {
+            const int zr = r / T.nry, hz = zr - kdiv, hy = r - zr * T.nry - kdiv;
+            const int z = T.t0[2] + hz, y = T.t0[1] + hy;
+            const bool home = hz >= 0 && hz < I.tdim[2] && hy >= 0 && hy < I.tdim[1];
+            RowRun run = {0, 0, 0, 0};
             if (z >= 0 && z < I.n[2] && y >= 0 && y < I.n[1]) {
-                const int32_t row = I.cell_base + (z * I.n[1] + y) * I.n[0];
-                a = b.cell_start[row + (home ? T.t0[0] : x0)];
-                n = b.cell_start[row + (home ? min(T.t0[0] + I.tdim[0], I.n[0]) : x1)] - a;
+                const int32_t *row = b.cell_start + (I.cell_base + (z * I.n[1] + y) * I.n[0]);
+                const int32_t a = row[x0], e = row[x1];
+                const int32_t ha = home ? row[T.t0[0]] : a, he = home ? row[min(T.t0[0] + I.tdim[0], I.n[0])] : a;
+                check_ok(row_run(a, e, ha, he, min(b.misc[0], b.N), run), &b.misc[2]);
             }
-            if (!SPH_BOUNDS_OK(n >= 0 && a >= 0 && n <= b.misc[0] - a, &b.misc[2]))
-                a = n = 0;
+            S.gs[r] = run.gs;
+            S.pre[r + 1] = run.n;
             if (home) {
-                S.hst[r] = a;
-                S.hlen[r] = n;
-                S.hyz[r] = (r % ny) | ((r / ny) << 16);
-            } else {
-                S.gs[r] = a;
-                S.pre[r + 1] = n;
+                const int h = hz * I.tdim[1] + hy;
+                S.hoff[h] = run.hoff;
+                S.hlen[h] = run.hlen;
+                S.hyz[h] = hy | (hz << 16);
             }
         }
         if (tid == 0) {
@@ -877,10 +879,14 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
         }
         __syncthreads();
         if (wib == 0) {
+            // the tile fits if no row is longer than the buffer (so that the sums cannot
+            // overflow) and the sum is not either: then every slot lies in the buffer
             int carry = 0;
+            bool fit = true;
             for (int r0 = 0; r0 < nrow; r0 += 32) {
                 const int r = r0 + lane;
                 int x = r < nrow ? S.pre[r + 1] : 0;
+                fit = fit && x <= kStage;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const int y = __shfl_up_sync(0xffffffffu, x, o);
@@ -891,8 +897,11 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
                     S.pre[r + 1] = carry + x;
                 carry += __shfl_sync(0xffffffffu, x, 31);
             }
-            if (lane == 0)
+            fit = __all_sync(0xffffffffu, fit) && carry <= kStage;
+            if (lane == 0) {
                 S.pre[0] = 0;
+                S.fit = fit;
+            }
         } else if (wib == 1) {
             int x = lane < nh ? (S.hlen[lane] + G - 1) / G : 0;
 #pragma unroll
@@ -909,7 +918,7 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
         __syncthreads();
         T.total = S.pre[nrow];
         const int nclus = S.hpre[nh];
-        const bool fits = T.total <= kStage;
+        const bool fits = S.fit != 0;
         if (fits) {
             bool wild = false;
             const float lim = 1e15f, dmin = -0.5f * kc.rho0;

@@ -13,7 +13,6 @@
 // (reported as SPH_ETIMEOUT) and returns, and every other CTA then runs out at its
 // next barrier, so the launch always ends.  A cooperative launch guarantees that
 // all CTAs are resident at once.
-#define SPH_CHECK_BOUNDS  // a launch of many steps must not run on after one of its waits or counts went wrong
 #include "cells.cuh"
 #include "pair_wide.cuh"
 #include "step.cuh"
