@@ -123,7 +123,7 @@ __device__ __forceinline__ void scan_final_tile(const uint32_t *count,
         int64_t c = base + k;
         if (c <= C) {
             cell_start[c] = (int32_t)(uint32_t)run;
-            if (v[k] >> 32)
+            if ((v[k] >> 32) && check_ok((int64_t)(run >> 32) < C, &misc[2]))
                 active[(uint32_t)(run >> 32)] = (int32_t)c;
             if (c == C) {
                 misc[0] = (int32_t)(uint32_t)run;        // in-domain particles
@@ -192,15 +192,19 @@ __device__ __forceinline__ void sort_reorder_range(const Bufs &b, int32_t ninst,
 {
     using Key = typename std::conditional<MODE == SPH_FP64, int32_t, uint64_t>::type;
     const Key *keys = MODE == SPH_FP64 ? reinterpret_cast<const Key *>(b.ptmp) : reinterpret_cast<const Key *>(b.pkey);
-    const int32_t n_in = b.misc[0];
+    const int32_t n_in = min(b.misc[0], b.N);
     for (int32_t slot = thread0; slot < n_in; slot += stride) {
         const Key key = keys[slot];
         const int32_t id = (int32_t)(uint32_t)(key & 0xffffffffu);
+        if (!check_ok((uint32_t)id < (uint32_t)b.N, &b.misc[2]))
+            continue;
         const int32_t c = (int32_t)b.key[id];
         const dvec4 p = b.pos[id];
         const uint8_t type = b.type[id];
         const int32_t s0 = b.cell_start[c], s1 = b.cell_start[c + 1];
         const Inst &I = b.inst[b.inst_of[id]];
+        if (!check_ok(s0 >= 0 && s0 <= slot && slot < s1 && s1 <= n_in, &b.misc[2]))
+            continue;  // (the slot of a particle lies in its cell's run)
         int32_t s = s0;
         for (int32_t k = s0; k < s1; ++k)
             s += keys[k] < key;

@@ -149,7 +149,7 @@ struct Bufs {
     long long *step;         // [1] step counter
     int32_t *euler;          // [1] 1 when the current step is first-order
     int32_t *misc;           // [0] n_in, [1] n_active, [2] status, [3] pair work queue,
-                             // [4] n_tiles
+                             // [4] n_tiles, [5] persistent launch: a check has failed
     unsigned *bar;           // grid-barrier counter of the persistent time loop
     Inst *inst;              // [ninst]
     // probes and diagnostics scratch

@@ -13,6 +13,25 @@
 // (reported as SPH_ETIMEOUT) and returns, and every other CTA then runs out at its
 // next barrier, so the launch always ends.  A cooperative launch guarantees that
 // all CTAs are resident at once.
+//
+// A failed check (an index out of its range, counters out of step with the keys;
+// the access is skipped) ends the launch before the next update, so that the
+// remaining steps do not run on wrong data; sph_sync reports SPH_ESTATE.
+//
+// What each phase reads of what an earlier one wrote in the same launch, and the
+// barrier in between (numbered as in the step below; the last one ends the step):
+//   1 pair       sA sB scell sflag (8-9), cell_start (7), tiles misc[4] (8-9), misc[3] (3)
+//   2 dt maxima  deriv mumax (1), scell sflag (8-9 of the step before)
+//   3 dt         red (2); misc[2] (anywhere before)
+//   4 update     dt euler misc[5] (3), deriv (1), perm (8-9), pos vel velp (own particle)
+//   5 scan       count (4; the scatter of the step before leaves zeros)
+//   6 scan       scan_blocks (5)
+//   7 scan       scan_blocks (6), count (4)
+//   8 scatter    key xof (4), cell_start (7), count (4, taken down by this phase alone)
+//   9 tile list  cell_start (7), misc[4] (set to 0 in 7)
+//   9 sort       pkey (8), key pos vel xof (4), cell_start misc[0] (7)
+// The update (4) writes key, xof and count, the sort (9) perm, scell, sflag, sA and
+// sB: none of them is read by another CTA in the same phase.
 #include "cells.cuh"
 #include "pair_wide.cuh"
 #include "step.cuh"
@@ -49,10 +68,15 @@ __global__ void __launch_bounds__(kPersistWarps * 32, 2)
         SPH_BARRIER();
         if (blockIdx.x == 0) {
             dt_finalize_block(b, ninst, ns);
-            if (tid == 0)
+            if (tid == 0) {
                 b.misc[3] = 0;  // the pair pass's work queue, for the next step
+                b.misc[5] = (__ldcg(&b.misc[2]) & (ST_OVERFLOW | ST_BOUNDS)) != 0;
+            }
         }
         SPH_BARRIER();
+        // written by one thread between two barriers, so that every CTA leaves here or none
+        if (b.misc[5])
+            return;
         integrate_range<SPH_MIXED>(b, N, C, gthread, gstride);
         SPH_BARRIER();
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x)

@@ -18,7 +18,7 @@ namespace sph {
 template <int MODE>
 __device__ __forceinline__ void dt_reduce_part(const Bufs &b, int ninst, int part, int nparts)
 {
-    const int32_t n_in = b.misc[0];
+    const int32_t n_in = min(b.misc[0], b.N);
     const int32_t per = (n_in + nparts - 1) / nparts;
     const int32_t s_begin = part * per, s_end = min(n_in, s_begin + per);
     int cur = -1;
@@ -133,7 +133,7 @@ __device__ __forceinline__ void dt_finalize_block(const Bufs &b, int ninst, int 
 template <int MODE>
 __device__ __forceinline__ void integrate_range(const Bufs &b, int64_t N, uint32_t C, int32_t thread0, int32_t stride)
 {
-    const int32_t n_in = b.misc[0];
+    const int32_t n_in = min(b.misc[0], b.N);
     // neighbour lists: no binning here (a rebuild bins by itself); a particle
     // that moved more than s/2 since the last rebuild, or left the grid,
     // requests the next one
@@ -143,6 +143,8 @@ __device__ __forceinline__ void integrate_range(const Bufs &b, int64_t N, uint32
     const bool euler = b.euler[0] != 0;
     for (int32_t s = thread0; s < n_in; s += stride) {
         const int32_t id = b.perm[s];
+        if (!check_ok((uint32_t)id < (uint32_t)b.N, &b.misc[2]))
+            continue;
         const int k = b.inst_of[id];
         const Inst &I = b.inst[k];
         const double dt = b.dt[k];
