@@ -771,10 +771,9 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
         for (int g = 0; g < G; ++g) {
             const int a = warp_sum(nn[g]), p = warp_sum(np[g]);
             if (lane == 0 && g < nreal) {
-                // the particle's own pair comes off both counts, as in the staged kernel (where a boundary
-                // particle's own pair is not listed, so that its count of evaluated pairs is one short)
+                // the particle's own pair comes off: a hit, and evaluated for a fluid particle
                 b.nneigh[s0 + g] = a - 1;
-                b.npair[s0 + g] = p - 1;
+                b.npair[s0 + g] = p - (int)((fl >> g) & 1u);
                 b.ncand[s0 + g] = T.total;
             }
         }

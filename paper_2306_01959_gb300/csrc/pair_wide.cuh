@@ -552,7 +552,7 @@ __device__ __forceinline__ void pair_wide_body(const Bufs &b, int ninst, int kdi
                             valid[g] = ii < ie;
                             // every hit of a fluid particle is evaluated, so nn = np there
                             nsum[g] = (((fl >> g) & 1u) ? np[g] : nn[g]) - selfc;
-                            npair[g] = np[g] - selfc;
+                            npair[g] = np[g] - (((fl >> g) & 1u) ? selfc : 0);  // (a boundary particle's is not listed)
                         }
                         combine_group<G, COMP, DFS>(S, acc, slot, valid, nsum, npair, nbits);
                     }
