@@ -775,6 +775,7 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
                 b.nneigh[s0 + g] = a - 1;
                 b.npair[s0 + g] = p - (int)((fl >> g) & 1u);
                 b.ncand[s0 + g] = T.total;
+                lc[0] -= (fl >> g) & 1u;  // the own pair of a fluid particle was counted
             }
         }
     }

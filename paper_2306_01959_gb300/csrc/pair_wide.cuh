@@ -553,6 +553,8 @@ __device__ __forceinline__ void pair_wide_body(const Bufs &b, int ninst, int kdi
                             // every hit of a fluid particle is evaluated, so nn = np there
                             nsum[g] = (((fl >> g) & 1u) ? np[g] : nn[g]) - selfc;
                             npair[g] = np[g] - (((fl >> g) & 1u) ? selfc : 0);  // (a boundary particle's is not listed)
+                            if (CNT && lane == 0)
+                                lc_ff -= ((fl >> g) & 1u) ? selfc : 0;
                         }
                         combine_group<G, COMP, DFS>(S, acc, slot, valid, nsum, npair, nbits);
                     }
