@@ -56,20 +56,10 @@ __device__ __forceinline__ OwnD own_d(const PairConstD &k, double x, double y, d
 
 // The FP64 pipe of this GPU issues one warp operation every 64 cycles per
 // scheduler, so the pair term is priced in FP64 operations alone; the library's
-// reciprocal square root and correctly rounded reciprocals took about 10 and 8
-// of them each.  Both start here from the hardware's 20-bit approximation and
-// take one step of third order (Householder's method, from the series of
-// (1 - e)^-1 and (1 - e)^-1/2 in the residual e of the approximation): the
-// remaining error, e^3 < 2^-57, is below the rounding of the last operation.
-
-// 1 / a for a normal a (3 operations).
-__device__ __forceinline__ double rcp3(double a)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double e = fma(-a, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
+// reciprocal square root took about 10 of them.  This one starts from the
+// hardware's 20-bit approximation and takes one step of third order (Householder's
+// method, from the series of (1 - e)^-1/2 in the residual e of the approximation):
+// the remaining error, e^3 < 2^-57, is below the rounding of the last operation.
 
 // sqrt(a) for a >= 0 (5 operations); 0 for 0: the approximation is taken at
 // no less than 2^-1000 (an integer maximum of the bit patterns).
@@ -136,7 +126,7 @@ __device__ __forceinline__ long long fixed_t3(unsigned long long R, unsigned lon
 
 // 1 / (V d) for an integer 2^49 <= V < 2^63 and d = (1 + f) 2^(ex - 1023), ex in [128, 1792),
 // from d's bits: the product of the two mantissas, W in [1/4, 1), its reciprocal by
-// one third-order step from the FP32 approximation (as rcp3), rounded once.  Error
+// one third-order step from the FP32 approximation (Householder's again), rounded once.  Error
 // 1.11e-16, against 2.8e-16 for the FP64 operations it replaces (a product and three
 // more).  With one product for viscosity and mu in place of two: 13.1 -> 12.5 ms on
 // 0.9 M particles.
@@ -204,16 +194,26 @@ __device__ __forceinline__ PairGeoD pair_geo_d(const OwnD &o, double xj, double 
     return p;
 }
 
-// 1 / ((|r_ij|^2 + eta^2) (rho_i + rho_j)).
+// Eqs. 4-5: Pi_ij = -alpha c_bar mu / rho_bar (0 unless u_ij . r_ij < 0; a -0.0 gives
+// a zero term), c_bar / rho_bar = (c_i + c_j) / (rho_i + rho_j), and muh = mu / h =
+// (u_ij . r_ij) / (|r_ij|^2 + eta^2), 0 for an approaching pair: the running maximum
+// starts there.  cs: -alpha h (c_i + c_j), rsum: rho_i + rho_j.
 template <bool FIX>
-__device__ __forceinline__ double pair_rcp(const PairGeoD &p, double rsum)
+__device__ __forceinline__ void pair_visc(const PairGeoD &p, double udotr, double cs, double rsum, double &visc,
+                                          double &muh)
 {
-    if (!FIX)
-        return rcp3(p.re * rsum);
-    // densities whose sum is not positive, or no number, take the FP64 operations
-    if ((unsigned)((__double2hiint(rsum) >> 20) - 128) < 1664u)
-        return fixed_rcp(p.V, rsum);
-    return rcp3(int_to_double((long long)p.V) * rsum);
+    const bool app = __double2hiint(udotr) < 0;
+    if (FIX && (unsigned)((__double2hiint(rsum) >> 20) - 128) < 1664u) {
+        // one reciprocal, of (|r_ij|^2 + eta^2)(rho_i + rho_j), and one product for both
+        const double prod = udotr * fixed_rcp(p.V, rsum) * (app ? cs : rsum);
+        visc = app ? prod : 0.0;
+        muh = app ? 0.0 : prod;
+    } else {
+        // density sums that are not positive, or no number: muh does not depend on them
+        const double m = udotr * __drcp_rn(FIX ? int_to_double((long long)p.V) : p.re);
+        visc = app ? cs * m * __drcp_rn(rsum) : 0.0;
+        muh = app ? 0.0 : m;
+    }
 }
 
 // Contribution of neighbour j to particle i (Eqs. 3-7), in double.
@@ -246,16 +246,8 @@ __device__ __forceinline__ void pair_term_d(const OwnD &o, bool fluid_i, double 
     } else {
         a.drho = fma(t3, udotr - g, a.drho);
     }
-    // Eqs. 4-5: Pi_ij = -alpha c_bar mu / rho_bar, c_bar / rho_bar = (c_i + c_j) / (rho_i + rho_j),
-    // mu = h (u_ij . r_ij) / (|r_ij|^2 + eta^2) = h muh, muh = mur (rho_i + rho_j)
-    double rsum = o.rho + rhoj;
-    double mur = udotr * pair_rcp<FIX>(p, rsum);
-    // u_ij . r_ij < 0 (a -0.0 gives a zero term): the viscosity; else muh, whose
-    // maximum starts at 0: one product for both
-    const bool app = __double2hiint(udotr) < 0;
-    const double cs = fma(o.k.nah, cj, o.nac);
-    const double prod = mur * (app ? cs : rsum);
-    const double visc = app ? prod : 0.0, muh = app ? 0.0 : prod;
+    double visc, muh;
+    pair_visc<FIX>(p, udotr, fma(o.k.nah, cj, o.nac), o.rho + rhoj, visc, muh);
     // Eq. 3: a_i -= m_j (...) grad_i W_ij = m_j (...) F r_ij, with
     // (P_i + P_j) / (rho_i rho_j) = (P_i / rho_i + P_j / rho_i) / rho_j
     double coef = fma(fma(Pj, o.inv_rho, o.prho), inv_rhoj, visc) * t3;
@@ -286,12 +278,8 @@ __device__ __forceinline__ void pair_share_j(const OwnD &o, bool fluid_i, double
     double g = ff ? fma(o.drho, inv_rhoj, o.k.dfac) : 0.0;
     double gj = ff ? fma(-o.k.dfac * rhoj, o.inv_rho, o.k.dfac) : 0.0;
     a.drho = fma(t3, udotr - g, a.drho);
-    double rsum = o.rho + rhoj;
-    double mur = udotr * pair_rcp<FIX>(p, rsum);
-    const bool app = __double2hiint(udotr) < 0;
-    const double cs = fma(o.k.nah, cj, o.nac);
-    const double prod = mur * (app ? cs : rsum);
-    const double visc = app ? prod : 0.0, muh = app ? 0.0 : prod;
+    double visc, muh;
+    pair_visc<FIX>(p, udotr, fma(o.k.nah, cj, o.nac), o.rho + rhoj, visc, muh);
     double coef = fma(fma(Pj, o.inv_rho, o.prho), inv_rhoj, visc) * t3;
     a.ax += coef * rx;
     a.ay += coef * ry;
