@@ -54,7 +54,6 @@ struct sph_s {
     // is base_div * fine.
     int32_t base_div = 1, fine = 1, pub_fine = 1;
     bool auto_div = false;  // the mixed form's automatic cell size
-    bool fixed = false;     // FP64 form: fixed-point sorted positions
     bool tiled = false;     // the mixed pair pass is the tiled one (pair_mixed.cuh), else pair_wide.cuh
     int32_t ntiles = 0, ntiles_alloc = 0;  // tiles of the mixed pair pass
     int32_t C_alloc = 0;      // cells the workspace holds: the largest grid, at cell_div 3
@@ -157,16 +156,6 @@ static size_t layout(Bufs &b, char *base, int64_t N, int32_t C, int32_t ninst, i
     return (L.off + 255) & ~(size_t)255;
 }
 
-// The form of the FP64 sorted positions, the same for every instance of the handle.
-static void set_fixed_point(sph_s *s)
-{
-    s->fixed = s->mode == SPH_FP64;
-    for (const HostInst &hi : s->inst)
-        s->fixed = s->fixed && fixed_point_fits(hi.dev);
-    for (HostInst &hi : s->inst)
-        fill_fixed_point(hi.dev, s->fixed);
-}
-
 static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const sph_params *p)
 {
     if (!p || p->size != sizeof(sph_params))
@@ -211,7 +200,6 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
     }
     if (N == 0)
         return fail(s, SPH_EINVAL, "no particles");
-    set_fixed_point(s);
     // room for the finest grid the autotuner may choose (cells of 2h/3)
     int64_t C3 = 0;
     {
@@ -346,7 +334,7 @@ static void enqueue_pair(sph_t *s, cudaStream_t st, bool count = false, bool nei
 {
     if (s->mode == SPH_FP64) {
         launch_pair_fp64(s->b, s->N, s->ninst, s->p.cell_div, s->pair_warps, s->pair_ctas, s->p.delta_mode,
-                         count || neighbours, s->fixed, st);
+                         count || neighbours, st);
     } else if (s->b.lflag && !count) {
         launch_list_pass(s->b, s->N, s->ninst, s->p.delta_mode, st);
     } else if (!s->tiled) {
@@ -480,7 +468,6 @@ static int apply_grid(sph_t *s, int base, int fine)
     }
     if (C > s->C_alloc)
         return fail(s, SPH_EINVAL, "grid larger than the workspace holds");
-    set_fixed_point(s);
     CK(cudaStreamSynchronize(s->st));
     s->base_div = base;
     s->fine = fine;

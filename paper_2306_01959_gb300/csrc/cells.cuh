@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "device.cuh"
+#include "fixed.h"
 
 namespace sph {
 
@@ -215,12 +216,9 @@ __device__ __forceinline__ void sort_reorder_range(const Bufs &b, int32_t ninst,
             b.xbuild[id] = p;  // neighbour lists: reference of the displacement test
         if (MODE == SPH_FP64) {
             const dvec4 v = reinterpret_cast<const dvec4 *>(b.vel)[id];
-            const double fs = I.fx_scale;
-            reinterpret_cast<dvec4 *>(b.sA)[s] =
-                I.fx ? make_dvec4(__longlong_as_double(__double2ll_rn(p.x * fs)),
-                                  __longlong_as_double(__double2ll_rn(p.y * fs)),
-                                  __longlong_as_double(__double2ll_rn(p.z * fs)), v.w)
-                     : make_dvec4(p.x, p.y, p.z, v.w);
+            reinterpret_cast<dvec4 *>(b.sA)[s] = make_dvec4(__longlong_as_double(fixed_position(p.x, I.fx_shift)),
+                                                            __longlong_as_double(fixed_position(p.y, I.fx_shift)),
+                                                            __longlong_as_double(fixed_position(p.z, I.fx_shift)), v.w);
             reinterpret_cast<dvec4 *>(b.sB)[s] = make_dvec4(v.x, v.y, v.z, tait_d(I, v.w));
             b.sC[s] = make_double2(1.0 / v.w, sound_d(I, v.w));
             b.sD[s] = make_float4((float)p.x, (float)p.y, (float)p.z, type == T_FLUID ? 1.f : 0.f);

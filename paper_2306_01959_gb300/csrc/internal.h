@@ -57,11 +57,10 @@ struct Inst {
     double kW;  // 21 / (16 pi h^3)
     // factors of the FP64 pair terms
     double half_inv_h, kFm, dfac_d, nah;  // 0.5 / h, kF m, 2 delta h c0, -alpha h
-    // FP64 form with fixed-point positions (fx != 0, pair_fp64.cu): positions in
-    // units of 2^-s, 2h = [2^52, 2^53) of them; the constants above in those units
-    int32_t fx;
-    double fx_scale;                // 2^s
-    unsigned long long fx_kh, fx_eta;  // 2^126 / (2h 2^(s+10)); eta^2 in units of 2^(44-2s)
+    // FP64 form: positions in fixed point (fixed.h), the constants above in its units
+    int32_t fx_shift;               // s: positions in units of 2^-s, 2h in [2^62, 2^63) of them
+    uint32_t fx_eta_f;              // eta^2 in units of 2^(64 - 2s): fraction and integer part
+    uint64_t fx_eta, fx_kh;         // fx_kh: 2^126 / 2h
     double fx_hinv, fx_dfac, fx_nah;
     double pair_sF, pair_hmu;       // scale of the FP64 pair sums and of the largest mu
     // spacing of the cell origins of the mixed form's FP32 offsets: cs rounded to
@@ -115,7 +114,7 @@ struct Bufs {
     float *xof;              // mixed form, id order: x offset from the origin of the particle's cell
     int32_t *scell;          // sorted index -> cell
     // sorted particle data for the pair kernel
-    void *sA;                // FP64: dvec4 (x, y, z, rho), x, y, z the bits of 64-bit integers with Inst::fx; mixed: float4 (offset to cell origin, rho - rho0)
+    void *sA;                // FP64: dvec4 (x, y, z, rho), x, y, z the bits of 64-bit integers (fixed.h); mixed: float4 (offset to cell origin, rho - rho0)
     void *sB;                // FP64: dvec4 (u, P); mixed: float4 (u, P)
     double2 *sC;             // FP64 form: (1 / rho, c) per sorted particle; unused by the mixed form
     float4 *sD;              // FP64 form: FP32 copies of the sorted positions, for the pre-test; w: 1 for fluid
@@ -172,9 +171,8 @@ void launch_cells(const Bufs &b, int mode, int64_t N, int32_t C, cudaStream_t st
 void launch_reorder(const Bufs &b, int mode, int64_t N, int32_t ninst, int32_t ctas_per_sm, cudaStream_t st);
 // neighbours: the pass must write every particle's nneigh (with
 // pair_symmetric the partners' counts are left out of time steps).
-// fixed: the sorted positions are fixed point (Inst::fx).
 void launch_pair_fp64(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas,
-                      int32_t delta_mode, bool neighbours, bool fixed, cudaStream_t st);
+                      int32_t delta_mode, bool neighbours, cudaStream_t st);
 // stats: also write every particle's neighbour and pair counts and sum the work
 // counts (a separate instantiation, so that time steps pay nothing for them).
 void launch_pair_mixed(const Bufs &b, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas, int32_t group,
@@ -214,9 +212,6 @@ int effective_cell_div(const sph_params &p);
 // divides each of those cells again (the mixed form's own grid, see sph_s).
 // tiled: the mixed form's tiled pair pass will run on it.
 void fill_inst(HostInst &hi, const sph_params &p, int fine = 1, bool tiled = false);
-// Fixed-point positions for the FP64 pair pass (every instance of a handle, or none).
-bool fixed_point_fits(const Inst &d);
-void fill_fixed_point(Inst &d, bool on);
 // Whether the tiled pair pass (pair_mixed.cuh) suits an instance.
 bool tiles_fit(const sph_instance &in, const sph_params &p);
 // Tile dimensions of every instance (mixed form) and their count; n_total particles in all.

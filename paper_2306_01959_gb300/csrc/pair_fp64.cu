@@ -13,6 +13,7 @@
 // expensive pair arithmetic runs on full 32-lane batches (all but the last
 // batch of each particle); the lane partial sums are combined by warp shuffles.
 #include "device.cuh"
+#include "fixed.h"
 
 namespace sph {
 
@@ -31,14 +32,15 @@ struct AccD {
 // Constants of an instance used by every pair.
 struct PairConstD {
     double half_inv_h, eta2, dfac, nah;  // dfac = 2 delta h c0, nah = -alpha h
-    unsigned long long kh, eta;          // fixed-point positions only
+    uint64_t kh;                         // fixed-point positions only, and eta^2 in their units
+    Fixed2 eta;
 };
 
 template <bool FIX>
 __device__ __forceinline__ PairConstD pair_const_d(const Inst &I)
 {
-    return FIX ? PairConstD{I.fx_hinv, (double)I.fx_eta, I.fx_dfac, I.fx_nah, I.fx_kh, I.fx_eta}
-               : PairConstD{I.half_inv_h, I.eta2, I.dfac_d, I.nah, 0ull, 0ull};
+    return FIX ? PairConstD{I.fx_hinv, 0.0, I.fx_dfac, I.fx_nah, I.fx_kh, Fixed2{I.fx_eta, I.fx_eta_f}}
+               : PairConstD{I.half_inv_h, I.eta2, I.dfac_d, I.nah, 0ull, Fixed2{0ull, 0u}};
 }
 
 // Particle i of a pair, with the products that all its pairs share, and the constants.
@@ -73,114 +75,47 @@ __device__ __forceinline__ double sqrt3(double a)
 }
 
 // ---------------------------------------------------------------------------
-// Fixed-point distances.  The FP64 pipe is the bound and the integer pipes idle
-// beside it, so the steps from the positions to t^3 = (1 - q/2)^3, 15 of the 39
-// FP64 operations of a pair, run in 64-bit integers instead.  Positions are
-// multiples of 2^-s with 2h in [2^52, 2^53) units: differences are exact, and the
-// rounding of a position, 2^-54 of 2h, is below that of the doubles over most of
-// a tank.  With D = 2^10 times a difference, R = sum (D^2 / 2^64) is r^2 to 2^-60 of
-// (2h)^2, r comes from it by one third-order step from the FP32 reciprocal square
-// root (as sqrt3), t and its cube are 62-bit fractions: |error of t^3| <= 2.4e-16,
-// against 2.8e-16 for the FP64 operations (both against extended precision, any
-// distance above 2h / 64 and 2h from 0.01 to 2; closer pairs, whose R has fewer
-// bits, take the FP64 operations).
-// 0.9 M-particle case: 16.8 -> 13.2 ms per pass (20.1 ms before the pair terms were
-// shortened); grids of more than 512 supports keep the doubles, whose resolution
-// there is no better but which the integers could not hold.
-// Scaling by powers of two is exact, so the sums carry the units along: with r_ij
-// in units of 2^-s, t^3 in 2^-62 and |r_ij|^2 + eta^2 in 2^(44 - 2s), the constants
-// of PairConstD absorb the factors and pair_sF, pair_hmu undo them.
+// Fixed-point distances (fixed.h).  The FP64 pipe is the bound and the integer pipes
+// idle beside it, so the steps from the positions to t^3 = (1 - q/2)^3, |r_ij|^2 +
+// eta^2 and the reciprocal, 20 of the 39 FP64 operations of a pair, run in 64-bit
+// integers instead.  Differences are exact, |r_ij|^2 + eta^2 to 2^-81 and t to 2^-58,
+// and each result is rounded once, so that nothing is less accurate than in doubles.
+// Largest errors over pairs from 2h / 128 to 2h, 2h from 0.064 to 0.116, against
+// 113-bit arithmetic (FP64 operations in brackets): r_ij 1.1e-16 of |r_ij| (1.1e-16),
+// |r_ij|^2 + eta^2 3e-18 (5e-16), t^3 5.7e-17 (3.0e-16), the reciprocal of
+// (|r_ij|^2 + eta^2)(rho_i + rho_j) 1.1e-16 (6.3e-16), next to the coordinate planes
+// and away from them.  Closer pairs, whose |r_ij|^2 has too few bits for its root,
+// take that in FP64 (R < 2^48: below 2h / 128 to 2h / 64).
+// Scaling by powers of two is exact, so the sums carry the units along: with r_ij in
+// units of 2^-s and |r_ij|^2 + eta^2 in 2^(64 - 2s), the constants of PairConstD absorb
+// the factors and pair_sF, pair_hmu undo them.
 // ---------------------------------------------------------------------------
-// An integer of at most 2^53 in magnitude (exact), or any below 2^63 (truncated).
-__device__ __forceinline__ double int_to_double(long long v)
-{
-    const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-    const int n = __clzll((long long)u);
-    const unsigned long long m = (u << (n & 63)) >> 11;
-    const int hi = (int)(m >> 32) + ((1085 - n) << 20);
-    const int sign = (int)((unsigned long long)v >> 32) & (int)0x80000000;
-    return u ? __hiloint2double(hi | sign, (int)m) : 0.0;
-}
-
-// t^3 in units of 2^-62 from R = |r_ij|^2 (see above), 2^48 <= R < 2^62.
-__device__ __forceinline__ long long fixed_t3(unsigned long long R, unsigned long long kh)
-{
-    const int n = __clzll((long long)R) & ~1;
-    const unsigned long long m = R << n;  // [2^62, 2^64): v = m / 2^62 in [1, 4)
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((float)(unsigned)(m >> 32)));
-    const unsigned Y = __float2uint_rz(y * 140737488355328.f);  // 2^32 / sqrt(v), saturating
-    auto mul = [&](unsigned long long a) {  // a Y / 2^32
-        return (a >> 32) * Y + __umulhi((unsigned)a, Y);
-    };
-    const unsigned long long S = mul(m);                                // sqrt(v), 62 fraction bits
-    const long long E = (1ll << 62) - (long long)mul(S);                // 1 - v y^2
-    const int e = (int)(E >> 12);
-    const long long g = (E >> 1) + ((3 * (((long long)e * e) >> 38)) >> 3);  // E / 2 + 3/8 E^2
-    const unsigned long long q = S + (__mul64hi((long long)S, g << 22) >> 20);
-    const unsigned long long r = q >> (n / 2 - 1);  // in units of 2^-(s + 10)
-    const long long t = max((1ll << 62) - (long long)__umul64hi(r, kh), 0ll);
-    const unsigned long long t1 = (unsigned long long)t << 1;
-    return (long long)__umul64hi(__umul64hi(t1, t1) << 1, t1);
-}
-
-// 1 / (V d) for an integer 2^49 <= V < 2^63 and d = (1 + f) 2^(ex - 1023), ex in [128, 1792),
-// from d's bits: the product of the two mantissas, W in [1/4, 1), its reciprocal by
-// one third-order step from the FP32 approximation (Householder's again), rounded once.  Error
-// 1.11e-16, against 2.8e-16 for the FP64 operations it replaces (a product and three
-// more).  With one product for viscosity and mu in place of two: 13.1 -> 12.5 ms on
-// 0.9 M particles.
-__device__ __forceinline__ double fixed_rcp(unsigned long long V, double d)
-{
-    const int ex = __double2hiint(d) >> 20;
-    const int n = __clzll((long long)V);
-    const unsigned long long m = ((unsigned long long)__double_as_longlong(d) << 11) | 1ull << 63;
-    const unsigned long long w = __umul64hi(V << n, m);  // W, 64 fraction bits
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((float)(unsigned)(w >> 32)));
-    const unsigned Y = __float2uint_rz(y * 4611686018427387904.f);  // 2^30 / W, saturating
-    const long long E = (1ll << 62) - (long long)((w >> 32) * Y + __umulhi((unsigned)w, Y));  // 1 - W Y
-    const int e = (int)(E >> 12);
-    const long long g = E + (((long long)e * e) >> 38);  // E + E^2
-    const unsigned long long z = ((unsigned long long)Y << 31) +
-                                 (unsigned long long)(__mul64hi((long long)Y << 30, g << 21) >> 18);  // 2^61 / W
-    const int k = __clzll((long long)z);
-    const unsigned long long u = z << k;
-    return __longlong_as_double((long long)((u >> 11) + ((u >> 10) & 1) +
-                                            ((unsigned long long)(1085 - k + n + 897 - ex) << 52)));
-}
-
 // Geometry of a pair: r_ij, |r_ij|^2 + eta^2 and t^3, in the units of k.  The
 // positions are doubles, or (FIX) 64-bit integers in the same registers, and so is
 // |r_ij|^2 + eta^2 (V in place of re).
 struct PairGeoD {
     double rx, ry, rz, re, t3;
-    unsigned long long V;
+    Fixed2 V;
 };
 template <bool FIX>
 __device__ __forceinline__ PairGeoD pair_geo_d(const OwnD &o, double xj, double yj, double zj)
 {
     PairGeoD p;
     if (FIX) {
-        const long long dx = __double_as_longlong(xj) - __double_as_longlong(o.x);
-        const long long dy = __double_as_longlong(yj) - __double_as_longlong(o.y);
-        const long long dz = __double_as_longlong(zj) - __double_as_longlong(o.z);
-        const unsigned long long ax = (unsigned long long)(dx < 0 ? -dx : dx) << 10;
-        const unsigned long long ay = (unsigned long long)(dy < 0 ? -dy : dy) << 10;
-        const unsigned long long az = (unsigned long long)(dz < 0 ? -dz : dz) << 10;
-        const unsigned long long R = __umul64hi(ax, ax) + __umul64hi(ay, ay) + __umul64hi(az, az);
+        const int64_t dx = __double_as_longlong(xj) - __double_as_longlong(o.x);
+        const int64_t dy = __double_as_longlong(yj) - __double_as_longlong(o.y);
+        const int64_t dz = __double_as_longlong(zj) - __double_as_longlong(o.z);
+        const Fixed2 d2 = fixed_dist2(dx, dy, dz);
         p.rx = int_to_double(dx);
         p.ry = int_to_double(dy);
         p.rz = int_to_double(dz);
-        if (R >= (1ull << 48)) {
-            p.V = R + o.k.eta;
-            // (a pair just within 2h can round to 2h, at most 2^62)
-            p.t3 = int_to_double(fixed_t3(min(R, (1ull << 62) - 1), o.k.kh));
+        p.V.f = d2.f + o.k.eta.f;
+        p.V.R = d2.R + o.k.eta.R + (p.V.f < d2.f);
+        if (d2.R >= (1ull << 48)) {
+            p.t3 = fixed_t3(d2, o.k.kh);
         } else {
-            const double r2 = p.rx * p.rx + p.ry * p.ry + p.rz * p.rz;
-            const double t = 1.0 - sqrt3(r2) * o.k.half_inv_h;
-            p.V = (unsigned long long)__double2ll_rn(fma(r2, 0x1p-44, o.k.eta2));
-            p.t3 = t * t * t * 0x1p62;
+            const double t = 1.0 - sqrt3(p.rx * p.rx + p.ry * p.ry + p.rz * p.rz) * o.k.half_inv_h;
+            p.t3 = t * t * t;
         }
     } else {
         p.rx = xj - o.x;
@@ -210,7 +145,7 @@ __device__ __forceinline__ void pair_visc(const PairGeoD &p, double udotr, doubl
         muh = app ? 0.0 : prod;
     } else {
         // density sums that are not positive, or no number: muh does not depend on them
-        const double m = udotr * __drcp_rn(FIX ? int_to_double((long long)p.V) : p.re);
+        const double m = udotr * __drcp_rn(FIX ? int_to_double((int64_t)p.V.R) + p.V.f * 0x1p-32 : p.re);
         visc = app ? cs * m * __drcp_rn(rsum) : 0.0;
         muh = app ? 0.0 : m;
     }
@@ -264,13 +199,12 @@ __device__ __forceinline__ void pair_term_d(const OwnD &o, bool fluid_i, double 
 // has the same continuity term and j's own delta term
 // 2 delta h c0 (1 - rho_j / rho_i), mu is the same; units as pair_term_d
 // (t^3 in place of m F, mu / h).  i's own share is accumulated in a.
-template <bool FIX>
 __device__ __forceinline__ void pair_share_j(const OwnD &o, bool fluid_i, double xj, double yj, double zj, double uxj,
                                              double uyj, double uzj, double rhoj, double inv_rhoj, double Pj,
                                              double cj, bool fluid_j, dvec4 *jacc, long long *jmu, int32_t j,
                                              AccD &a)
 {
-    const PairGeoD p = pair_geo_d<FIX>(o, xj, yj, zj);
+    const PairGeoD p = pair_geo_d<true>(o, xj, yj, zj);
     const double rx = p.rx, ry = p.ry, rz = p.rz, t3 = p.t3;
     double ux = uxj - o.ux, uy = uyj - o.uy, uz = uzj - o.uz;
     double udotr = ux * rx + uy * ry + uz * rz;
@@ -279,7 +213,7 @@ __device__ __forceinline__ void pair_share_j(const OwnD &o, bool fluid_i, double
     double gj = ff ? fma(-o.k.dfac * rhoj, o.inv_rho, o.k.dfac) : 0.0;
     a.drho = fma(t3, udotr - g, a.drho);
     double visc, muh;
-    pair_visc<FIX>(p, udotr, fma(o.k.nah, cj, o.nac), o.rho + rhoj, visc, muh);
+    pair_visc<true>(p, udotr, fma(o.k.nah, cj, o.nac), o.rho + rhoj, visc, muh);
     double coef = fma(fma(Pj, o.inv_rho, o.prho), inv_rhoj, visc) * t3;
     a.ax += coef * rx;
     a.ay += coef * ry;
@@ -315,7 +249,6 @@ struct WarpD {
 // the partner's share by pair_share_j; k_pair_fp64_finish adds the shares.
 // CNT (with SYM): also count the partners' neighbours (nneigh is read by
 // sph_derivatives and the work counts, not by a time step).
-// FIX: fixed-point sorted positions.
 // Bound by the FP64 pipe (82 % busy on 0.9 M particles, of the 84 % that FMAs alone
 // reach) as long as enough warps cover the gathers and the serial integer chains of
 // a batch: what the lanes of a warp share, the row ranges too, lies in shared memory,
@@ -323,7 +256,7 @@ struct WarpD {
 // (200 us) with all of it in 124 registers and 16 warps, 10.7 (163) without the rows
 // and 24 warps, 9.8 (145) with the rows and 24 warps, 8.9 (146) with 32, 9.9 (154)
 // with 40, which spill.
-template <bool FIX, bool DFS, bool SYM, bool CNT = true>
+template <bool DFS, bool SYM, bool CNT = true>
 __global__ void __launch_bounds__(256, 4) k_pair_fp64(Bufs b, int ninst, int kdiv)
 {
     extern __shared__ int32_t smem_q[];
@@ -349,7 +282,7 @@ __global__ void __launch_bounds__(256, 4) k_pair_fp64(Bufs b, int ninst, int kdi
                 const dvec4 A = sA[i], B = sB[i];
                 const double2 C = b.sC[i];
                 const float4 D = b.sD[i];
-                W.own = own_d(pair_const_d<FIX>(I), A.x, A.y, A.z, B.x, B.y, B.z, A.w, C.x, B.w, C.y);
+                W.own = own_d(pair_const_d<true>(I), A.x, A.y, A.z, B.x, B.y, B.z, A.w, C.x, B.w, C.y);
                 W.d = make_float4(D.x, D.y, D.z, I.sup2_inner);
                 W.filter = I.sup2_filter;
                 W.sup2 = I.sup2;
@@ -398,10 +331,10 @@ __global__ void __launch_bounds__(256, 4) k_pair_fp64(Bufs b, int ninst, int kdi
                 const dvec4 Aj = sA[j], Bj = sB[j];
                 const double2 Cj = b.sC[j];
                 if (SYM)
-                    pair_share_j<FIX>(W.own, fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, fluid_j,
+                    pair_share_j(W.own, fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y, fluid_j,
                                       b.fjacc, b.fjmu, j, acc);
                 else
-                    pair_term_d<DFS, FIX>(W.own, fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y,
+                    pair_term_d<DFS, true>(W.own, fluid_i, Aj.x, Aj.y, Aj.z, Bj.x, Bj.y, Bj.z, Aj.w, Cj.x, Bj.w, Cj.y,
                                           fluid_j, acc);
             }
         };
@@ -496,10 +429,14 @@ __global__ void k_pair_fp64_finish(Bufs b, int ninst)
     }
 }
 
-template <bool FIX>
-static void launch_form(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int grid, int warps,
-                        int32_t delta_mode, bool neighbours, cudaStream_t st)
+void launch_pair_fp64(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas,
+                      int32_t delta_mode, bool neighbours, cudaStream_t st)
 {
+    if (warps <= 0 || warps > 8)
+        warps = 8;  // the kernel is compiled for at most 256 threads per CTA
+    if (ctas <= 0)
+        ctas = 8;
+    const int grid = sm_count() * ctas;
     const size_t dyn = warps * kQ * sizeof(int32_t);
     if (b.fjacc) {
         // the partners' accumulators start at zero (mu / h >= 0 as bits)
@@ -508,32 +445,18 @@ static void launch_form(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_di
         const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((N + 255) / 256, (int64_t)sm_count() * 8));
         if (neighbours) {
             cudaMemsetAsync(b.fjnn, 0, sizeof(int32_t) * (size_t)N, st);
-            k_pair_fp64<FIX, false, true, true><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
+            k_pair_fp64<false, true, true><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
             k_pair_fp64_finish<true><<<blocks, 256, 0, st>>>(b, ninst);
         } else {
-            k_pair_fp64<FIX, false, true, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
+            k_pair_fp64<false, true, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
             k_pair_fp64_finish<false><<<blocks, 256, 0, st>>>(b, ninst);
         }
         return;
     }
     if (delta_mode == SPH_DELTA_FULL_SUPPORT)
-        k_pair_fp64<FIX, true, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
+        k_pair_fp64<true, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
     else
-        k_pair_fp64<FIX, false, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
-}
-
-void launch_pair_fp64(const Bufs &b, int64_t N, int32_t ninst, int32_t cell_div, int32_t warps, int32_t ctas,
-                      int32_t delta_mode, bool neighbours, bool fixed, cudaStream_t st)
-{
-    if (warps <= 0 || warps > 8)
-        warps = 8;  // the kernel is compiled for at most 256 threads per CTA
-    if (ctas <= 0)
-        ctas = 8;
-    const int grid = sm_count() * ctas;
-    if (fixed)
-        launch_form<true>(b, N, ninst, cell_div, grid, warps, delta_mode, neighbours, st);
-    else
-        launch_form<false>(b, N, ninst, cell_div, grid, warps, delta_mode, neighbours, st);
+        k_pair_fp64<false, false><<<grid, warps * 32, dyn, st>>>(b, ninst, cell_div);
 }
 
 // ---------------------------------------------------------------------------

@@ -107,6 +107,26 @@ int validate_instance(const sph_instance &in, const sph_params &p, std::string &
     return SPH_OK;
 }
 
+// Constants of the FP64 pair pass in the units of its fixed-point positions (fixed.h).
+static void fill_fixed_point(Inst &d)
+{
+    if (!std::isfinite(d.h))
+        return;  // (refused later: such an instance has no particles)
+    const int s = 62 - std::ilogb(2.0 * d.h);
+    d.fx_shift = s;
+    const uint64_t h2 = (uint64_t)std::ldexp(2.0 * d.h, s);  // an integer in [2^62, 2^63)
+    const unsigned __int128 k = ((unsigned __int128)1 << 126) / h2;
+    d.fx_kh = k >> 64 ? ~0ull : (uint64_t)k;
+    const double eta = std::ldexp(d.eta2, 2 * s - 64);
+    d.fx_eta = (uint64_t)eta;
+    d.fx_eta_f = (uint32_t)std::ldexp(eta - (double)d.fx_eta, 32);
+    d.fx_hinv = std::ldexp(d.half_inv_h, -s);
+    d.fx_dfac = std::ldexp(d.dfac_d, s);
+    d.fx_nah = std::ldexp(d.nah, s - 64);
+    d.pair_sF = std::ldexp(-d.kFm, -s);
+    d.pair_hmu = std::ldexp(d.h, s - 64);
+}
+
 void fill_inst(HostInst &hi, const sph_params &p, int fine, bool tiled)
 {
     const sph_instance &in = hi.d;
@@ -169,6 +189,7 @@ void fill_inst(HostInst &hi, const sph_params &p, int fine, bool tiled)
     d.kFm = d.kF * d.mass;
     d.dfac_d = 2.0 * d.delta * d.h * d.c0;
     d.nah = -d.alpha * d.h;
+    fill_fixed_point(d);
     d.csound = p.csound;
     d.delta_mode = p.delta_mode;
     d.nf = (int32_t)hi.nf;
@@ -209,36 +230,6 @@ void fill_inst(HostInst &hi, const sph_params &p, int fine, bool tiled)
     d.dfac = (float)(2.0 * d.delta * d.h * d.c0);
     d.gammaf = (float)d.gamma;
     d.gf = (float)d.g;
-}
-
-// Fixed-point positions (pair_fp64.cu) take 53 bits for 2h, so that a difference
-// within the support is an exact double, and hold grids of up to 512 supports.
-bool fixed_point_fits(const Inst &d)
-{
-    double most = 0.0;
-    for (int a = 0; a < 3; ++a)
-        most = std::fmax(most, std::fmax(std::fabs(d.lo[a]), std::fabs(d.lo[a] + d.n[a] * d.cs)));
-    return most <= 512.0 * 2.0 * d.h && std::isfinite(d.h);
-}
-
-void fill_fixed_point(Inst &d, bool on)
-{
-    d.fx = on ? 1 : 0;
-    d.pair_sF = -d.kFm;
-    d.pair_hmu = d.h;
-    if (!on)
-        return;
-    const int s = 52 - std::ilogb(2.0 * d.h);
-    d.fx_scale = std::ldexp(1.0, s);
-    const uint64_t h2 = (uint64_t)std::ldexp(2.0 * d.h, s + 10);  // an integer in [2^62, 2^63)
-    const unsigned __int128 k = ((unsigned __int128)1 << 126) / h2;
-    d.fx_kh = k >> 64 ? ~0ull : (unsigned long long)k;
-    d.fx_eta = (unsigned long long)std::nearbyint(std::ldexp(d.eta2, 2 * s - 44));
-    d.fx_hinv = std::ldexp(d.half_inv_h, -s);
-    d.fx_dfac = std::ldexp(d.dfac_d, s);
-    d.fx_nah = std::ldexp(d.nah, s - 44);
-    d.pair_sF = std::ldexp(-d.kFm, -(62 + s));
-    d.pair_hmu = std::ldexp(d.h, s - 44);
 }
 
 // The tiled pair pass stages a tile of at least (2h)^3 with the cells within 2h of
