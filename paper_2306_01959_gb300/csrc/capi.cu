@@ -431,7 +431,7 @@ static int check_status(sph_t *s)
     if (misc[2] & ST_OVERFLOW)
         return fail(s, SPH_ESTATE, "cell counters out of step with the particle keys");
     if (misc[2] & ST_BOUNDS)
-        return fail(s, SPH_ESTATE, "a shared-memory bounds check of the pair kernel failed (debug build)");
+        return fail(s, SPH_ESTATE, "an index check of a kernel failed; what it guards was skipped");
     return SPH_OK;
 }
 
