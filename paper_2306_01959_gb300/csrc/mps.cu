@@ -25,8 +25,6 @@ namespace {
 
 using namespace sph;
 
-constexpr int kCgChunk = 16;  // the iteration cap is rounded up to a multiple of this
-
 struct MpsConst {
     double lo[3];
     double cs;  // cell size r_e
@@ -1127,7 +1125,7 @@ static int solve_pressure(mps_t *s)
             return mfail(s, SPH_ECUDA, "the CG kernel does not fit the device");
         const int64_t most = std::min<int64_t>((int64_t)per_sm * sm_count(), kCgMaxBlocks);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((N + kCgThreads - 1) / kCgThreads, most));
-        int cap = (int)std::min<int64_t>(((int64_t)s->p.cg_max + kCgChunk - 1) / kCgChunk * kCgChunk, 0x7fffffff);
+        int cap = s->p.cg_max;
         int spin = s->p.spin_limit > 0 ? s->p.spin_limit : kCgSpin;
         void *args[] = {(void *)&s->b, &cap, &spin};
         MCK(cudaMemsetAsync(s->b.cgi, 0, 4 * sizeof(int32_t), s->st));

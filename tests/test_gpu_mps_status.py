@@ -40,3 +40,13 @@ def test_set_state_clears_a_failed_step():
     t.step(1)
     s = t.get_state()
     assert np.array_equal(s["u"][fluid & out], u[fluid & out]) and np.array_equal(s["r"][out], r[out])
+
+
+def test_iteration_cap_is_exact():
+    args = ((1.0, 0.5, 0.5), (0.4, 0.5, 0.3), L0, 8e-4)
+    its = mps.Tank(*args).pressure()["iterations"]
+    assert its > 1
+    assert mps.Tank(*args, cg_max=its).pressure()["iterations"] == its
+    with pytest.raises(sph.SphError) as e:
+        mps.Tank(*args, cg_max=its - 1).pressure()
+    assert e.value.code == sph.SPH_EUNSTABLE
