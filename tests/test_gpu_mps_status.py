@@ -1,7 +1,8 @@
-"""Failed MPS steps: the bounded waits of the CG solve, and the handle after a
-failure once a state is loaded."""
+"""Failed MPS steps (the bounded waits of the CG solve, its iteration cap, the handle
+after a failure once a state is loaded) and which neighbour passes a step takes."""
 import numpy as np
 import pytest
+import torch
 
 from paper_2306_01959_gb300 import mps, sph
 
@@ -50,3 +51,23 @@ def test_iteration_cap_is_exact():
     with pytest.raises(sph.SphError) as e:
         mps.Tank(*args, cg_max=its - 1).pressure()
     assert e.value.code == sph.SPH_EUNSTABLE
+
+
+def _lists_overflowed(t):
+    """Word 5 of the handle's counters in its workspace (in-grid particles, non-empty
+    cells, status, two zeros, the flag, zeros; on a 256-byte boundary)."""
+    rows = t.workspace[: t.workspace.numel() // 256 * 256].view(torch.int32).view(-1, 64)
+    hit = (rows[:, 0] == t.n) & (rows[:, 1] > 0) & (rows[:, 2] == 0) & (rows[:, 6:16] == 0).all(1)
+    hit &= (rows[:, 5] == 0) | (rows[:, 5] == 1)
+    at = torch.nonzero(hit).flatten()
+    assert len(at) == 1
+    return int(rows[at[0], 5])
+
+
+@pytest.mark.parametrize("width,over", [(64, 0), (32, 0), (31, 1)])
+def test_which_neighbour_passes_run(width, over):
+    # the shallow pool of test_gpu_mps_rows.py: a floor particle has 32 particles within
+    # r_e, so that 31 entries leave the passes to the kernels that search by themselves
+    t = mps.Tank((18 * L0, 7 * L0, 0.2), (13 * L0, 7 * L0, 2 * L0), L0, 3e-4, row_width=width)
+    t.pressure()
+    assert _lists_overflowed(t) == over
