@@ -49,10 +49,10 @@ struct sph_s {
     int32_t ninst = 0;
     // Grid: cells of 2h / base_div (the cell_div of the parameters), each divided
     // again by `fine`: the automatic cell size of the mixed form is 2h for callers
-    // (sph_sizes, sph_cells) while its pair pass works on cells of h.  pub_fine is
-    // the division callers see (1; after autotuning, the tuned one).  p.cell_div
-    // is base_div * fine.
-    int32_t base_div = 1, fine = 1, pub_fine = 1;
+    // (sph_sizes, sph_cells) while its pair pass works on cells of h.  p.cell_div is
+    // base_div * fine.  Callers see the grid of cell_div pub_div: 1, after autotuning
+    // the tuned one.
+    int32_t base_div = 1, fine = 1, pub_div = 1;
     bool auto_div = false;  // the mixed form's automatic cell size
     bool tiled = false;     // the mixed pair pass is the tiled one (pair_mixed.cuh), else pair_wide.cuh
     int32_t ntiles = 0, ntiles_alloc = 0;  // tiles of the mixed pair pass
@@ -175,7 +175,7 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
         s->tiled = s->tiled && tiles_fit(in[k], *p);
     s->auto_div = s->tiled && p->cell_div == 0;
     s->fine = s->auto_div ? 2 : 1;
-    s->pub_fine = 1;
+    s->pub_div = s->base_div;
     s->p.cell_div = s->base_div * s->fine;
     s->inst.resize(n_inst);
     int64_t N = 0, C = 0;
@@ -435,15 +435,17 @@ static int check_status(sph_t *s)
     return SPH_OK;
 }
 
-// Cells of the grid callers see (cell counts per axis are multiples of `fine`).
+// Cells of the grid callers see.
 static int64_t public_cells(const sph_t *s)
 {
+    if (s->fine == 1)
+        return s->C;
+    sph_params p = s->p;
+    p.cell_div = s->pub_div;
     int64_t C = 0;
-    for (const HostInst &hi : s->inst) {
-        int64_t n = 1;
-        for (int a = 0; a < 3; ++a)
-            n *= hi.dev.n[a] / s->fine * s->pub_fine;
-        C += n;
+    for (HostInst hi : s->inst) {
+        fill_inst(hi, p);
+        C += hi.dev.ncells;
     }
     return C;
 }
@@ -971,7 +973,7 @@ int sph_cells(sph_t *s, int64_t *cell, int64_t *sorted, int64_t *cell_start, int
         enqueue_prepare(s, s->st);  // the lists keep the order of their last rebuild: rebin now
     // the structure on the grid callers see; the pass's own one is rebuilt afterwards
     const int base = s->base_div, fine = s->fine;
-    int rc = apply_grid(s, base, s->pub_fine);
+    int rc = fine > 1 ? apply_grid(s, s->pub_div, 1) : SPH_OK;
     if (rc)
         return rc;
     std::vector<uint32_t> key(N);
@@ -1095,7 +1097,7 @@ int sph_autotune(sph_t *s, int32_t steps, int32_t best[3])
             int rc = s->auto_div ? apply_grid(s, 1, best_d) : apply_grid(s, best_d, 1);
             if (rc)
                 return rc;
-            s->pub_fine = s->fine;
+            s->pub_div = best_d;
         }
     }
     // (warps per CTA, CTAs per SM, particles per warp)
@@ -1185,7 +1187,7 @@ int sph_tuned_config(const sph_t *s, int32_t out[5])
     out[0] = s->pair_warps;
     out[1] = s->pair_ctas;
     out[2] = s->pair_group;
-    out[3] = s->p.cell_div;
+    out[3] = s->pub_div;
     out[4] = s->reorder_ctas;
     return SPH_OK;
 }
