@@ -26,8 +26,11 @@
 //     makes its terms exactly zero.
 //  5. The 32 lane sums of the cluster are combined by a value-splitting shuffle
 //     butterfly and written out; nothing is carried between warps.
-// A tile whose neighbourhood exceeds the staging buffer (a dense clump), or that
-// holds values a zero weight could not cancel (non-finite or huge), takes the
+// A tile whose neighbourhood exceeds the staging buffer (compressed fluid, a clump) is
+// halved until its parts fit (fluid of the 0.9 M-particle obstacle case compressed to
+// 1.6 times its density: 3.20 -> 1.89 ms per step, against 3.02 ms staged in chunks by
+// the kernel of pair_wide.cuh).  A single cell whose neighbourhood does not, or a part
+// that holds values a zero weight could not cancel (non-finite or huge), takes the
 // same path with the candidates read from global memory and every term masked.
 //
 // Why this split: one list per particle, a group's particles spread over a cell of
@@ -55,6 +58,7 @@ namespace sph {
 constexpr int kMaxRowsM = 96;  // staged rows of a tile: (tdim_y + 2 cell_div)(tdim_z + 2 cell_div)
 constexpr int kMaxHome = 16;   // rows of the tile itself
 constexpr int kMaxWin = 51;    // rows within cell_div of a particle's, (2 * 3 + 1)^2, and the end of the list
+constexpr int kMaxParts = 12;  // pending halves of a tile: one for each halving, at most 4 + 3 + 3 (tdim <= 12, 6, 6)
 constexpr int kList = 448;     // capacity of a warp's candidate list; drained when short of room
 
 // Dynamic shared memory of a CTA of NW warps: staged A and B (with a dummy slot
@@ -65,11 +69,17 @@ constexpr int kOffWarp = (kOffF + kStage + 1 + 15) / 16 * 16;
 constexpr int kWarpBytes = kList * (int)sizeof(int32_t) + (kMaxWin + 1) * (int)sizeof(int2);
 __host__ __device__ __forceinline__ size_t mixed_dyn_smem(int NW) { return kOffWarp + (size_t)NW * kWarpBytes; }
 
+// A neighbourhood and the staging buffer: it fits; the box was halved; a single cell, read from global memory.
+enum : int32_t { kGlobal = 0, kFits = 1, kHalved = 2 };
+
 struct PairSmem {
     int32_t item;   // tile, -1 when the queue is exhausted
     int32_t next;   // next cluster of the tile
-    int32_t fit;    // the tile's neighbourhood fits the staging buffer
+    int32_t fit;    // kFits, kHalved or kGlobal
     int32_t wild;   // a staged value is not finite or huge: take the masked path
+    int32_t nh;     // home rows
+    int32_t box;    // the part of the tile in work (box_pack), 0: all of it
+    int32_t nparts, parts[kMaxParts];  // the parts to come
     unsigned long long st_ff, st_visc, st_cand;  // work counts of this CTA
     int32_t pre[kMaxRowsM + 1];  // staged index of each row's first particle
     int32_t gs[kMaxRowsM];       // its sorted index
@@ -452,6 +462,28 @@ struct TileGeo {
     float dy0, dz0;  // distance of the true cell lattice from the frame's lattice at the frame's origin
 };
 
+// A part of a tile: first cell from the tile's and cells per axis, 4 bits each.
+__device__ __forceinline__ int32_t box_pack(int ox, int oy, int oz, int dx, int dy, int dz)
+{
+    return ox | (oy << 4) | (oz << 8) | (dx << 12) | (dy << 16) | (dz << 20);
+}
+__device__ __forceinline__ int box_off(int32_t box, int a) { return (box >> (4 * a)) & 15; }
+__device__ __forceinline__ int box_dim(int32_t box, int a) { return (box >> (12 + 4 * a)) & 15; }
+
+// The two halves of a box along its longest axis (the last of the longest: the
+// clusters run along x); false for a single cell.
+__device__ __forceinline__ bool box_halves(int32_t box, int dx, int dy, int dz, int32_t (&half)[2])
+{
+    const int a = dz >= max(dx, dy) ? 2 : (dy >= dx ? 1 : 0);
+    const int d = a == 2 ? dz : (a == 1 ? dy : dx), cut = d / 2;
+    if (d < 2)
+        return false;
+    const int32_t whole = box_pack(box_off(box, 0), box_off(box, 1), box_off(box, 2), dx, dy, dz);
+    half[0] = whole - ((d - cut) << (12 + 4 * a));
+    half[1] = whole - (cut << (12 + 4 * a)) + (cut << (4 * a));
+    return true;
+}
+
 // One cluster (G particles of one home row) by one warp.  STG: candidates from
 // the staged copy; otherwise from global memory, with every term masked.
 template <int NW, int G, bool COMP, bool STAT, bool DFS, bool STG>
@@ -496,7 +528,7 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
     };
 
     // home row of cluster q, its particles
-    const int nh = I.tdim[1] * I.tdim[2];
+    const int nh = S.nh;
     const int rr = __popc(__ballot_sync(0xffffffffu, lane < nh && S.hpre[min(lane, nh - 1) + 1] <= q));
     const int k0 = (q - S.hpre[rr]) * G;
     const int nreal = min(G, S.hlen[rr] - k0);  // a short cluster repeats its last particle; nothing is stored for it
@@ -814,13 +846,17 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
         S.st_ff = 0ull;
         S.st_visc = 0ull;
         S.st_cand = 0ull;
+        S.nparts = 0;
         stA[kStage] = make_float4(1e15f, 1e15f, 1e15f, 0.f);  // the dummy: beyond 2h of everything
         stB[kStage] = make_float4(0.f, 0.f, 0.f, 0.f);
         stF[kStage] = T_FLUID;
     }
 
     for (;;) {
-        if (tid == 0) {
+        if (tid == 0 && S.nparts > 0) {
+            S.box = S.parts[--S.nparts];
+        } else if (tid == 0) {
+            S.box = 0;
             const int32_t item = atomicAdd(&b.misc[3], 1);
             int32_t t = item < n_tiles && check_ok(n_tiles <= b.ntiles, &b.misc[2]) ? b.tiles[item] : -1;
             if (!check_ok(t >= -1 && t < b.ntiles, &b.misc[2]))
@@ -844,30 +880,35 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
             T.t0[1] = (q - T.t0[2] * I.ntile[1]) * I.tdim[1];
             T.t0[2] *= I.tdim[2];
         }
+        const int32_t box = S.box;
+        int dim[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
-            T.cen[a] = T.t0[a] + I.tdim[a] / 2;
-        T.nry = I.tdim[1] + 2 * kdiv;
+        for (int a = 0; a < 3; ++a) {
+            T.t0[a] += box_off(box, a);
+            dim[a] = box ? box_dim(box, a) : I.tdim[a];
+            T.cen[a] = T.t0[a] + dim[a] / 2;
+        }
+        T.nry = dim[1] + 2 * kdiv;
         T.dy0 = (float)(T.cen[1] * (I.cs - I.oc));
         T.dz0 = (float)(T.cen[2] * (I.cs - I.oc));
-        const int nrow = T.nry * (I.tdim[2] + 2 * kdiv), nh = I.tdim[1] * I.tdim[2];
-        const int x0 = max(T.t0[0] - kdiv, 0), x1 = min(T.t0[0] + I.tdim[0] + kdiv, I.n[0]);
+        const int nrow = T.nry * (dim[2] + 2 * kdiv), nh = dim[1] * dim[2];
+        const int x0 = max(T.t0[0] - kdiv, 0), x1 = min(T.t0[0] + dim[0] + kdiv, I.n[0]);
         // the staged rows, one thread per row: the only reads of the cell starts
         for (int r = tid; r < nrow; r += blockDim.x) {
             const int zr = r / T.nry, hz = zr - kdiv, hy = r - zr * T.nry - kdiv;
             const int z = T.t0[2] + hz, y = T.t0[1] + hy;
-            const bool home = hz >= 0 && hz < I.tdim[2] && hy >= 0 && hy < I.tdim[1];
+            const bool home = hz >= 0 && hz < dim[2] && hy >= 0 && hy < dim[1];
             RowRun run = {0, 0, 0, 0};
             if (z >= 0 && z < I.n[2] && y >= 0 && y < I.n[1]) {
                 const int32_t *row = b.cell_start + (I.cell_base + (z * I.n[1] + y) * I.n[0]);
                 const int32_t a = row[x0], e = row[x1];
-                const int32_t ha = home ? row[T.t0[0]] : a, he = home ? row[min(T.t0[0] + I.tdim[0], I.n[0])] : a;
+                const int32_t ha = home ? row[T.t0[0]] : a, he = home ? row[min(T.t0[0] + dim[0], I.n[0])] : a;
                 check_ok(row_run(a, e, ha, he, min(b.misc[0], b.N), run), &b.misc[2]);
             }
             S.gs[r] = run.gs;
             S.pre[r + 1] = run.n;
             if (home) {
-                const int h = hz * I.tdim[1] + hy;
+                const int h = hz * dim[1] + hy;
                 S.hoff[h] = run.hoff;
                 S.hlen[h] = run.hlen;
                 S.hyz[h] = hy | (hz << 16);
@@ -876,6 +917,7 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
         if (tid == 0) {
             S.next = 0;
             S.wild = 0;
+            S.nh = nh;
         }
         __syncthreads();
         if (wib == 0) {
@@ -900,7 +942,15 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
             fit = __all_sync(0xffffffffu, fit) && carry <= kStage;
             if (lane == 0) {
                 S.pre[0] = 0;
-                S.fit = fit;
+                S.fit = fit ? kFits : kGlobal;
+                int32_t half[2];
+                if (!fit && box_halves(box, min(dim[0], I.n[0] - T.t0[0]), min(dim[1], I.n[1] - T.t0[1]),
+                                       min(dim[2], I.n[2] - T.t0[2]), half) &&
+                    check_ok(S.nparts + 2 <= kMaxParts, &b.misc[2])) {
+                    S.parts[S.nparts++] = half[1];
+                    S.parts[S.nparts++] = half[0];
+                    S.fit = kHalved;
+                }
             }
         } else if (wib == 1) {
             int x = lane < nh ? (S.hlen[lane] + G - 1) / G : 0;
@@ -918,7 +968,9 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
         __syncthreads();
         T.total = S.pre[nrow];
         const int nclus = S.hpre[nh];
-        const bool fits = S.fit != 0;
+        const bool fits = S.fit == kFits;
+        if (S.fit == kHalved)
+            continue;
         if (fits) {
             bool wild = false;
             const float lim = 1e15f, dmin = -0.5f * kc.rho0;
