@@ -224,10 +224,10 @@ __device__ __forceinline__ void sort_reorder_range(const Bufs &b, int32_t ninst,
             b.sD[s] = make_float4((float)p.x, (float)p.y, (float)p.z, type == T_FLUID ? 1.f : 0.f);
         } else {
             const float4 v = reinterpret_cast<const float4 *>(b.vel)[id];
-            // offsets from the origin of the cell
+            // offsets in the cell
             int cx, cy, cz;
             decompose(I, c, cx, cy, cz);
-            const double oy0 = I.lo[1] + cy * I.oc, oz0 = I.lo[2] + cz * I.oc;
+            const double oy0 = I.olo[1] + cy * I.oc, oz0 = I.olo[2] + cz * I.oc;
             reinterpret_cast<float4 *>(b.sA)[s] =
                 make_float4(b.xof[id], (float)(p.y - oy0), (float)(p.z - oz0), v.w);
             reinterpret_cast<float4 *>(b.sB)[s] = make_float4(v.x, v.y, v.z, tait_f(I, v.w));

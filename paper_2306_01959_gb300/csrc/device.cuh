@@ -59,8 +59,8 @@ __device__ __forceinline__ bool cell_coords_fast(const Inst &I, double x, double
     return ix && iy && iz;
 }
 
-// x offset of a particle from the origin of its cell (mixed form).
-__device__ __forceinline__ float x_offset(const Inst &I, double x, int cx) { return (float)(x - (I.lo[0] + cx * I.oc)); }
+// x offset of a particle in its cell (mixed form).
+__device__ __forceinline__ float x_offset(const Inst &I, double x, int cx) { return (float)(x - (I.olo[0] + cx * I.oc)); }
 
 // Streaming multiprocessors of the current device (queried once per device;
 // grids of the memory-bound kernels are capped at a multiple of it).

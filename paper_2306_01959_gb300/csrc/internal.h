@@ -63,10 +63,11 @@ struct Inst {
     uint64_t fx_eta, fx_kh;         // fx_kh: 2^126 / 2h
     double fx_hinv, fx_dfac, fx_nah;
     double pair_sF, pair_hmu;       // scale of the FP64 pair sums and of the largest mu
-    // spacing of the cell origins of the mixed form's FP32 offsets: cs rounded to
-    // 20 mantissa bits, so that a shift by a few cells is exact in FP32 (with
-    // neighbour lists: cs)
-    double oc;
+    // The mixed form's FP32 offsets run from the centre of the particle's cell, olo + c oc
+    // (with wide neighbourhoods and neighbour lists from its corner, olo = lo).  oc is
+    // cs rounded to 19 mantissa bits, so that a shift by a few half cells is exact in
+    // FP32 (there: cs).
+    double oc, olo[3];
     int32_t n[3];
     int32_t cell_base, ncells;
     // tiles of the mixed pair pass: boxes of tdim cells, ntile per axis
@@ -76,7 +77,7 @@ struct Inst {
     int32_t delta_mode;  // SPH_DELTA_ALL_FLUID or SPH_DELTA_FULL_SUPPORT
     double gate_v[3];  // prescribed velocity of the gate particles
     // FP32 copies for the mixed form
-    float csf, ocf, hf, inv_hf, c0f, rho0f, inv_rho0f, alphaf, massf, Bf, eta2f, sup2f, kFf, dfac;  // dfac = 2 delta h c0
+    float csf, ohf, hf, inv_hf, c0f, rho0f, inv_rho0f, alphaf, massf, Bf, eta2f, sup2f, kFf, dfac;  // ohf = oc / 2, dfac = 2 delta h c0
     float gammaf, gf;
     float gate_vf[3];
     // FP64 form: squared radius of a conservative FP32 pre-test on the FP32
@@ -111,10 +112,10 @@ struct Bufs {
     int32_t *perm;           // sorted index -> particle id
     int32_t *ptmp;           // FP64 form: scatter target before the per-cell id sort
     uint64_t *pkey;          // mixed form: the same with the sort key, x offset (orderable bits) << 32 | id
-    float *xof;              // mixed form, id order: x offset from the origin of the particle's cell
+    float *xof;              // mixed form, id order: x offset in the particle's cell (Inst::olo)
     int32_t *scell;          // sorted index -> cell
     // sorted particle data for the pair kernel
-    void *sA;                // FP64: dvec4 (x, y, z, rho), x, y, z the bits of 64-bit integers (fixed.h); mixed: float4 (offset to cell origin, rho - rho0)
+    void *sA;                // FP64: dvec4 (x, y, z, rho), x, y, z the bits of 64-bit integers (fixed.h); mixed: float4 (offset in the cell, rho - rho0)
     void *sB;                // FP64: dvec4 (u, P); mixed: float4 (u, P)
     double2 *sC;             // FP64 form: (1 / rho, c) per sorted particle; unused by the mixed form
     float4 *sD;              // FP64 form: FP32 copies of the sorted positions, for the pre-test; w: 1 for fluid

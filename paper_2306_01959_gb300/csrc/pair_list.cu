@@ -454,9 +454,9 @@ __global__ void k_list_regather(Bufs b, int ninst)
         decompose(I, c, cx, cy, cz);
         const dvec4 p = b.pos[id];
         const float4 v = reinterpret_cast<const float4 *>(b.vel)[id];
-        reinterpret_cast<float4 *>(b.sA)[s] = make_float4((float)(p.x - (I.lo[0] + cx * I.oc)),
-                                                          (float)(p.y - (I.lo[1] + cy * I.oc)),
-                                                          (float)(p.z - (I.lo[2] + cz * I.oc)), v.w);
+        reinterpret_cast<float4 *>(b.sA)[s] = make_float4((float)(p.x - (I.olo[0] + cx * I.oc)),
+                                                          (float)(p.y - (I.olo[1] + cy * I.oc)),
+                                                          (float)(p.z - (I.olo[2] + cz * I.oc)), v.w);
         reinterpret_cast<float4 *>(b.sB)[s] = make_float4(v.x, v.y, v.z, tait_f(I, v.w));
     }
 }

@@ -163,9 +163,11 @@ void fill_inst(HostInst &hi, const sph_params &p, int fine, bool tiled)
     if (tiled) {
         int e;
         const double f = std::frexp(d.cs, &e);
-        d.oc = std::ldexp(std::nearbyint(std::ldexp(f, 20)), e - 20);
+        d.oc = std::ldexp(std::nearbyint(std::ldexp(f, 19)), e - 19);
     }
-    d.ocf = (float)d.oc;
+    d.ohf = (float)(0.5 * d.oc);
+    for (int a = 0; a < 3; ++a)
+        d.olo[a] = d.lo[a] + (tiled ? 0.5 * d.oc : 0.0);
     d.ncells = d.n[0] * d.n[1] * d.n[2];
     d.h = in.h;
     d.c0 = in.c0;

@@ -2,6 +2,7 @@
 until their parts fit, down to single cells, and beyond those read from global memory."""
 import numpy as np
 import pytest
+from scipy import spatial
 
 import oracle
 from gpu_common import jittered, load_state, normwise, oracle_case
@@ -53,7 +54,11 @@ def test_larger_tiles(hfac):
     err = [normwise(got[k], ref[k]) for k in range(3)]
     assert max(err) <= MIXED_TOL, err
     s = sim.pair_stats()
-    assert abs(s["in_support"] - int(ref[3][ref[3] >= 0].sum())) <= 2000  # (pairs at 2h to one rounding)
+    # pairs within one FP32 rounding of 2h may fall on either side: at h = 1.5 dp all
+    # pairs of the boundary lattice that are 3 dp apart, elsewhere next to none
+    tree = spatial.cKDTree(st.r)
+    ties = int(tree.count_neighbors(tree, 2 * c.h * (1 + 1e-6)) - tree.count_neighbors(tree, 2 * c.h * (1 - 1e-6)))
+    assert abs(s["in_support"] - int(ref[3][ref[3] >= 0].sum())) <= ties
 
 
 def test_persistent_launch_equals_per_phase():
