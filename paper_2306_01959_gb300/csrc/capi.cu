@@ -49,11 +49,11 @@ struct sph_s {
     int32_t ninst = 0;
     // Grid: cells of 2h / base_div (the cell_div of the parameters), each divided
     // again by `fine`: the automatic cell size of the mixed form is 2h for callers
-    // (sph_sizes, sph_cells) while its pair pass works on cells of h.  p.cell_div is
+    // (sph_sizes, sph_cells) while its pair pass mostly works on cells of h.  p.cell_div is
     // base_div * fine.  Callers see the grid of cell_div pub_div: 1, after autotuning
     // the tuned one.
     int32_t base_div = 1, fine = 1, pub_div = 1;
-    bool auto_div = false;  // the mixed form's automatic cell size
+    bool auto_div = false;  // mixed form, cells of 2h for callers: the tiled pass may divide them
     bool tiled = false;     // the mixed pair pass is the tiled one (pair_mixed.cuh), else pair_wide.cuh
     int32_t ntiles = 0, ntiles_alloc = 0;  // tiles of the mixed pair pass
     int32_t C_alloc = 0;      // cells the workspace holds: the largest grid, at cell_div 3
@@ -169,14 +169,12 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
     s->p = *p;
     s->mode = p->precision;
     s->base_div = effective_cell_div(*p);
-    // cells of h for the mixed pair pass unless the caller chose a size; the lists work on cells of 2h + s
+    // the lists work on cells of 2h + s
     s->tiled = p->precision == SPH_MIXED;
     for (int k = 0; k < n_inst; ++k)
         s->tiled = s->tiled && tiles_fit(in[k], *p);
-    s->auto_div = s->tiled && p->cell_div == 0;
-    s->fine = s->auto_div ? 2 : 1;
+    s->auto_div = s->tiled && s->base_div == 1;
     s->pub_div = s->base_div;
-    s->p.cell_div = s->base_div * s->fine;
     s->inst.resize(n_inst);
     int64_t N = 0, C = 0;
     for (int k = 0; k < n_inst; ++k) {
@@ -186,20 +184,29 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
             return fail(s, rc, "instance " + std::to_string(k) + ": " + e);
         HostInst &hi = s->inst[k];
         hi.d = in[k];
-        fill_inst(hi, *p, s->fine, s->tiled);
-        hi.dev.pbase = (int32_t)N;
-        hi.dev.cell_base = (int32_t)C;
+        fill_inst(hi, *p);
         N += hi.nf + hi.nw + hi.no + hi.ng;
-        C += hi.dev.ncells;
         s->nf_tot += hi.nf;
         s->nw_tot += hi.nw;
         s->no_tot += hi.no;
         s->ng_tot += hi.ng;
-        if (N >= (int64_t)1 << 31 || C >= ((int64_t)1 << 31) - 4)
+        if (N >= (int64_t)1 << 31)
             return fail(s, SPH_EINVAL, "too many particles or cells (limit 2^31)");
     }
     if (N == 0)
         return fail(s, SPH_EINVAL, "no particles");
+    s->fine = s->auto_div ? tile_cell_div(s->inst, N, p->cell_div == 0) : 1;
+    s->p.cell_div = s->base_div * s->fine;
+    int32_t pbase = 0;
+    for (HostInst &hi : s->inst) {
+        fill_inst(hi, *p, s->fine, s->tiled);
+        hi.dev.pbase = pbase;
+        hi.dev.cell_base = (int32_t)C;
+        pbase += (int32_t)(hi.nf + hi.nw + hi.no + hi.ng);
+        C += hi.dev.ncells;
+        if (C >= ((int64_t)1 << 31) - 4)
+            return fail(s, SPH_EINVAL, "too many particles or cells (limit 2^31)");
+    }
     // room for the finest grid the autotuner may choose (cells of 2h/3)
     int64_t C3 = 0;
     {
@@ -215,14 +222,20 @@ static int prepare_sizes(sph_t *s, int32_t n_inst, const sph_instance *in, const
         return fail(s, SPH_EINVAL, "too many cells (limit 2^31)");
     s->C_alloc = (int32_t)std::max<int64_t>(C3, C);
     if (s->tiled) {
-        // room for the tiles of every cell size the autotuner may choose
+        // room for the cells and tiles of every cell size the autotuner may choose
         for (int d = 1; d <= 2; ++d) {
             sph_params pd = *p;
             if (!s->auto_div)
                 pd.cell_div = d;
             std::vector<HostInst> tmp = s->inst;
-            for (HostInst &hi : tmp)
+            int64_t Cd = 0;
+            for (HostInst &hi : tmp) {
                 fill_inst(hi, pd, s->auto_div ? d : 1, true);
+                Cd += hi.dev.ncells;
+            }
+            if (Cd >= ((int64_t)1 << 31) - 4)
+                return fail(s, SPH_EINVAL, "too many cells (limit 2^31)");
+            s->C_alloc = (int32_t)std::max<int64_t>(s->C_alloc, Cd);
             s->ntiles_alloc = std::max(s->ntiles_alloc, (int32_t)fill_tiles(tmp, d, N));
         }
         s->ntiles = (int32_t)fill_tiles(s->inst, s->p.cell_div, N);

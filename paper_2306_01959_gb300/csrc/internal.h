@@ -215,6 +215,8 @@ int effective_cell_div(const sph_params &p);
 void fill_inst(HostInst &hi, const sph_params &p, int fine = 1, bool tiled = false);
 // Whether the tiled pair pass (pair_mixed.cuh) suits an instance.
 bool tiles_fit(const sph_instance &in, const sph_params &p);
+// Cells per 2h of the tiled pass where callers see cells of 2h (1 or 2).
+int tile_cell_div(const std::vector<HostInst> &inst, int64_t n_total, bool automatic);
 // Tile dimensions of every instance (mixed form) and their count; n_total particles in all.
 int64_t fill_tiles(std::vector<HostInst> &inst, int cell_div, int64_t n_total);
 void build_scene(const HostInst &hi, const sph_params &p, double *r, double *rho, uint8_t *type);

@@ -246,6 +246,21 @@ bool tiles_fit(const sph_instance &in, const sph_params &p)
     return !(p.list_skin > 0) && n * n * n <= kStage;
 }
 
+// Cells per 2h of the tiled pass where callers see cells of 2h.  Cells of h leave fewer
+// candidates to test, but hold less than 6 particles each below h = 1.75 dp, and rows of
+// 2h fill the clusters better there (us per step, cells of 2h | h: 0.9 M particles h = 1.5 dp
+// 772 | 890, 1.8 dp 1040 | 1036, 2.08 dp 1367 | 1292; 31 k particles 90 | 100, 91 | 94,
+// 99 | 100).  The automatic size takes that below 48 k particles only (18 k at h = 1.5
+// dp: 68 us, 78 with cells of h, 69 before the tiled pass): larger tanks get tiles whose
+// FP32 frames are longer with cells of 2h, at 185 k particles a tenth less accurate.
+int tile_cell_div(const std::vector<HostInst> &inst, int64_t n_total, bool automatic)
+{
+    double most = 0.0;
+    for (const HostInst &hi : inst)
+        most = std::max(most, hi.d.h / hi.d.dp);
+    return most < 1.75 && (!automatic || n_total < 48000) ? 1 : 2;
+}
+
 // A larger tile stages fewer candidates per particle of its own (27 at (2h)^3, 18 at
 // twice that length); it has to fit the staging buffer like the smallest, and there
 // must be enough tiles to fill the GPU (2 CTAs on each of 152 SMs) four times over.
