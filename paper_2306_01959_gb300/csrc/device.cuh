@@ -253,11 +253,10 @@ __device__ __forceinline__ int inst_of_tile(const Inst *inst, int ninst, int32_t
 
 __device__ __forceinline__ void decompose(const Inst &I, int32_t c, int &cx, int &cy, int &cz)
 {
-    int lc = c - I.cell_base;
-    cx = lc % I.n[0];
-    int t = lc / I.n[0];
-    cy = t % I.n[1];
-    cz = t / I.n[1];
+    const int lc = c - I.cell_base, t = divide(lc, I.by_nx);
+    cx = lc - t * I.n[0];
+    cz = divide(t, I.by_ny);
+    cy = t - cz * I.n[1];
 }
 
 }  // namespace sph

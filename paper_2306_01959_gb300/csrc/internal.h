@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "divide.h"
 #include "sph.h"
 
 namespace sph {
@@ -70,6 +71,7 @@ struct Inst {
     double oc, olo[3];
     int32_t n[3];
     int32_t cell_base, ncells;
+    Divisor by_nx, by_ny;  // n[0] and n[1], for decompose
     // tiles of the mixed pair pass: boxes of tdim cells, ntile per axis
     int32_t tdim[3], ntile[3], tile_base;
     int32_t pbase, np, nf, nw, no, ng;

@@ -169,6 +169,8 @@ void fill_inst(HostInst &hi, const sph_params &p, int fine, bool tiled)
     for (int a = 0; a < 3; ++a)
         d.olo[a] = d.lo[a] + (tiled ? 0.5 * d.oc : 0.0);
     d.ncells = d.n[0] * d.n[1] * d.n[2];
+    d.by_nx = divisor(std::max(d.n[0], 1));
+    d.by_ny = divisor(std::max(d.n[1], 1));
     d.h = in.h;
     d.c0 = in.c0;
     d.rho0 = in.rho0;
