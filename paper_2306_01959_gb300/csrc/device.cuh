@@ -7,20 +7,10 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "grid.h"
 #include "internal.h"
 
 namespace sph {
-
-// Cell along one axis from the coordinate in cells; false outside [0, n).  One FP64
-// conversion (rounding down) instead of a floor, two comparisons and a conversion:
-// the kernels that bin every particle are bound by the FP64 pipe (mixed update of
-// 0.9 M particles 69 -> 54 us, of 1.77 M 140 -> 107 us).  The conversion saturates;
-// a NaN, which it would turn into 0, is told by its bits.
-__device__ __forceinline__ bool cell_of(double f, int n, int &c)
-{
-    c = __double2int_rd(f);
-    return (unsigned)c < (unsigned)n && (__double2hiint(f) & 0x7ff00000) != 0x7ff00000;
-}
 
 // Cell coordinates with the exact IEEE division (x - lo) / cs, as the
 // definition of the grid states it; false when outside the grid.
@@ -30,23 +20,6 @@ __device__ __forceinline__ bool cell_coords_exact(const Inst &I, double x, doubl
     const bool ix = cell_of((x - I.lo[0]) / I.cs, I.n[0], cx), iy = cell_of((y - I.lo[1]) / I.cs, I.n[1], cy),
                iz = cell_of((z - I.lo[2]) / I.cs, I.n[2], cz);
     return ix && iy && iz;
-}
-
-// The cell along one axis as the definition states it, from d = x - lo, by the
-// product with 1/cs.  Adding 1.5 2^36 leaves the coordinate in cells as an integer of
-// 2^-16 in the low word (up to 2^16 cells; the high word tells what is outside).  The
-// product and the quotient differ by less than 2^-36 there, so that only a coordinate
-// within 2^-16 of a face takes the division: a particle on a face (a lattice plane,
-// where the two may round to either side) is binned alike by every kernel.  Update of
-// 0.9 M mixed particles: as fast as the product alone.
-__device__ __forceinline__ bool cell_of_product(double d, double cs, double inv_cs, int n, int &c)
-{
-    const double q = fma(d, inv_cs, 0x1.8p36);
-    const unsigned lo = (unsigned)__double2loint(q);
-    if (n > 0xffff || ((lo + 1u) & 0xffffu) <= 2u)
-        return cell_of(d / cs, n, c);
-    c = (int)(lo >> 16);
-    return __double2hiint(q) == 0x42380000 && c < n;
 }
 
 // The cells of cell_coords_exact, at the cost of three products.
