@@ -487,7 +487,7 @@ static int apply_grid(sph_t *s, int base, int fine)
     s->base_div = base;
     s->fine = fine;
     s->p.cell_div = base * fine;
-    s->C = (int32_t)C;
+    s->b.C = s->C = (int32_t)C;
     if (s->tiled)
         s->b.ntiles = s->ntiles = (int32_t)fill_tiles(s->inst, s->p.cell_div, s->N);
     for (int k = 0; k < s->ninst; ++k)
@@ -525,6 +525,7 @@ static int create_common(sph_t **out, int32_t n_inst, const sph_instance *in, co
     s->ws_bytes = bytes;
     layout(s->b, s->ws, s->N, s->C_alloc, s->ninst, s->mode, s->list_cap, s->p.pair_symmetric != 0, s->ntiles_alloc);
     s->b.ntiles = s->ntiles;
+    s->b.C = s->C;
     s->st = (cudaStream_t)stream;
     s->pair_warps = p->pair_warps;
     s->pair_ctas = p->pair_ctas_per_sm;

@@ -141,10 +141,15 @@ __device__ __forceinline__ void scan_final_tile(const uint32_t *count,
 // of each to its slot; decrementing the counters returns them to zero.
 template <class T, class F>
 __device__ __forceinline__ void scatter_entries(const uint32_t *key, uint32_t *count, const int32_t *cell_start, T *tmp,
-                                                int32_t *misc, int64_t N, int64_t thread0, int64_t stride, F &&entry)
+                                                int32_t *misc, int64_t N, uint32_t C, int64_t thread0, int64_t stride,
+                                                F &&entry)
 {
     for (int64_t id = thread0; id < N; id += stride) {
         uint32_t c = key[id];
+        if (c > C) {  // (C: the out-of-domain bucket)
+            atomicOr(&misc[2], ST_OVERFLOW);
+            continue;
+        }
         uint32_t v = atomicSub(&count[c], 1u);
         int64_t slot = (int64_t)cell_start[c] + (int64_t)v - 1;
         if (v == 0u || slot < 0 || slot >= N) {  // counters out of step with the keys
@@ -157,9 +162,10 @@ __device__ __forceinline__ void scatter_entries(const uint32_t *key, uint32_t *c
 
 // The scatter of particle ids.
 __device__ __forceinline__ void scatter_range(const uint32_t *key, uint32_t *count, const int32_t *cell_start,
-                                              int32_t *tmp, int32_t *misc, int64_t N, int64_t thread0, int64_t stride)
+                                              int32_t *tmp, int32_t *misc, int64_t N, uint32_t C, int64_t thread0,
+                                              int64_t stride)
 {
-    scatter_entries(key, count, cell_start, tmp, misc, N, thread0, stride, [](int64_t id) { return (int32_t)id; });
+    scatter_entries(key, count, cell_start, tmp, misc, N, C, thread0, stride, [](int64_t id) { return (int32_t)id; });
 }
 
 // ---------------------------------------------------------------------------
@@ -181,9 +187,9 @@ template <int MODE>
 __device__ __forceinline__ void scatter_phase(const Bufs &b, int64_t N, int64_t thread0, int64_t stride)
 {
     if (MODE == SPH_FP64)
-        scatter_range(b.key, b.count, b.cell_start, b.ptmp, b.misc, N, thread0, stride);
+        scatter_range(b.key, b.count, b.cell_start, b.ptmp, b.misc, N, (uint32_t)b.C, thread0, stride);
     else
-        scatter_entries(b.key, b.count, b.cell_start, b.pkey, b.misc, N, thread0, stride, [&](int64_t id) {
+        scatter_entries(b.key, b.count, b.cell_start, b.pkey, b.misc, N, (uint32_t)b.C, thread0, stride, [&](int64_t id) {
             return ((uint64_t)orderable(b.xof[id]) << 32) | (uint32_t)id;
         });
 }
@@ -200,6 +206,8 @@ __device__ __forceinline__ void sort_reorder_range(const Bufs &b, int32_t ninst,
         if (!check_ok((uint32_t)id < (uint32_t)b.N, &b.misc[2]))
             continue;
         const int32_t c = (int32_t)b.key[id];
+        if (!check_ok((uint32_t)c < (uint32_t)b.C, &b.misc[2]))
+            continue;
         const dvec4 p = b.pos[id];
         const uint8_t type = b.type[id];
         const int32_t s0 = b.cell_start[c], s1 = b.cell_start[c + 1];

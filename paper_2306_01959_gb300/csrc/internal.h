@@ -103,7 +103,7 @@ struct Bufs {
     uint8_t *type;           // SPH_FLUID / SPH_WALL / SPH_OBSTACLE
     uint16_t *inst_of;       // instance of each particle
     uint32_t *key;           // cell of each particle (C = out of domain)
-    int32_t N;               // particles
+    int32_t N, C;            // particles and cells
     // neighbour structure
     uint32_t *count;         // C + 1 per-cell counters (zero between steps)
     int32_t *cell_start;     // C + 2 lower bounds into the sorted order

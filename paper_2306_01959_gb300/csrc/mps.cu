@@ -110,8 +110,8 @@ __global__ void k_mps_scan_final(MpsBufs b, int64_t C)
 }
 __global__ void k_mps_scatter(MpsBufs b, int64_t N)
 {
-    scatter_range(b.key, b.count, b.cell_start, b.ptmp, b.misc, N, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
-                  (int64_t)gridDim.x * blockDim.x);
+    scatter_range(b.key, b.count, b.cell_start, b.ptmp, b.misc, N, (uint32_t)b.c->ncells,
+                  blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // One warp per non-empty cell: rank its particles by id, gather the sorted
