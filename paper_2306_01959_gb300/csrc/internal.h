@@ -64,10 +64,12 @@ struct Inst {
     uint64_t fx_eta, fx_kh;         // fx_kh: 2^126 / 2h
     double fx_hinv, fx_dfac, fx_nah;
     double pair_sF, pair_hmu;       // scale of the FP64 pair sums and of the largest mu
-    // The mixed form's FP32 offsets run from the centre of the particle's cell, olo + c oc
-    // (with wide neighbourhoods and neighbour lists from its corner, olo = lo).  oc is
-    // cs rounded to 19 mantissa bits, so that a shift by a few half cells is exact in
-    // FP32 (there: cs).
+    // The mixed form's FP32 offsets run from olo + c oc in cell c: its corner, or with
+    // cells of 2h under the tiled pass its centre (`centred`: from the corner those would
+    // have a bit less than cells of h).  oc is cs rounded to 20 mantissa bits, so that a
+    // shift by a few cells, or half cells, is exact in FP32 (with wide neighbourhoods
+    // and neighbour lists: cs).
+    int32_t centred;
     double oc, olo[3];
     int32_t n[3];
     int32_t cell_base, ncells;

@@ -7,9 +7,9 @@
 //  1. The CTA stages the particles of the tile and of every cell within
 //     cell_div cells of it into shared memory.  Rows of cells along x are
 //     contiguous in the sorted order and sorted by x, so each (y, z) row is one
-//     copy.  Every staged position is shifted from the centre of its own cell to
-//     that of the tile; the FP32 offsets stay small, so relative distances
-//     keep full FP32 precision however large the tank is.  The centres lie on a
+//     copy.  Every staged position is shifted from its own cell to the middle of
+//     the tile; the FP32 offsets stay small, so relative distances
+//     keep full FP32 precision however large the tank is.  The origins lie on a
 //     lattice whose spacing (Inst::oc) has few mantissa bits, so the shifts are
 //     exact in FP32.
 //  2. A warp takes a cluster of G particles (G = 2 or 4) that follow one
@@ -455,8 +455,8 @@ __device__ __forceinline__ int warp_split_totals(float (&v)[K], float (&e)[K], i
 // Geometry of the tile a CTA works on.
 struct TileGeo {
     int32_t t0[3];   // first cell
-    int32_t cen[3];  // centre in half cells, the origin of the frame
-    int dim[2];      // cells along y and z
+    int32_t cen[3];  // origin of the frame, in half cells: the tile's centre, or a corner of its middle cell
+    int mid[2];      // its distance from the first cell along y and z
     int nry;         // staged rows along y
     int32_t total;   // staged particles
     int row0, row1;  // (dy & 0xff) | dz << 8 of this lane's row around a particle's (the first 32, the next)
@@ -511,9 +511,9 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
         float4 a = gA[t];
         int cx, cy, cz;
         decompose(I, b.scell[t], cx, cy, cz);
-        a.x += (float)(2 * cx + 1 - T.cen[0]) * I.ohf;
-        a.y += (float)(2 * cy + 1 - T.cen[1]) * I.ohf;
-        a.z += (float)(2 * cz + 1 - T.cen[2]) * I.ohf;
+        a.x += (float)(2 * cx + I.centred - T.cen[0]) * I.ohf;
+        a.y += (float)(2 * cy + I.centred - T.cen[1]) * I.ohf;
+        a.z += (float)(2 * cz + I.centred - T.cen[2]) * I.ohf;
         return a;
     };
     auto cand_x = [&](int32_t t) -> float { return STG ? lds_f32(st + 16u * (uint32_t)ck(t)) : cand_a(t).x; };
@@ -573,8 +573,8 @@ __device__ __forceinline__ void pair_cluster(const Bufs &b, const Inst &I, const
             if (ra < rb) {
                 // centre and half width of the cross-section
                 const float hc = 0.5f * kc.cs, eps = 2e-6f * kc.cs;
-                const float yc = (float)(2 * (hy + dy) + 1 - T.dim[0]) * hc + T.dy0;
-                const float zc = (float)(2 * (hz + dz) + 1 - T.dim[1]) * hc + T.dz0;
+                const float yc = (float)(2 * (hy + dy) + 1 - T.mid[0]) * hc + T.dy0;
+                const float zc = (float)(2 * (hz + dz) + 1 - T.mid[1]) * hc + T.dz0;
                 float xl = 3.0e38f, xh = -3.0e38f;
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
@@ -888,10 +888,10 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
         for (int a = 0; a < 3; ++a) {
             T.t0[a] += box_off(box, a);
             dim[a] = box ? box_dim(box, a) : I.tdim[a];
-            T.cen[a] = 2 * T.t0[a] + dim[a];
+            T.cen[a] = 2 * T.t0[a] + (I.centred ? dim[a] : dim[a] & ~1);
         }
-        T.dim[0] = dim[1];
-        T.dim[1] = dim[2];
+        T.mid[0] = T.cen[1] - 2 * T.t0[1];
+        T.mid[1] = T.cen[2] - 2 * T.t0[2];
         T.nry = dim[1] + 2 * kdiv;
         T.dy0 = (float)(0.5 * T.cen[1] * (I.cs - I.oc));
         T.dz0 = (float)(0.5 * T.cen[2] * (I.cs - I.oc));
@@ -984,15 +984,15 @@ __device__ __forceinline__ void pair_mixed_body(const Bufs &b, int ninst, int kd
                     continue;
                 const int zr = r / T.nry;
                 const int y = T.t0[1] + (r - zr * T.nry) - kdiv, z = T.t0[2] + zr - kdiv;
-                const float sy = (float)(2 * y + 1 - T.cen[1]) * I.ohf, sz = (float)(2 * z + 1 - T.cen[2]) * I.ohf;
-                const int32_t row = I.cell_base + (z * I.n[1] + y) * I.n[0];
+                const float sy = (float)(2 * y + I.centred - T.cen[1]) * I.ohf, sz = (float)(2 * z + I.centred - T.cen[2]) * I.ohf;
+                const int32_t row = I.cell_base + (z * I.n[1] + y) * I.n[0], sx = I.centred - T.cen[0];
 #pragma unroll 3
                 for (int32_t l = lane; l < len; l += 32) {
                     const int32_t j = g0 + l;
                     float4 a = gA[j];
                     const float4 v = gB[j];
                     const uint8_t f = b.sflag[j];
-                    a.x += (float)(2 * (b.scell[j] - row) + 1 - T.cen[0]) * I.ohf;
+                    a.x += (float)(2 * (b.scell[j] - row) + sx) * I.ohf;
                     a.y += sy;
                     a.z += sz;
                     // a NaN or an infinity fails the comparison too

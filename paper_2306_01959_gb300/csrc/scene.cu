@@ -163,11 +163,12 @@ void fill_inst(HostInst &hi, const sph_params &p, int fine, bool tiled)
     if (tiled) {
         int e;
         const double f = std::frexp(d.cs, &e);
-        d.oc = std::ldexp(std::nearbyint(std::ldexp(f, 19)), e - 19);
+        d.oc = std::ldexp(std::nearbyint(std::ldexp(f, 20)), e - 20);
     }
     d.ohf = (float)(0.5 * d.oc);
+    d.centred = tiled && effective_cell_div(p) * fine == 1;
     for (int a = 0; a < 3; ++a)
-        d.olo[a] = d.lo[a] + (tiled ? 0.5 * d.oc : 0.0);
+        d.olo[a] = d.lo[a] + (d.centred ? 0.5 * d.oc : 0.0);
     d.ncells = d.n[0] * d.n[1] * d.n[2];
     d.by_nx = divisor(std::max(d.n[0], 1));
     d.by_ny = divisor(std::max(d.n[1], 1));
