@@ -28,8 +28,8 @@
 //     butterfly and written out; nothing is carried between warps.
 // A tile whose neighbourhood exceeds the staging buffer (compressed fluid, a clump) is
 // halved until its parts fit (fluid of the 0.9 M-particle obstacle case compressed to
-// 1.6 times its density: 3.20 -> 1.89 ms per step, against 3.02 ms staged in chunks by
-// the kernel of pair_wide.cuh).  A single cell whose neighbourhood does not, or a part
+// 1.6 times its density: 3.20 -> 1.87 ms per step, against 3.02 ms staged in chunks by
+// the kernel of pair_wide.cuh; the code for it costs the others 0.4 to 3 %).  A single cell whose neighbourhood does not, or a part
 // that holds values a zero weight could not cancel (non-finite or huge), takes the
 // same path with the candidates read from global memory and every term masked.
 //
@@ -39,8 +39,8 @@
 // warp instructions on the 0.9 M-particle obstacle case.  Rows of cross-section h
 // leave 640 tests, one list per cluster a quarter of the ballots, and the pair terms
 // evaluated for nothing (1.4 per useful one) cost less than the tests and stores
-// they replace: 0.90e9 instructions, 1.98 -> 1.17 ms per pass (8.1 M particles:
-// 19.4 -> 11.5 ms; h = 1.5 dp, 2.0 M particles: 3.38 -> 1.61 ms).
+// they replace: 0.89e9 instructions, 1.98 -> 1.17 ms per pass (8.1 M particles:
+// 19.4 -> 11.1 ms; h = 1.5 dp, 2.0 M particles: 3.38 -> 1.62 ms).
 // What bounds it: issue slots and fixed latencies at 16 warps per SM (128
 // registers); a list step of 32 candidates takes about 170 warp instructions for 4
 // pair terms, 135 of them arithmetic, a step of the sweep about 50.
