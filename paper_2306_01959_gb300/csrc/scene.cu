@@ -255,7 +255,7 @@ bool tiles_fit(const sph_instance &in, const sph_params &p)
 // 772 | 890, 1.8 dp 1040 | 1036, 2.08 dp 1367 | 1292; 31 k particles 90 | 100, 91 | 94,
 // 99 | 100).  The automatic size takes that below 48 k particles only (18 k at h = 1.5
 // dp: 68 us, 78 with cells of h, 69 before the tiled pass): larger tanks get tiles whose
-// FP32 frames are longer with cells of 2h, at 185 k particles a tenth less accurate.
+// FP32 frames are longer with cells of 2h, at 185 k particles 5 % less accurate.
 int tile_cell_div(const std::vector<HostInst> &inst, int64_t n_total, bool automatic)
 {
     double most = 0.0;
